@@ -790,53 +790,66 @@ __device__ __forceinline__ void block_reduce(float (&acc)[kAccPad], float (*red)
 // ---------------------------------------------------------------------------
 // Solver tail, run by one warp of every CTA
 //
-// GB300 runs FP64 at a small fraction of its FP32 rate with long dependent
-// latencies (measured on the part: ~64 cycles per DFMA, ~420 per divide or
-// reciprocal, ~670 per square root, ~1700 per sincos), and this tail sits on
-// the critical path of every pass.  The state, the normal equations, the
-// accept/reject decision and the composition are FP64 in both solve modes;
-// GLT_SOLVE_FP64 (the default) also factorises and exponentiates in FP64,
-// GLT_SOLVE_FP32 does those two in FP32 (their inputs carry FP32 rounding
-// anyway, or their result is a small increment):
+// It sits on the critical path of every pass, and GB300's FP64 is what bounds
+// it: measured on the part, an FP64 instruction occupies its sub-partition's
+// pipe for 64 cycles whether 1 or 32 lanes take part; the next FP64
+// instruction has its result after the same 64, any other after ~110, an
+// FP64 compare costs ~105; a shuffle costs ~24 and an FP32 FMA 4.  So the tail is written for the fewest FP64
+// instructions on the dependent chain: independent quantities share one
+// instruction on different lanes, comparisons go through the bit pattern, and
+// what a decision does not need is not computed.  The state, the normal
+// equations, the accept/reject decision and the composition are FP64 in both
+// solve modes; GLT_SOLVE_FP64 (the default) also factorises and exponentiates
+// in FP64, GLT_SOLVE_FP32 does those two in FP32 (their inputs carry FP32
+// rounding anyway, or their result is a small increment):
 //  * the damped normal matrix is factored as L D L^T (no square roots), one
-//    row per lane, columns eliminated right-looking with warp shuffles; in
+//    entry per lane, columns eliminated right-looking with warp shuffles; in
 //    GLT_SOLVE_FP32 first in FP32, and a pivot below 1e-4 of its damped
 //    diagonal sends the system to the FP64 elimination, which alone decides
 //    "not positive definite";
-//  * FP64 pivot reciprocals are an FP32 seed refined by one Newton step
-//    (relative error ~4e-15);
+//  * FP64 pivot reciprocals are an FP32 seed and an FP32 correction of it;
 //  * the SE(3) exponential uses the power series of its coefficients in
 //    theta^2 below theta = 0.1 (sincos only beyond), each lane one element
 //    of exp(delta) (GLT_SOLVE_FP32: of exp(delta) - I in FP32, composed with
 //    the FP64 pose as T + T (exp(delta) - I), and the frame's final pose
 //    orthonormalised once in FP64);
-//  * FP64 <-> FP32 conversions go through the bit pattern (integer
-//    instructions), and accept/reject compares E' n <= E n' instead of
-//    dividing.
+//  * accept/reject compares E' n <= E n' instead of dividing, and only for
+//    steps that are not small enough to be taken anyway.
 // ---------------------------------------------------------------------------
+// 1 / d as the unevaluated sum r0 + rl of two doubles, for a positive d in
+// [2^-100, 2^100).  With d = 2^E m, m = mh + ml in [1, 2) split at FP32's 24
+// bits (ml cut at 2^-46): q = rcp.approx.ftz.f32(mh), the residual e = 1 - m q
+// in two FP32 FMAs (error below 2^-46, |e| < 2^-21), and 1 / m = q / (1 - e) =
+// q + q (e + e^2) + O(e^3): r0 = q, rl the FP32 correction, both scaled by
+// 2^-E through their exponent bits.  No FP64 instruction, relative error below
+// 2^-45; the Newton step in FP64 that this replaces cost two dependent FP64
+// instructions (128 cycles) for 2^-44.  (A correction of zero gives rl =
+// 2^-127 r0, which no double sum sees.)
+__device__ __forceinline__ void rcp_pair(double d, double& r0, double& rl)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const float mh = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u);
+    const float ml = fmaf(__uint_as_float(((lo >> 6) & 0x7fffffu) | 0x3f800000u), 0x1p-23f, -0x1p-23f);
+    float q;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
+    const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
+    const float c = q * fmaf(e, e, e);
+    // FP32 bits to FP64's: the exponent re-biased and lowered by E
+    const unsigned off = ((896u + 1023u) << 20) - (hi & 0x7ff00000u);
+    const unsigned qb = __float_as_uint(q), cb = __float_as_uint(c);
+    r0 = __hiloint2double((int)((qb >> 3) + off), (int)(qb << 29));
+    rl = __hiloint2double((int)((((cb >> 3) & 0x0fffffffu) + off) | (cb & 0x80000000u)), (int)(cb << 29));
+}
+
+// Reciprocal of any d: rcp_pair for 2^-100 <= |d| < 2^100 (exponent tested as
+// an integer); zero, infinities, NaN and the rest divide.
 __device__ __forceinline__ double rcp_d(double d)
 {
-    // Reciprocal by one Newton-Raphson iteration for f(r) = 1/r - d,
-    // r' = r + r (1 - d r), from an FP32 seed: the seed is rcp.approx.ftz.f32
-    // of d rounded to FP32 through its bit pattern (no F2F conversions on the
-    // FP64 pipe), relative error e0 <= 2^-22, and the iteration squares it
-    // (e1 = e0^2 plus FP64 rounding): relative error < 1e-13.  Only for
-    // 2^-100 <= |d| < 2^100 (exponent tested as an integer), where the
-    // exponent fits FP32; zero, infinities, NaN and the rest divide.
-    const int hi = __double2hiint(d);
-    const unsigned lo = (unsigned)__double2loint(d);
-    const int ebits = (hi >> 20) & 0x7ff;
+    const int ebits = (__double2hiint(d) >> 20) & 0x7ff;
     if (ebits < 1023 - 100 || ebits >= 1023 + 100) return 1.0 / d;
-    const int e32 = ebits - 896;
-    const unsigned fb = ((unsigned)hi & 0x80000000u) | ((unsigned)e32 << 23) |
-                        (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29);
-    float rf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint_as_float(fb)));
-    const unsigned rb = __float_as_uint(rf);
-    const int rhi = (int)((rb & 0x80000000u) | ((((rb >> 23) & 0xffu) + 896u) << 20) | ((rb >> 3) & 0xfffffu));
-    double r = __hiloint2double(rhi, (int)(rb << 29));
-    const double e = fma(-d, r, 1.0);
-    return fma(r, e, r);
+    double r0, rl;
+    rcp_pair(fabs(d), r0, rl);
+    return copysign(r0 + rl, d);
 }
 
 // FP64 -> FP32 through the bit pattern (integer instructions only, nothing on
@@ -860,6 +873,23 @@ __device__ __forceinline__ float f32_of(double x)
     else
         b = sign | ((unsigned)(eb - 896) << 23) | man;
     return __uint_as_float(b);
+}
+
+// FP64 -> FP32 rounded to nearest even, as the conversion instruction does it,
+// in integer instructions (the conversion takes its turn on the FP64 pipe);
+// results below FP32's normal range, infinities and NaN are left to it.
+__device__ __forceinline__ float f32_rn(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned eb = (hi >> 20) & 0x7ffu;
+    if (eb - 897u >= 254u && ((hi & 0x7fffffffu) | lo) != 0u) return (float)x;
+    // sign, re-biased exponent, 23 bits of the significand; a carry out of the
+    // rounded significand steps the exponent
+    unsigned b = __funnelshift_l(lo, hi, 3) & 0x7fffffu;
+    b |= (eb - 896u) << 23;
+    const unsigned rem = lo << 3;                  // what the cut leaves, 2^31 is half
+    b += (rem > 0x80000000u || (rem == 0x80000000u && (b & 1u))) ? 1u : 0u;
+    return __uint_as_float((eb ? b : 0u) | (hi & 0x80000000u));
 }
 
 // FP32 -> FP64 through the bit pattern: exact for zero and normal numbers
@@ -932,41 +962,30 @@ __device__ __forceinline__ void make_pass_params_warp(const double* T, double a,
     }
 }
 
-// Same, with lane l < 12 holding pose entry l in `v` (no shared-memory read).
-__device__ __forceinline__ void make_pass_params_lane(double v, double a, double b, int level,
-                                                      PassParams& P, int lane)
-{
-    if (lane < 12) {
-        const int r = lane >> 2, c = lane & 3;
-        const double m = v - ((c == r) ? 1.0 : 0.0);
-        if (c < 3)
-            P.Rm[3 * r + c] = (float)m;
-        else
-            P.t[r] = (float)m;
-    } else if (lane == 12) {
-        P.ea = expf((float)a);
-    } else if (lane == 13) {
-        P.b = (float)b;
-        P.level = level;
-        P.scale = ldexpf(1.0f, -level);
-        P.done = 0;
-    }
-}
-
 // LM state machine, replicated in every CTA of a stream's cluster (each CTA
 // runs it on bit-identical inputs, so all take the same decisions).
 enum { PH_START = 0, PH_CAND = 1 };
 
+constexpr int kXs0 = 8, kXs1 = 9, kXsPoly = 10, kXsTable = 19;
+
 struct Solver {
-    double T[12], a, b;       // accepted state
+    // two states (pose, affine pair): the accepted one at [cur], the candidate
+    // under evaluation at [cur ^ 1]; accepting a candidate flips cur
+    double T[2][12], ab[2][2];
     double ema;               // cached-Hessian form: e^-a (a is held fixed there)
-    double Tc[12], ac, bc;    // candidate under evaluation
-    double H[64], g[8];       // normal equations at the accepted state
-    double E, nd, lambda, res_E;   // energy / samples (as double) at the accepted state
+    double N[kAccPad];        // sums at the accepted state
+    double Hi[36];            // cached-Hessian form: -e^-a H^-1 of the level
+    double E, nd, res_E;      // energy / samples (as double) at the accepted state
+    double lam_dn, lam_up;    // the damping after the candidate is accepted / rejected
+    double xs[kXsTable];      // the step (translation, rotation, da, db), then the constants
+                              // 0, 1 and the series of A, B, C (see tail_map_init)
+    double Lm[72];            // L (row by row), then D^-1 L^-1 times the right-hand side
     long long maxstep_bits;   // max |delta_xi| of the candidate, as abs_bits
+    int cur, hc_ok;           // hc_ok: the level's reference Hessian is positive definite
     int n, res_n, level, it, phase, status, passes, done;
     int moved;                // the pose changed since the initial state
     int iters[kMaxLevels];
+    unsigned map_ldl[32], map_dot[32], map_ent[32];   // per lane, packed (tail_map_init)
 };
 
 // Upper-triangle index of (i, j), i <= j, in the accumulator layout.
@@ -975,9 +994,10 @@ __device__ __forceinline__ int upper_index(int i, int j) { return i * 8 - (i * (
 // Initial state (one thread): Gram-Schmidt the initial rotation, first level.
 __device__ inline void solver_init(const StreamDesc& D, const double* init, Solver& S, PassParams& P)
 {
-    for (int i = 0; i < 12; ++i) S.T[i] = init[i];
+    S.cur = 0;
+    for (int i = 0; i < 12; ++i) S.T[0][i] = init[i];
     {
-        double* T = S.T;
+        double* T = S.T[0];
         const double n0 = sqrt(T[0] * T[0] + T[1] * T[1] + T[2] * T[2]);
         for (int c = 0; c < 3; ++c) T[c] /= n0;
         const double d = T[4] * T[0] + T[5] * T[1] + T[6] * T[2];
@@ -988,12 +1008,12 @@ __device__ inline void solver_init(const StreamDesc& D, const double* init, Solv
         T[9] = T[2] * T[4] - T[0] * T[6];
         T[10] = T[0] * T[5] - T[1] * T[4];
     }
-    S.a = init[12];
-    S.b = init[13];
+    S.ab[0][0] = init[12];
+    S.ab[0][1] = init[13];
     S.status = 0;
     bool finite_start = true;
-    for (int i = 0; i < 12; ++i) finite_start &= abs_bits(S.T[i]) < kInfBits;
-    finite_start &= abs_bits(S.a) < kInfBits && abs_bits(S.b) < kInfBits;
+    for (int i = 0; i < 12; ++i) finite_start &= abs_bits(S.T[0][i]) < kInfBits;
+    finite_start &= abs_bits(S.ab[0][0]) < kInfBits && abs_bits(S.ab[0][1]) < kInfBits;
     S.passes = 0;
     S.it = 0;
     S.n = 0;
@@ -1005,7 +1025,7 @@ __device__ inline void solver_init(const StreamDesc& D, const double* init, Solv
     S.done = 0;
     S.moved = 0;
     for (int l = 0; l < kMaxLevels; ++l) S.iters[l] = 0;
-    S.ema = (D.Hc && finite_start) ? exp(-S.a) : 1.0;
+    S.ema = (D.Hc && finite_start) ? exp(-S.ab[0][0]) : 1.0;
     int l = D.L - 1;
     while (l >= 0 && D.max_iters[l] <= 0) --l;
     if (!finite_start) {
@@ -1020,61 +1040,407 @@ __device__ inline void solver_init(const StreamDesc& D, const double* init, Solv
         S.done = 1;
         P.done = 1;
     } else {
-        make_pass_params(S.T, S.a, S.b, l, P);
+        make_pass_params(S.T[0], S.ab[0][0], S.ab[0][1], l, P);
     }
 }
 
-// One LM decision after a pass whose cluster-wide sums are `tot`; executed
-// by all 32 lanes of one warp with uniform control flow.  FP64 instructions
-// are kept to the minimum the method needs (each costs ~64 issue cycles).
+// (H + lambda diag H) delta = -g by L D L^T, right-looking, one entry per
+// lane.  The right-hand side rides along as row 8 of the lower triangle
+// (entry (8, k) = y_k), so the 44 entries (i, k), k <= i <= 8, all follow
+//   a_ik -= a_ij a_kj / d_j   for k > j.
+// Columns 2-7 (27 entries) sit in register A of lanes 0-26 and take one pair
+// of FMAs per eliminated column; columns 0 and 1 sit in register B of lanes
+// 0-8 and 9-16, of which column 1 is updated once.  Column k starts at lane
+// cA(k) of A, so entry (i, j) is on lane cA(j) - j + i (B: i for j = 0, 8 + i
+// for j = 1); a lane without part in a step takes its factors from lane 31,
+// which holds zeros.  The product a_ij a_kj is formed while the pivot's
+// reciprocal is, so a column's dependent chain is a shuffle, the product and
+// the two FMAs with the reciprocal's two parts: 300 cycles, 4.2k for the whole
+// solve.  (The form with l_ij = a_ij / d_j, a Newton step in FP64 and separate
+// updates of the diagonal and the right-hand side took 6.9k.)
+__host__ __device__ constexpr int ldl_lane(int k) { return k == 2 ? 0 : k == 3 ? 7 : k == 4 ? 13 : k == 5 ? 18 : k == 6 ? 22 : 25; }
+
+// Per-lane tables of the tail, packed into three words, and the constants
+// behind the step (one warp, once per launch; the caller synchronises).
+__device__ inline void tail_map_init(Solver& S, int lane)
+{
+    // L D L^T: positions of the lane's entries in the sums, and (i, k) of both
+    const int kA = lane < 7 ? 2 : lane < 13 ? 3 : lane < 18 ? 4 : lane < 22 ? 5 : lane < 25 ? 6 : lane < 27 ? 7 : 8;
+    const int iA = kA < 8 ? kA + lane - ldl_lane(kA) : 9;
+    const int kB = lane < 9 ? 0 : lane < 17 ? 1 : 8;
+    const int iB = lane < 9 ? lane : lane < 17 ? lane - 8 : 9;
+    const int pA = iA > 8 ? kNumAcc : iA == 8 ? kIdxG + kA : upper_index(kA, iA);   // kNumAcc: a zero
+    const int pB = iB > 8 ? kNumAcc : iB == 8 ? kIdxG + kB : upper_index(kB, iB);
+    S.map_ldl[lane] = (unsigned)(pA | (pB << 6) | (iA << 12) | (kA << 16) | (iB << 20) | (kB << 24));
+    // the three products of a lane's dot (indices into xs): w . w on lanes
+    // 0-15, w . v on 16, (w x v)_r on 17 + r (its second product negated)
+    const int r = lane >= 17 && lane < 20 ? lane - 17 : 0, r1 = (r + 1) % 3, r2 = (r + 2) % 3;
+    const bool dot = lane == 16, cross = lane >= 17 && lane < 20;
+    const int p1 = cross ? 3 + r1 : 3, q1 = cross ? r2 : dot ? 0 : 3;
+    const int p2 = cross ? 3 + r2 : 4, q2 = cross ? r1 : dot ? 1 : 4;
+    const int p3 = cross ? kXs0 : 5, q3 = cross ? kXs0 : dot ? 2 : 5;
+    S.map_dot[lane] = (unsigned)(p1 | (q1 << 5) | (p2 << 10) | (q2 << 15) | (p3 << 20) | (q3 << 25));
+    // entry (er, ec) of the exponential on lane 4 er + ec < 12: w_er, the
+    // column's w (rotation), d_rc or v_er, and W_rc = +w_{r+2} if c = r+1,
+    // -w_{r+1} if c = r+2; lanes 12-14: the series of A, B, C
+    const int er = (lane >> 2) % 3, ec = lane & 3, er1 = (er + 1) % 3, er2 = (er + 2) % 3;
+    const bool poly = lane >= 12 && lane < 15;
+    const int g = lane - 12;
+    const int w = poly ? kXsPoly + 6 + g : 3 + er;
+    const int pq = ec < 3 ? 3 + ec : kXs0;
+    const int dd = poly ? kXsPoly + g : ec < 3 ? (er == ec ? kXs1 : kXs0) : er;
+    const int c1 = poly ? kXsPoly + 3 + g : kXs0;
+    const int W = ec == er1 ? 3 + er2 : (ec < 3 && ec == er2) ? 3 + er1 : kXs0;
+    S.map_ent[lane] = (unsigned)(w | (pq << 5) | (dd << 10) | (c1 << 15) | (W << 20)) |
+                      (ec == er1 ? 1u << 25 : 0u);
+    if (lane == 0) {
+        S.xs[kXs0] = 0.0;
+        S.xs[kXs1] = 1.0;
+        double* c = S.xs + kXsPoly;      // th^2 coefficients 2, 1, 0 of A, B, C
+        c[0] = 1.0 / 120.0;
+        c[1] = 1.0 / 720.0;
+        c[2] = 1.0 / 5040.0;
+        c[3] = -1.0 / 6.0;
+        c[4] = -1.0 / 24.0;
+        c[5] = -1.0 / 120.0;
+        c[6] = 1.0;
+        c[7] = 0.5;
+        c[8] = 1.0 / 6.0;
+    }
+    for (int i = lane; i < kAccPad; i += 32) S.N[i] = 0.0;
+}
+
+// src: a pass's sums (zeros beyond the last); Lm: 72 doubles of shared memory;
+// x: the solution on lanes 0-7.  EXACT: reciprocals of any pivot and the pivot
+// test d > 0, d > 1e-13 x the damped diagonal; otherwise every pivot must
+// pass that test by its exponent alone (2^-43 > 1e-13) and lie in rcp_pair's
+// range.  False if one does not.
+template <bool EXACT>
+__device__ __forceinline__ bool ldl_solve_t(const double* src, double lambda, bool fixed_ab, unsigned map,
+                                            double* Lm, int lane, double& x)
+{
+    const unsigned full = 0xffffffffu;
+    const int iA = (map >> 12) & 15, kA = (map >> 16) & 15, iB = (map >> 20) & 15, kB = map >> 24;
+    const bool dA = iA == kA, dB = iB == kB;                // diagonal entries
+    double B = src[(map >> 6) & 63], A = src[map & 63];
+    if (iB == 8) B = -B;                                    // y = -g
+    if (iA == 8) A = -A;
+    if (fixed_ab) {
+        // with (a, b) held fixed their rows and columns become the identity and
+        // their right-hand side zero, so the solve gives da = db = 0
+        if (iB == 6 || iB == 7) B = 0.0;
+        if (kA == 6 || kA == 7 || iA == 6 || iA == 7) A = dA ? 1.0 : 0.0;
+    }
+    B = fma(dB ? lambda : 0.0, B, B);                       // damped diagonal
+    A = fma(dA ? lambda : 0.0, A, A);
+    const double a0A = A, a0B = B;
+    double r0A = 0.0, rlA = 0.0, r0B = 0.0, rlB = 0.0;      // 1 / d of the lane's columns
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int cj = j == 0 ? 0 : j == 1 ? 8 : ldl_lane(j) - j;   // lane of (i, j) is cj + i
+        const double col = j < 2 ? B : A;
+        const double piv = __shfl_sync(full, col, cj + j);
+        double pA = 0.0, pB = 0.0;
+        if (j == 0) {
+            const bool on = kB == 1;
+            pB = __shfl_sync(full, col, on ? iB : 31) * __shfl_sync(full, col, on ? 1 : 31);
+        }
+        if (j < 7) {
+            const bool on = kA > j && kA < 8;
+            pA = __shfl_sync(full, col, on ? cj + iA : 31) * __shfl_sync(full, col, on ? cj + kA : 31);
+        }
+        double r0, rl = 0.0;
+        if (EXACT)
+            r0 = rcp_d(piv);
+        else
+            rcp_pair(piv, r0, rl);
+        if (j == 0) B = fma(-pB, rl, fma(-pB, r0, B));
+        if (j < 7) A = fma(-pA, rl, fma(-pA, r0, A));
+        if (j < 2) {
+            if (kB == j) {
+                r0B = r0;
+                rlB = rl;
+            }
+        } else if (kA == j) {
+            r0A = r0;
+            rlA = rl;
+        }
+    }
+    // L and z = D^-1 y (row 8): every entry times its column's reciprocal
+    const double sB = B * (r0B + rlB), sA = A * (r0A + rlA);
+    if (kB < 8) Lm[8 * iB + kB] = sB;
+    if (kA < 8) Lm[8 * iA + kA] = sA;
+    bool ok;
+    if (EXACT) {
+        ok = (!dA || (A > 1e-13 * a0A && A > 0.0)) && (!dB || (B > 1e-13 * a0B && B > 0.0));
+    } else {
+        // exponents of the pivot and of the damped diagonal (positive, normal)
+        const int pA = __double2hiint(A) >> 20, pB = __double2hiint(B) >> 20;
+        const int qA = __double2hiint(a0A) >> 20, qB = __double2hiint(a0B) >> 20;
+        ok = (!dA || (pA >= 1023 - 100 && pA < 1023 + 100 && qA > 0 && pA - qA >= -42)) &&
+             (!dB || (pB >= 1023 - 100 && pB < 1023 + 100 && qB > 0 && pB - qB >= -42));
+    }
+    if (!__all_sync(full, ok)) return false;
+    __syncwarp();
+    // L^T x = z: lane i < 8 holds x_i and its column of L
+    double Lcol[8];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) Lcol[j] = lane < j ? Lm[8 * j + lane] : 0.0;
+    x = lane < 8 ? Lm[64 + lane] : 0.0;
+#pragma unroll
+    for (int j = 7; j >= 1; --j) x = fma(-Lcol[j], __shfl_sync(full, x, j), x);
+    return true;
+}
+
+// kept out of line: near-singular systems only
+static __device__ __noinline__ bool ldl_solve_exact(const double* src, double lambda, bool fixed_ab, unsigned map,
+                                                    double* Lm, int lane, double* x)
+{
+    return ldl_solve_t<true>(src, lambda, fixed_ab, map, Lm, lane, *x);
+}
+
+__device__ __forceinline__ bool ldl_solve_warp(const double* src, double lambda, bool fixed_ab, Solver& S,
+                                               int lane, double& x)
+{
+    const unsigned map = S.map_ldl[lane];
+    if (ldl_solve_t<false>(src, lambda, fixed_ab, map, S.Lm, lane, x)) return true;
+    double xe = 0.0;
+    const bool ok = ldl_solve_exact(src, lambda, fixed_ab, map, S.Lm, lane, &xe);
+    x = xe;
+    return ok;
+}
+
+// entry (i, k) of the system as doubles (the FP32 elimination's inputs)
+__device__ __forceinline__ double ldl_entry(const double* src, int i, int k, bool fixed_ab)
+{
+    if (fixed_ab && (k >= 6 || i == 6 || i == 7)) return i == k ? 1.0 : 0.0;
+    return i < 8 ? src[upper_index(k, i)] : -src[kIdxG + k];
+}
+
+// The FP32 elimination of GLT_SOLVE_FP32 (H and g are FP32 sums, relative
+// error ~1e-7, so the step they define is known to ~cond x 1e-7 however it is
+// solved; the FP32 elimination adds an error of the same order, ~cond x
+// 2^-23).  Lanes 0-27 hold the strictly lower entries (i, k), i > k, column by
+// column; lanes 0-7 also the diagonal entry and the right-hand side of row
+// `lane`.  Used when every FP32 pivot is above 1e-4 of its damped diagonal,
+// where its rounding (~1e-6 of the diagonal) cannot change its sign; false
+// otherwise: the FP64 elimination decides.
+__device__ __forceinline__ bool ldl_solve_warp_fp32(const double* src, double lambda, bool fixed_ab, int lane,
+                                                    double& x64)
+{
+    const unsigned full = 0xffffffffu;
+    const int row = lane & 7;
+    const int ek = lane < 7 ? 0 : lane < 13 ? 1 : lane < 18 ? 2 : lane < 22 ? 3 : lane < 25 ? 4
+                 : lane < 27 ? 5 : lane < 28 ? 6 : 7;
+    const int ei = lane < 28 ? lane - (ek * 7 - (ek * (ek - 1)) / 2) + ek + 1 : 8;
+    float e = lane < 28 ? f32_of(ldl_entry(src, ei, ek, fixed_ab)) : 0.0f;
+    const double diag = ldl_entry(src, row, row, fixed_ab);
+    const double a0 = fma(lambda, diag, diag);
+    const float a0f = f32_of(a0);
+    float dg = a0f, dinv = 0.0f;
+    float y = f32_of(ldl_entry(src, 8, row, fixed_ab));
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float d = __shfl_sync(full, dg, j);
+        const float r = __frcp_rn(d);
+        if (lane == j) dinv = r;
+        if (j < 7) {
+            const float l = e * r;
+            const int cj = j * 7 - (j * (j - 1)) / 2 - j - 1;   // lane of (i, j) is cj + i
+            const bool trail = lane < 28 && ek > j;
+            const bool drow = lane > j && lane < 8;
+            const float li = __shfl_sync(full, l, cj + (trail ? ei : j + 1));
+            const float ak = __shfl_sync(full, e, cj + (trail ? ek : j + 1));
+            const float ld = __shfl_sync(full, l, cj + (drow ? lane : j + 1));
+            const float ad = __shfl_sync(full, e, cj + (drow ? lane : j + 1));
+            const float yj = __shfl_sync(full, y, j);
+            if (trail) e = fmaf(-li, ak, e);
+            if (drow) {
+                dg = fmaf(-ld, ad, dg);
+                y = fmaf(-ld, yj, y);
+            }
+            if (lane < 28 && ek == j) e = l;
+        }
+    }
+    if (!__all_sync(full, dg > 1e-4f * a0f || lane >= 8)) return false;
+    // column `row` of L (entries below the diagonal) gathered into the row's lane
+    float Lcol[8];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+        const int cr = row * 7 - (row * (row - 1)) / 2 - row - 1;
+        const float v = __shfl_sync(full, e, row < i ? cr + i : 0);
+        Lcol[i] = row < i ? v : 0.0f;
+    }
+    // diagonal, backward (L^T x = D^-1 y)
+    float x = y * dinv;
+#pragma unroll
+    for (int j = 7; j >= 1; --j) {
+        const float xj = __shfl_sync(full, x, j);
+        if (row < j) x = fmaf(-Lcol[j], xj, x);
+    }
+    x64 = f64_of(x);
+    return true;
+}
+
+// A, B or C (g = 0, 1, 2) beyond theta = 0.01: longer series, or closed forms
+static __device__ __noinline__ double se3_coefficient(double th2, int g)
+{
+    if (th2 < 0.01) {
+        const double c4 = g == 0 ? 1.0 / 362880.0 : g == 1 ? 1.0 / 3628800.0 : 1.0 / 39916800.0;
+        const double c3 = g == 0 ? -1.0 / 5040.0 : g == 1 ? -1.0 / 40320.0 : -1.0 / 362880.0;
+        const double c2 = g == 0 ? 1.0 / 120.0 : g == 1 ? 1.0 / 720.0 : 1.0 / 5040.0;
+        const double c1 = g == 0 ? -1.0 / 6.0 : g == 1 ? -1.0 / 24.0 : -1.0 / 120.0;
+        const double c0 = g == 0 ? 1.0 : g == 1 ? 0.5 : 1.0 / 6.0;
+        return fma(fma(fma(fma(th2, c4, c3), th2, c2), th2, c1), th2, c0);
+    }
+    const double th = sqrt(th2);
+    double sn, cs, sh, ch;
+    sincos(th, &sn, &cs);
+    sincos(0.5 * th, &sh, &ch);
+    return g == 0 ? sn / th : g == 1 ? 2.0 * sh * sh / th2 : (th - sn) / (th2 * th);
+}
+
+// exp(delta_xi) of the step S.xs as a 3x4 [R_e | t_e], entry (r, c) on lane
+// 4 r + c:
+//   R_e(r, c) = d_rc + A W_rc + B (w_r w_c - d_rc th2)            (W = [w]x)
+//   t_e(r)    = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
+// with A = sin th / th, B = (1 - cos th) / th^2, C = (th - sin th) / th^3.
+// Seven FP64 instructions on the chain (the one-entry-per-lane form with
+// uniform A, B, C took 17 and two compares): three give th2 (lanes 0-15),
+// w . v (lane 16) and w x v (lanes 17-19) at once, two the series of A, B, C
+// (lanes 12-14) together with w_r (.) - (.) th2 of every entry, two the entry.
+__device__ __forceinline__ double se3_exp_warp(const Solver& S, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const double* xs = S.xs;
+    const unsigned md = S.map_dot[lane], me = S.map_ent[lane];
+    const double p1 = xs[md & 31], q1 = xs[(md >> 5) & 31], p2 = xs[(md >> 10) & 31], q2 = xs[(md >> 15) & 31],
+                 p3 = xs[(md >> 20) & 31], q3 = xs[(md >> 25) & 31];
+    const double w = xs[me & 31], wc = xs[(me >> 5) & 31], dd = xs[(me >> 10) & 31], c1 = xs[(me >> 15) & 31];
+    double W = xs[(me >> 20) & 31];
+    if (me >> 25) W = -W;
+    const bool poly = lane >= 12 && lane < 15, rot = (lane & 3) < 3;
+    double s = p1 * q1;
+    s = fma(lane >= 17 && lane < 20 ? -p2 : p2, q2, s);
+    s = fma(p3, q3, s);                                      // th2 on lanes 0-15
+    const double wv = __shfl_sync(full, s, 16);
+    const double cr = __shfl_sync(full, s, 17 + (lane >> 2) % 3);
+    const double pq = rot ? wc : wv;
+    const double u = fma(s, dd, c1);                         // (.) th2, or the series' first step
+    double ey = fma(poly ? u : w, poly ? s : pq, poly ? w : -u);
+    const double th2 = __shfl_sync(full, s, 0);
+    if (!(__double_as_longlong(th2) < 0x3f1a36e2eb1c432dll)) {   // th2 >= 1e-4 (or NaN)
+        const double co = se3_coefficient(th2, lane >= 12 ? lane - 12 : 0);
+        if (poly) ey = co;
+    }
+    const double cx = __shfl_sync(full, ey, rot ? 12 : 13);  // of W_rc / (w x v)_r: A / B
+    const double cy = __shfl_sync(full, ey, rot ? 13 : 14);  // of ey: B / C
+    return fma(cy, ey, fma(cx, rot ? W : cr, dd));
+}
+
+// exp(delta_xi) - I in FP32, entry (r, c) on lane 4 r + c (GLT_SOLVE_FP32): its
+// entries are O(|delta|), so FP32 rounding leaves ~1e-7 |delta| (absolute).
+// Coefficients as above (power series below th^2 = 0.25, truncation < 3e-11
+// relative).
+__device__ __forceinline__ double se3_exp_minus_i_warp(const double* xs, int lane)
+{
+    const float v0 = f32_of(xs[0]), v1 = f32_of(xs[1]), v2 = f32_of(xs[2]);
+    const float w0 = f32_of(xs[3]), w1 = f32_of(xs[4]), w2 = f32_of(xs[5]);
+    const float th2 = fmaf(w0, w0, fmaf(w1, w1, w2 * w2));
+    float A, B, Cc;
+    if (th2 < 0.25f) {
+        A = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 362880.0f, -1.0f / 5040.0f), th2, 1.0f / 120.0f), th2, -1.0f / 6.0f), th2, 1.0f);
+        B = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 3628800.0f, -1.0f / 40320.0f), th2, 1.0f / 720.0f), th2, -1.0f / 24.0f), th2, 0.5f);
+        Cc = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 39916800.0f, -1.0f / 362880.0f), th2, 1.0f / 5040.0f), th2, -1.0f / 120.0f), th2, 1.0f / 6.0f);
+    } else {
+        const float th = sqrtf(th2);
+        const float sn = sinf(th), sh = sinf(0.5f * th);
+        A = sn / th;
+        B = 2.0f * sh * sh / th2;
+        Cc = (th - sn) / (th2 * th);
+    }
+    // one element (r, c) of the 3x4 increment per lane 0-11, every lane
+    // running the same instructions on its own operands:
+    //   (R_e - I)(r, c) = A W_rc + B (w_r w_c - d_rc th2)        (W = [w]x)
+    //   t_e(r)          = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
+    // as  base + cA (a1 b1 - a2 b2) + cB (p q - d th2).
+    const float wv = fmaf(w0, v0, fmaf(w1, v1, w2 * v2));
+    const int er = (lane >> 2) % 3, ec = lane & 3;
+    const float wr = er == 0 ? w0 : (er == 1 ? w1 : w2);
+    const float wr1 = er == 0 ? w1 : (er == 1 ? w2 : w0);   // w_{r+1}
+    const float wr2 = er == 0 ? w2 : (er == 1 ? w0 : w1);   // w_{r+2}
+    const float vr = er == 0 ? v0 : (er == 1 ? v1 : v2);
+    const float vr1 = er == 0 ? v1 : (er == 1 ? v2 : v0);
+    const float vr2 = er == 0 ? v2 : (er == 1 ? v0 : v1);
+    const float wc = ec == 0 ? w0 : (ec == 1 ? w1 : w2);
+    const bool rot = ec < 3;
+    const float drc = (rot && er == ec) ? 1.0f : 0.0f;
+    // W_rc = +w_{r+2} if c = r+1, -w_{r+1} if c = r+2, 0 on the diagonal
+    const float Wrc = ec == (er + 1) % 3 ? -wr2 : (ec == (er + 2) % 3 ? wr1 : 0.0f);
+    const float base = rot ? 0.0f : vr;
+    const float a1 = rot ? Wrc : wr1, b1 = rot ? 1.0f : vr2;
+    const float a2 = rot ? 0.0f : wr2, b2 = rot ? 0.0f : vr1;
+    const float pq = rot ? wc : wv, dd = rot ? drc : vr;
+    const float ex = fmaf(a1, b1, -(a2 * b2));
+    const float ey = fmaf(wr, pq, -(dd * th2));
+    return f64_of(fmaf(rot ? B : Cc, ey, fmaf(rot ? A : B, ex, base)));
+}
+
+// One LM decision after a pass whose cluster-wide sums are `tot`, of which `n`
+// valid samples; executed by all 32 lanes of one warp with uniform control
+// flow.
 // HC: the cached-Hessian form (tot holds g0 = sum w r J_ic, E and n; the
 // step is -e^-a H^-1 g0 with the level's per-reference H^-1, since the rows
 // are e^a J_ic and the normal matrix e^2a H).
 template <bool HC = false>
-__device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, Solver& S,
+__device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, int n, Solver& S,
                                         PassParams& P, int lane, bool write_trace)
 {
     const unsigned full = 0xffffffffu;
-    const int row = lane & 7;
+    constexpr int NSUM = HC ? kHcAcc : kNumAcc;
     const double E = tot[HC ? kHcE : kIdxE];
     const double nd = tot[HC ? kHcN : kIdxN];   // exact integer count
-    const int n = (int)nd;
     // sums that are not finite (an FP32 overflow) make the pass unusable
     bool fin = true;
 #pragma unroll
-    for (int i = lane; i < (HC ? kHcE : kIdxE); i += 32) fin &= abs_bits(tot[i]) < kInfBits;
-    const bool sums_finite = __all_sync(full, fin) && abs_bits(E) < kInfBits;
+    for (int i = lane; i <= (HC ? kHcE : kIdxE); i += 32) fin &= abs_bits(tot[i]) < kInfBits;
+    const bool sums_finite = __all_sync(full, fin);
     const bool enough = n >= D.min_valid && n > 0 && sums_finite;
     int status = S.status;
     if (!sums_finite) status |= GLT_TRACK_DIVERGED;
     const int level = S.level;
     const int phase = S.phase;
     int it = S.it;
-    double lambda = S.lambda;
+    int cur = S.cur;
     const long long step_bits = S.maxstep_bits;
-    bool load_normal = false, accept = false, finish = false, candidate = false;
+    const long long stop_bits = abs_bits(level > 0 ? D.eps_step_coarse : D.eps_step);
+    const long long take_bits = abs_bits(D.accept_step);
+    double lambda = D.lambda0;
+    bool accept = false, load_normal = false, finish = false, candidate = false;
     if (phase == PH_START) {
         if (!enough) {
             if (sums_finite) status |= GLT_TRACK_TOO_FEW_POINTS;
         } else {
             load_normal = true;
-            lambda = D.lambda0;
             it = 0;
             candidate = true;
         }
     } else {
         ++it;
-        // c' < c  <=>  E' n < E n'  (both counts positive); flat: c' - c <= eps c
-        const double En = E * S.nd;
-        const double Ecn = S.E * nd;
-        const bool small = step_bits < abs_bits(D.accept_step);
-        accept = enough && (En < Ecn || small);
-        const bool flat = !accept && enough && __double_as_longlong(D.eps_cost) != 0 &&
-                          (En - Ecn <= D.eps_cost * Ecn);   // off (no FP64 work) when eps_cost = 0
-        lambda *= accept ? D.lambda_down : D.lambda_up;
+        accept = enough && step_bits < take_bits;
+        bool flat = false;
+        if (enough && !accept) {
+            // c' < c  <=>  E' n < E n' (both sides non-negative: compared through
+            // their bits; both products in one instruction);  flat: c' - c <= eps c
+            const double En = (lane & 1) ? S.E * nd : E * S.nd;
+            const double e0 = __shfl_sync(full, En, 0), e1 = __shfl_sync(full, En, 1);
+            accept = __double_as_longlong(e0) < __double_as_longlong(e1);
+            flat = !accept && __double_as_longlong(D.eps_cost) != 0 && (e0 - e1 <= D.eps_cost * e1);
+        }
+        lambda = accept ? S.lam_dn : S.lam_up;
         load_normal = accept;
-        if (it >= D.max_iters[level] ||
-            step_bits < abs_bits(level > 0 ? D.eps_step_coarse : D.eps_step) || flat)
+        if (accept) cur ^= 1;
+        if (it >= D.max_iters[level] || step_bits < stop_bits || flat)
             finish = true;
         else
             candidate = true;
@@ -1084,378 +1450,151 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
         D.trace_n[S.passes] = n;
         D.trace_info[S.passes] = level * 4 + (phase == PH_CAND ? 1 + (accept ? 2 : 0) : 0);
     }
+    // the normal equations of the accepted state: this pass's, or the kept
+    // ones after a rejection
+    const double* src = load_normal ? tot : S.N;
+    bool next_level = (phase == PH_START && !enough) || finish;
+    bool solved = false;
+    double x = 0.0;                  // delta, entry i on lane i < 8
+    if (HC && candidate && phase == PH_START) {
+        // -e^-a H^-1 of the level, kept for its later passes
+        const double* Hi = D.Hc + 72 * level + 36;
+        const double h0 = Hi[lane], h1 = Hi[lane < 4 ? 32 + lane : 0];
+        S.Hi[lane] = -S.ema * h0;
+        if (lane < 4) S.Hi[32 + lane] = -S.ema * h1;
+        if (lane == 0) S.hc_ok = abs_bits(h0) < kInfBits;
+        __syncwarp();
+    }
+    if (candidate && HC) {
+        // ---- delta = -e^-a H^-1 g0, half a row per lane (rows 0-5 on lanes 0-5
+        // and 8-13); the affine pair is held fixed in this form
+        if (S.hc_ok) {
+            const int r6 = (lane & 7) < 6 ? (lane & 7) : 0, c0 = (lane & 8) ? 3 : 0;
+            const double* h = S.Hi + 6 * r6 + c0;
+            x = fma(h[0], src[c0], fma(h[1], src[c0 + 1], h[2] * src[c0 + 2]));
+            x += __shfl_xor_sync(full, x, 8);
+            if (lane == 6 || lane == 7) x = 0.0;
+            solved = true;
+        }
+    } else if (candidate) {
+        if (D.solve != GLT_SOLVE_FP64) solved = ldl_solve_warp_fp32(src, lambda, !D.affine, lane, x);
+        if (!solved) solved = ldl_solve_warp(src, lambda, !D.affine, S, lane, x);
+    }
+    if (candidate && !solved) {
+        status |= GLT_TRACK_NOT_PD;
+        finish = true;
+        next_level = true;
+    }
+    if (lane < 8) S.xs[lane] = x;
     __syncwarp();
-    // commit the pass outcome to the shared state
-    if (accept && lane < 12) S.T[lane] = S.Tc[lane];
-    if (HC) {
-        if (load_normal) {
-            // g0 of the accepted state, and the level's H^-1 (read again at every
-            // acceptance: two loads per lane)
-            if (lane < 6) S.g[lane] = tot[lane];
-            const double* Hi = D.Hc + 72 * level + 36;
-            S.H[lane] = Hi[lane];
-            if (lane < 4) S.H[32 + lane] = Hi[32 + lane];
+    bool evaluated = false;          // P already holds the next state
+    bool moved = accept;
+    if (solved) {
+        const bool fp32 = D.solve == GLT_SOLVE_FP32;
+        // ---- Tc = T exp(delta) (FP32 form: T + T (exp(delta) - I)), three FP64
+        // instructions on all lanes: entry (r, c) on lane 16 + 4 r + c, the same
+        // minus the identity (what the pass parameters need) on lane 4 r + c,
+        // a + da and b + db on lanes 12 and 13, the two next dampings on 14, 15
+        const int q = lane & 15, er = (q >> 2) % 3, ec = q & 3;
+        const double* T = S.T[cur] + 4 * er;
+        double t0 = T[0], t1 = T[1], t2 = T[2], t3 = T[ec];
+        double e2 = 0.0, add = ec == 3 || fp32 ? t3 : 0.0;
+        if (q >= 12) {
+            t0 = t1 = 0.0;
+            t2 = lane == 12 || lane == 13 ? 1.0 : lane == 14 || lane == 15 ? lambda : 0.0;
+            e2 = lane == 12 ? S.xs[6] : lane == 13 ? S.xs[7] : lane == 14 ? D.lambda_down : D.lambda_up;
+            add = lane == 12 ? S.ab[cur][0] : lane == 13 ? S.ab[cur][1] : 0.0;
+        } else if (lane < 12 && er == ec) {
+            if (fp32)
+                asm volatile("add.rn.f64 %0, %0, 0dBFF0000000000000;" : "+d"(add));   // never speculated
+            else
+                add = -1.0;
         }
-    } else if (load_normal && lane < 8) {
-        // with (a, b) held fixed their rows and columns become the identity and
-        // their right-hand side zero, so the solve gives da = db = 0
-        const bool fixed_ab = !D.affine;
+        const double ent = fp32 ? se3_exp_minus_i_warp(S.xs, lane) : se3_exp_warp(S, lane);
+        const double x0 = __shfl_sync(full, ent, ec), x1 = __shfl_sync(full, ent, 4 + ec),
+                     x2 = __shfl_sync(full, ent, 8 + ec);
+        const double v = fma(t0, x0, fma(t1, x1, fma(t2, q >= 12 ? e2 : x2, add)));
+        // (finite t0 = t1 = 0 on lanes 12-15 drop x0, x1 unless those are not finite,
+        // which lanes 0-11 report as well)
+        long long mbits = 0;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            double v = tot[c >= lane ? upper_index(lane, c) : upper_index(c, lane)];
-            if (fixed_ab && (lane >= 6 || c >= 6)) v = lane == c ? 1.0 : 0.0;
-            S.H[8 * lane + c] = v;
+        for (int c = 0; c < 6; ++c) mbits = max(mbits, abs_bits(S.xs[c]));
+        // a step below the level's stop threshold (and below accept_step)
+        // would be taken whatever its cost and would end the level, so it
+        // is taken here without a pass of its own: the next level's start
+        // pass is the first evaluation of the new state; on the finest
+        // level the result keeps the cost and count of the last evaluated
+        // state
+        const bool take_now = mbits < stop_bits && mbits < take_bits;
+        if (!__all_sync(full, abs_bits(v) < kInfBits || lane == 14 || lane == 15)) {
+            // the solve produced a state that is not finite: keep the
+            // accepted one and end the level
+            status |= GLT_TRACK_DIVERGED;
+            finish = true;
+            next_level = true;
+        } else {
+            // the next pass evaluates the new state either way
+            const float vf = f32_rn(v);
+            const float ea = expf(vf);
+            float* pf = lane < 12 ? (ec < 3 ? &P.Rm[3 * er + ec] : &P.t[er]) : lane == 12 ? &P.ea : &P.b;
+            double* pd = lane < 16 ? (lane < 14 ? &S.ab[cur ^ 1][lane & 1] : lane == 14 ? &S.lam_dn : &S.lam_up)
+                                   : &S.T[cur ^ 1][(lane - 16) % 12];
+            if (lane < 14) *pf = lane == 12 ? ea : vf;
+            if (lane >= 12 && lane < 28) *pd = v;
+            evaluated = true;
+            if (take_now) {
+                ++it;
+                finish = true;
+                next_level = true;
+                cur ^= 1;
+                moved = true;
+            }
+            if (lane == 0) {
+                S.maxstep_bits = mbits;
+                S.phase = PH_CAND;
+            }
         }
-        S.g[lane] = (fixed_ab && lane >= 6) ? 0.0 : tot[kIdxG + lane];
+    }
+    // commit the pass outcome
+    if (load_normal) {
+        if (lane < NSUM) S.N[lane] = tot[lane];
+        if (lane < NSUM - 32) S.N[32 + lane] = tot[32 + lane];
     }
     if (lane == 0) {
         S.passes += 1;
+        S.cur = cur;
+        if (moved) S.moved = 1;
         S.it = it;
-        S.lambda = lambda;
         S.status = status;
-        if (accept) {
-            S.a = S.ac;
-            S.b = S.bc;
-            S.moved = 1;
-        }
         if (load_normal) {
             S.E = E;
             S.nd = nd;
             S.n = n;
         }
-    }
-    __syncwarp();
-
-    bool next_level = (phase == PH_START && !enough) || finish;
-    bool solved = false;
-    double dl[8];
-    if (candidate && HC) {
-        // ---- delta = -e^-a H^-1 g0, one row per lane (lanes 0-5); the affine
-        // pair is held fixed in this form
-        if (!(abs_bits(S.H[0]) < kInfBits)) {
-            if (lane == 0) S.status |= GLT_TRACK_NOT_PD;
-            finish = true;
-            next_level = true;
-        } else {
-            const int r6 = lane < 6 ? lane : 0;
-            double x = 0.0;
-#pragma unroll
-            for (int j = 0; j < 6; ++j) x = fma(S.H[6 * r6 + j], S.g[j], x);
-            x *= -S.ema;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) dl[c] = __shfl_sync(full, x, c);
-            dl[6] = 0.0;
-            dl[7] = 0.0;
-            solved = true;
+        if (finish) {
+            S.iters[level] = it;
+            S.res_E = S.E;
+            S.res_n = S.n;
         }
-    } else if (candidate) {
-        // ---- (H + lambda diag H) delta = -g by L D L^T, right-looking, one
-        // matrix entry per lane: lanes 0-27 hold the strictly lower entries
-        // (i, k), i > k, column by column; lanes 0-7 also hold the diagonal
-        // entry of row `lane`.  Each column costs one reciprocal, one scale
-        // and two FMAs per warp (trailing entries and diagonal) instead of
-        // one FMA per trailing column.
-        const int ek = lane < 7 ? 0 : lane < 13 ? 1 : lane < 18 ? 2 : lane < 22 ? 3 : lane < 25 ? 4
-                     : lane < 27 ? 5 : lane < 28 ? 6 : 7;
-        const int ei = lane < 28 ? lane - (ek * 7 - (ek * (ek - 1)) / 2) + ek + 1 : 8;
-        // GLT_SOLVE_FP32 first factorises in FP32 (H and g are FP32 sums,
-        // relative error ~1e-7, so the step they define is known to ~cond x
-        // 1e-7 however it is solved; the FP32 elimination adds an error of the
-        // same order, ~cond x 2^-23).  Used when every FP32 pivot is above 1e-4
-        // of its damped diagonal, where its rounding (~1e-6 of the diagonal)
-        // cannot change its sign; otherwise, and always for GLT_SOLVE_FP64
-        // (the default), the FP64 elimination below decides, as for every
-        // system it accepts or rejects as not positive definite.
-        bool ok32 = false;
-        if (D.solve != GLT_SOLVE_FP64) {
-            float e = lane < 28 ? f32_of(S.H[8 * ei + ek]) : 0.0f;
-            const double diag = S.H[8 * row + row];
-            const double a0 = fma(lambda, diag, diag);
-            const float a0f = f32_of(a0);
-            float dg = a0f, dinv = 0.0f;
-            float y = -f32_of(S.g[row]);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float d = __shfl_sync(full, dg, j);
-                const float r = __frcp_rn(d);
-                if (lane == j) dinv = r;
-                if (j < 7) {
-                    const float l = e * r;
-                    const int cj = j * 7 - (j * (j - 1)) / 2 - j - 1;
-                    const bool trail = lane < 28 && ek > j;
-                    const bool drow = lane > j && lane < 8;
-                    const float li = __shfl_sync(full, l, cj + (trail ? ei : j + 1));
-                    const float ak = __shfl_sync(full, e, cj + (trail ? ek : j + 1));
-                    const float ld = __shfl_sync(full, l, cj + (drow ? lane : j + 1));
-                    const float ad = __shfl_sync(full, e, cj + (drow ? lane : j + 1));
-                    const float yj = __shfl_sync(full, y, j);
-                    if (trail) e = fmaf(-li, ak, e);
-                    if (drow) {
-                        dg = fmaf(-ld, ad, dg);
-                        y = fmaf(-ld, yj, y);
-                    }
-                    if (lane < 28 && ek == j) e = l;
-                }
-            }
-            ok32 = __all_sync(full, dg > 1e-4f * a0f || lane >= 8);
-            if (ok32) {
-                // column `row` of L (entries below the diagonal) gathered into the row's lane
-                float Lcol[8];
-#pragma unroll
-                for (int i = 1; i < 8; ++i) {
-                    const int cr = row * 7 - (row * (row - 1)) / 2 - row - 1;
-                    const float v = __shfl_sync(full, e, row < i ? cr + i : 0);
-                    Lcol[i] = row < i ? v : 0.0f;
-                }
-                // diagonal, backward (L^T x = D^-1 y)
-                float x = y * dinv;
-#pragma unroll
-                for (int j = 7; j >= 1; --j) {
-                    const float xj = __shfl_sync(full, x, j);
-                    if (row < j) x = fmaf(-Lcol[j], xj, x);
-                }
-                const double x64 = f64_of(x);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) dl[c] = __shfl_sync(full, x64, c);
-                solved = true;
-            }
-        }
-        if (!ok32) {
-            // ---- the FP64 elimination (the layout above, FP64 reciprocals)
-            double e = lane < 28 ? S.H[8 * ei + ek] : 0.0;
-            const double diag = S.H[8 * row + row];
-            const double a0 = fma(lambda, diag, diag);   // damped diagonal (lanes 0-7)
-            double dg = a0;
-            double dinv = 0.0;
-            // the forward substitution L y = -g rides along: y_i -= l_ij y_j with the
-            // l_ij the diagonal update already fetched (lanes 0-7 hold y_i)
-            double y = -S.g[row];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const double d = __shfl_sync(full, dg, j);
-                const double r = rcp_d(d);
-                if (lane == j) dinv = r;
-                if (j < 7) {
-                    const double l = e * r;                         // l_ij on the lanes of column j
-                    const int cj = j * 7 - (j * (j - 1)) / 2 - j - 1;   // lane of (i, j) is cj + i
-                    const bool trail = lane < 28 && ek > j;        // entry (i, k), k > j: -= l_ij a_kj
-                    const bool drow = lane > j && lane < 8;          // diagonal d_i, i > j: -= l_ij a_ij
-                    const double li = __shfl_sync(full, l, cj + (trail ? ei : j + 1));
-                    const double ak = __shfl_sync(full, e, cj + (trail ? ek : j + 1));
-                    const double ld = __shfl_sync(full, l, cj + (drow ? lane : j + 1));
-                    const double ad = __shfl_sync(full, e, cj + (drow ? lane : j + 1));
-                    const double yj = __shfl_sync(full, y, j);
-                    if (trail) e = fma(-li, ak, e);
-                    if (drow) {
-                        dg = fma(-ld, ad, dg);
-                        y = fma(-ld, yj, y);
-                    }
-                    if (lane < 28 && ek == j) e = l;
-                }
-            }
-            // pivots checked once, each lane its own: d > 0 and d > 1e-13 * damped diagonal
-            const bool piv_ok = dg > 1e-13 * a0 && dg > 0.0;
-            const bool ok = __all_sync(full, piv_ok || lane >= 8);
-            if (!ok) {
-                if (lane == 0) S.status |= GLT_TRACK_NOT_PD;
-                finish = true;
-                next_level = true;
-            } else {
-                // column `row` of L (entries below the diagonal) gathered into the row's lane
-                double Lcol[8];
-#pragma unroll
-                for (int i = 1; i < 8; ++i) {
-                    const int cr = row * 7 - (row * (row - 1)) / 2 - row - 1;
-                    const double v = __shfl_sync(full, e, row < i ? cr + i : 0);
-                    Lcol[i] = row < i ? v : 0.0;
-                }
-                // diagonal, backward (L^T x = D^-1 y)
-                double x = y * dinv;
-#pragma unroll
-                for (int j = 7; j >= 1; --j) {
-                    const double xj = __shfl_sync(full, x, j);
-                    if (row < j) x = fma(-Lcol[j], xj, x);
-                }
-#pragma unroll
-                for (int c = 0; c < 8; ++c) dl[c] = __shfl_sync(full, x, c);
-                solved = true;
-            }
-        }
-    }
-    if (solved) {
-        {
-            long long mbits = 0;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) mbits = max(mbits, abs_bits(dl[c]));
-            double tc;
-            if (D.solve == GLT_SOLVE_FP32) {
-                // ---- exp(delta_xi) - I in FP32: its entries are O(|delta|), so FP32
-                // rounding leaves ~1e-7 |delta| (absolute); the product with T is FP64.
-                //   R_e - I = A [w]x + B [w]x^2,  t_e = v + B (w x v) + C w x (w x v),
-                // A = sin th / th, B = (1 - cos th) / th^2, C = (th - sin th) / th^3
-                // (power series below th^2 = 0.25, truncation < 3e-11 relative)
-                const float v0 = f32_of(dl[0]), v1 = f32_of(dl[1]), v2 = f32_of(dl[2]);
-                const float w0 = f32_of(dl[3]), w1 = f32_of(dl[4]), w2 = f32_of(dl[5]);
-                const float th2 = fmaf(w0, w0, fmaf(w1, w1, w2 * w2));
-                float A, B, Cc;
-                if (th2 < 0.25f) {
-                    A = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 362880.0f, -1.0f / 5040.0f), th2, 1.0f / 120.0f), th2, -1.0f / 6.0f), th2, 1.0f);
-                    B = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 3628800.0f, -1.0f / 40320.0f), th2, 1.0f / 720.0f), th2, -1.0f / 24.0f), th2, 0.5f);
-                    Cc = fmaf(fmaf(fmaf(fmaf(th2, 1.0f / 39916800.0f, -1.0f / 362880.0f), th2, 1.0f / 5040.0f), th2, -1.0f / 120.0f), th2, 1.0f / 6.0f);
-                } else {
-                    const float th = sqrtf(th2);
-                    const float sn = sinf(th), sh = sinf(0.5f * th);
-                    A = sn / th;
-                    B = 2.0f * sh * sh / th2;
-                    Cc = (th - sn) / (th2 * th);
-                }
-                // one element (r, c) of the 3x4 increment per lane 0-11, every lane
-                // running the same instructions on its own operands:
-                //   (R_e - I)(r, c) = A W_rc + B (w_r w_c - d_rc th2)        (W = [w]x)
-                //   t_e(r)          = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
-                // as  base + cA (a1 b1 - a2 b2) + cB (p q - d th2).
-                const float wv = fmaf(w0, v0, fmaf(w1, v1, w2 * v2));
-                const int er = (lane >> 2) % 3, ec = lane & 3;
-                const float wr = er == 0 ? w0 : (er == 1 ? w1 : w2);
-                const float wr1 = er == 0 ? w1 : (er == 1 ? w2 : w0);   // w_{r+1}
-                const float wr2 = er == 0 ? w2 : (er == 1 ? w0 : w1);   // w_{r+2}
-                const float vr = er == 0 ? v0 : (er == 1 ? v1 : v2);
-                const float vr1 = er == 0 ? v1 : (er == 1 ? v2 : v0);
-                const float vr2 = er == 0 ? v2 : (er == 1 ? v0 : v1);
-                const float wc = ec == 0 ? w0 : (ec == 1 ? w1 : w2);
-                const bool rot = ec < 3;
-                const float drc = (rot && er == ec) ? 1.0f : 0.0f;
-                // W_rc = +w_{r+2} if c = r+1, -w_{r+1} if c = r+2, 0 on the diagonal
-                const float Wrc = ec == (er + 1) % 3 ? -wr2 : (ec == (er + 2) % 3 ? wr1 : 0.0f);
-                const float base = rot ? 0.0f : vr;
-                const float a1 = rot ? Wrc : wr1, b1 = rot ? 1.0f : vr2;
-                const float a2 = rot ? 0.0f : wr2, b2 = rot ? 0.0f : vr1;
-                const float pq = rot ? wc : wv, dd = rot ? drc : vr;
-                const float ex = fmaf(a1, b1, -(a2 * b2));
-                const float ey = fmaf(wr, pq, -(dd * th2));
-                const float dE = fmaf(rot ? B : Cc, ey, fmaf(rot ? A : B, ex, base));
-                // ---- Tc = T exp(delta) = T + T (exp(delta) - I) in FP64:
-                // Tc(r, c) = T(r, c) + sum_k T(r, k) dE(k, c)   (c = 3: dE(k, 3) = t_e(k))
-                const double e0 = f64_of(__shfl_sync(full, dE, ec));
-                const double e1 = f64_of(__shfl_sync(full, dE, 4 + ec));
-                const double e2 = f64_of(__shfl_sync(full, dE, 8 + ec));
-                tc = lane < 12 ? fma(S.T[4 * er], e0, fma(S.T[4 * er + 1], e1, fma(S.T[4 * er + 2], e2, S.T[4 * er + ec])))
-                               : 0.0;
-            } else {
-                // ---- exp(delta_xi): R_e = I + A [w]x + B [w]x^2, t_e = v + B (w x v) + C w x (w x v)
-                const double w0 = dl[3], w1 = dl[4], w2 = dl[5];
-                const double th2 = fma(w0, w0, fma(w1, w1, w2 * w2));
-                double A, B, Cc;
-                if (th2 < 1e-4) {
-                    A = fma(fma(th2, 1.0 / 120.0, -1.0 / 6.0), th2, 1.0);
-                    B = fma(fma(th2, 1.0 / 720.0, -1.0 / 24.0), th2, 0.5);
-                    Cc = fma(fma(th2, 1.0 / 5040.0, -1.0 / 120.0), th2, 1.0 / 6.0);
-                } else if (th2 < 0.01) {
-                    A = fma(fma(fma(fma(th2, 1.0 / 362880.0, -1.0 / 5040.0), th2, 1.0 / 120.0), th2, -1.0 / 6.0), th2, 1.0);
-                    B = fma(fma(fma(fma(th2, 1.0 / 3628800.0, -1.0 / 40320.0), th2, 1.0 / 720.0), th2, -1.0 / 24.0), th2, 0.5);
-                    Cc = fma(fma(fma(fma(th2, 1.0 / 39916800.0, -1.0 / 362880.0), th2, 1.0 / 5040.0), th2, -1.0 / 120.0), th2, 1.0 / 6.0);
-                } else {
-                    const double th = sqrt(th2);
-                    double sn, cs, sh, ch;
-                    sincos(th, &sn, &cs);
-                    sincos(0.5 * th, &sh, &ch);
-                    A = sn / th;
-                    B = 2.0 * sh * sh / th2;
-                    Cc = (th - sn) / (th2 * th);
-                }
-                // ---- E = exp(delta_xi) as a 3x4 [R_e | t_e], one element (r, c) per lane
-                // 0-11, every lane running the same FP64 instructions on its own operands:
-                //   R_e(r, c) = d_rc + A W_rc + B (w_r w_c - d_rc th2)            (W = [w]x)
-                //   t_e(r)    = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
-                // as  base + cA (a1 b1 - a2 b2) + cB (p q - d th2).
-                const double v0 = dl[0], v1 = dl[1], v2 = dl[2];
-                const double wv = fma(w0, v0, fma(w1, v1, w2 * v2));
-                const int er = (lane >> 2) % 3, ec = lane & 3;
-                const double wr = er == 0 ? w0 : (er == 1 ? w1 : w2);
-                const double wr1 = er == 0 ? w1 : (er == 1 ? w2 : w0);   // w_{r+1}
-                const double wr2 = er == 0 ? w2 : (er == 1 ? w0 : w1);   // w_{r+2}
-                const double vr = er == 0 ? v0 : (er == 1 ? v1 : v2);
-                const double vr1 = er == 0 ? v1 : (er == 1 ? v2 : v0);
-                const double vr2 = er == 0 ? v2 : (er == 1 ? v0 : v1);
-                const double wc = ec == 0 ? w0 : (ec == 1 ? w1 : w2);
-                const bool rot = ec < 3;
-                const double drc = (rot && er == ec) ? 1.0 : 0.0;
-                // W_rc = +w_{r+2} if c = r+1, -w_{r+1} if c = r+2, 0 on the diagonal
-                const double Wrc = ec == (er + 1) % 3 ? -wr2 : (ec == (er + 2) % 3 ? wr1 : 0.0);
-                const double base = rot ? drc : vr;
-                const double a1 = rot ? Wrc : wr1, b1 = rot ? 1.0 : vr2;
-                const double a2 = rot ? 0.0 : wr2, b2 = rot ? 0.0 : vr1;
-                const double pq = rot ? wc : wv, dd = rot ? drc : vr;
-                const double ex = fma(a1, b1, -(a2 * b2));
-                const double ey = fma(wr, pq, -(dd * th2));
-                const double E = fma(rot ? B : Cc, ey, fma(rot ? A : B, ex, base));
-                // ---- Tc = T E: Tc(r, c) = sum_k T(r, k) E(k, c) (+ T(r, 3) for c = 3)
-                const double e0 = __shfl_sync(full, E, ec);
-                const double e1 = __shfl_sync(full, E, 4 + ec);
-                const double e2 = __shfl_sync(full, E, 8 + ec);
-                tc = lane < 12 ? fma(S.T[4 * er], e0, fma(S.T[4 * er + 1], e1,
-                                      fma(S.T[4 * er + 2], e2, rot ? 0.0 : S.T[4 * er + 3])))
-                               : 0.0;
-            }
-            const double ac = S.a + dl[6], bc = S.b + dl[7];
-            const bool cand_finite = __all_sync(full, abs_bits(tc) < kInfBits) &&
-                                     abs_bits(ac) < kInfBits && abs_bits(bc) < kInfBits;
-            // a step below the level's stop threshold (and below accept_step)
-            // would be taken whatever its cost and would end the level, so it
-            // is taken here without a pass of its own: the next level's start
-            // pass is the first evaluation of the new state; on the finest
-            // level the result keeps the cost and count of the last evaluated
-            // state
-            const bool take_now = mbits < abs_bits(level > 0 ? D.eps_step_coarse : D.eps_step) &&
-                                  mbits < abs_bits(D.accept_step);
-            if (!cand_finite) {
-                // the solve produced a state that is not finite: keep the
-                // accepted one and end the level
-                if (lane == 0) S.status |= GLT_TRACK_DIVERGED;
-                finish = true;
-                next_level = true;
-            } else if (take_now) {
-                if (lane < 12) S.T[lane] = tc;
-                if (lane == 0) {
-                    S.a = ac;
-                    S.b = bc;
-                    S.moved = 1;
-                }
-                ++it;
-                finish = true;
-                next_level = true;
-            } else {
-                if (lane < 12) S.Tc[lane] = tc;
-                if (lane == 0) {
-                    S.ac = ac;
-                    S.bc = bc;
-                    S.maxstep_bits = mbits;
-                    S.phase = PH_CAND;
-                }
-                make_pass_params_lane(tc, ac, bc, level, P, lane);
-            }
-        }
-    }
-    if (finish && lane == 0) {
-        S.iters[level] = it;
-        S.res_E = S.E;
-        S.res_n = S.n;
     }
     __syncwarp();
     if (next_level) {
-        int l = level - 1;
-        while (l >= 0 && D.max_iters[l] <= 0) --l;
+        int l = level;
+        do --l;
+        while (l >= 0 && D.max_iters[l] <= 0);
+        cur = S.cur;
         if (l < 0) {
             // GLT_SOLVE_FP32: the poses composed from FP32 increments drift
             // from orthonormal by ~1e-9 per step: one Newton step R' = R (3 I - R^T R) / 2 =
             // R + R (I - R^T R) / 2 on the final pose (FP64; the deviation
             // becomes its square)
             if (S.moved && D.solve == GLT_SOLVE_FP32) {
+                double* T = S.T[cur];
                 const int i = lane / 3, j = lane % 3;
                 double dlt = lane < 9 ? (i == j ? 1.0 : 0.0) : 0.0;
                 if (lane < 9) {
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) dlt = fma(-S.T[4 * k + i], S.T[4 * k + j], dlt);
+                    for (int k = 0; k < 3; ++k) dlt = fma(-T[4 * k + i], T[4 * k + j], dlt);
                 }
                 const int r = lane >> 2, c = lane & 3;
                 const int cc = c < 3 ? c : 0;
@@ -1463,10 +1602,9 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
                              d2 = __shfl_sync(full, dlt, 6 + cc);
                 double v = 0.0;
                 if (lane < 12 && c < 3)
-                    v = fma(0.5, fma(S.T[4 * r], d0, fma(S.T[4 * r + 1], d1, S.T[4 * r + 2] * d2)),
-                            S.T[lane]);
+                    v = fma(0.5, fma(T[4 * r], d0, fma(T[4 * r + 1], d1, T[4 * r + 2] * d2)), T[lane]);
                 __syncwarp();
-                if (lane < 12 && c < 3) S.T[lane] = v;
+                if (lane < 12 && c < 3) T[lane] = v;
             }
             if (lane == 0) {
                 S.done = 1;
@@ -1477,7 +1615,12 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
                 S.level = l;
                 S.phase = PH_START;
             }
-            make_pass_params_warp(S.T, S.a, S.b, l, P, lane);
+            if (!evaluated)
+                make_pass_params_warp(S.T[cur], S.ab[cur][0], S.ab[cur][1], l, P, lane);
+            else if (lane == 13) {
+                P.level = l;
+                P.scale = ldexpf(1.0f, -l);
+            }
         }
     }
     __syncwarp();
@@ -1486,9 +1629,9 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
 __device__ inline void solver_write_result(const StreamDesc& D, const Solver& S, glt_result* out)
 {
     if (D.trace_count) *D.trace_count = S.passes;
-    for (int i = 0; i < 12; ++i) out->T[i] = S.T[i];
-    out->a = S.a;
-    out->b = S.b;
+    for (int i = 0; i < 12; ++i) out->T[i] = S.T[S.cur][i];
+    out->a = S.ab[S.cur][0];
+    out->b = S.ab[S.cur][1];
     out->cost = S.res_n > 0 ? S.res_E / (double)S.res_n : S.res_E;
     out->n_valid = S.res_n;
     int tot = 0;

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
     __shared__ __align__(16) float part[2][XW];
     __shared__ __align__(16) Exchange<XW> X;
     __shared__ double tot[kAccPad];
+    __shared__ int tot_n;            // tot's sample count as an integer
     __shared__ int xfail;
 
     cg::cluster_group cluster = cg::this_cluster();
@@ -139,6 +140,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
         int* dst = reinterpret_cast<int*>(&sD);
         for (int i = tid; i < (int)(sizeof(StreamDesc) / sizeof(int)); i += THREADS) dst[i] = src[i];
     }
+    if (tid < 32) tail_map_init(S, tid);
+    if (tid < kAccPad) tot[tid] = 0.0;
     __syncthreads();
     if (tid == 0) {
         solver_init(sD, init + 14 * user, S, P);
@@ -221,6 +224,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
                 }
             }
             tot[tid] = (double)hi + (double)lo;
+            if (tid == (HC ? kHcN : kIdxN)) tot_n = (int)hi + (int)lo;
         }
         xph ^= 1u << par;
         __syncthreads();
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
         }
         // the FP64 tail runs on one warp; CTAs of different streams that share an
         // SM use different warps so their tails spread over the SM's sub-partitions
-        if ((tid >> 5) == tail_warp) solver_step_warp<HC>(sD, tot, S, P, tid & 31, rank == 0);
+        if ((tid >> 5) == tail_warp) solver_step_warp<HC>(sD, tot, tot_n, S, P, tid & 31, rank == 0);
         __syncthreads();
         par ^= 1;
     }
@@ -271,11 +275,14 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
     __shared__ __align__(16) float part[2][XW];
     __shared__ __align__(16) Exchange<XW> X;
     __shared__ double tot[kAccPad];
+    __shared__ int tot_n;            // tot's sample count as an integer
     __shared__ int xfail;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x;
+    if (tid < 32) tail_map_init(S, tid);
+    if (tid < kAccPad) tot[tid] = 0.0;
     if (tid == 0) {
         int* z = reinterpret_cast<int*>(&sD);
         for (int i = 0; i < (int)(sizeof(StreamDesc) / sizeof(int)); ++i) z[i] = 0;
@@ -350,11 +357,12 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
                     if (tid == upper_index(i, i)) x = 100.0 + 10.0 * i;
             }
             tot[tid] = x + (double)hi + (double)lo;
+            if (tid == (HC ? kHcN : kIdxN)) tot_n = 1000 + (int)hi + (int)lo;
         }
         xph ^= 1u << par;
         __syncthreads();
         if (xfail) break;
-        if ((tid >> 5) == (int)(blockIdx.x % NW)) solver_step_warp<HC>(sD, tot, S, P, tid & 31, false);
+        if ((tid >> 5) == (int)(blockIdx.x % NW)) solver_step_warp<HC>(sD, tot, tot_n, S, P, tid & 31, false);
         __syncthreads();
         par ^= 1;
     }
