@@ -118,7 +118,7 @@ __device__ __forceinline__ T* checked(T* p, size_t, T*, size_t, int)
 // The state one linearisation pass is evaluated at, in the form the FP32
 // gather uses: R - I and t rounded from the FP64 pose, e^a, b.
 struct PassParams {
-    float Rm[9];
+    float Rm[9];           // the first 14 floats are also written by index (tail_map_init)
     float t[3];
     float ea, b;
     float scale;           // 2^-level
@@ -816,16 +816,15 @@ __device__ __forceinline__ void block_reduce(float (&acc)[kAccPad], float (*red)
 //  * accept/reject compares E' n <= E n' instead of dividing, and only for
 //    steps that are not small enough to be taken anyway.
 // ---------------------------------------------------------------------------
-// 1 / d as the unevaluated sum r0 + rl of two doubles, for a positive d in
-// [2^-100, 2^100).  With d = 2^E m, m = mh + ml in [1, 2) split at FP32's 24
-// bits (ml cut at 2^-46): q = rcp.approx.ftz.f32(mh), the residual e = 1 - m q
-// in two FP32 FMAs (error below 2^-46, |e| < 2^-21), and 1 / m = q / (1 - e) =
-// q + q (e + e^2) + O(e^3): r0 = q, rl the FP32 correction, both scaled by
-// 2^-E through their exponent bits.  No FP64 instruction, relative error below
-// 2^-45; the Newton step in FP64 that this replaces cost two dependent FP64
-// instructions (128 cycles) for 2^-44.  (A correction of zero gives rl =
-// 2^-127 r0, which no double sum sees.)
-__device__ __forceinline__ void rcp_pair(double d, double& r0, double& rl)
+// 1 / d for a positive d in [2^-100, 2^100) without an FP64 instruction.  With
+// d = 2^E m, m = mh + ml in [1, 2) split at FP32's 24 bits (ml cut at 2^-46):
+// q = rcp.approx.ftz.f32(mh), the residual e = 1 - m q in two FP32 FMAs (error
+// below 2^-46, |e| <= 2^-22), and 1 / m = q / (1 - e) = q + q (e + e^2) +
+// O(e^3): the FP32 correction is added to q's significand as an integer in
+// units of 2^-52, and the exponent lowered by E.  Relative error below 2^-45;
+// the Newton step in FP64 that this replaces cost two dependent FP64
+// instructions (128 cycles) for 2^-44.
+__device__ __forceinline__ double rcp_mid(double d)
 {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     const float mh = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u);
@@ -833,23 +832,19 @@ __device__ __forceinline__ void rcp_pair(double d, double& r0, double& rl)
     float q;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
     const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
-    const float c = q * fmaf(e, e, e);
-    // FP32 bits to FP64's: the exponent re-biased and lowered by E
+    const int c = __float2int_rn((q * 0x1p52f) * fmaf(e, e, e));
     const unsigned off = ((896u + 1023u) << 20) - (hi & 0x7ff00000u);
-    const unsigned qb = __float_as_uint(q), cb = __float_as_uint(c);
-    r0 = __hiloint2double((int)((qb >> 3) + off), (int)(qb << 29));
-    rl = __hiloint2double((int)((((cb >> 3) & 0x0fffffffu) + off) | (cb & 0x80000000u)), (int)(cb << 29));
+    const long long m = ((long long)__float_as_uint(q) << 29) + 2ll * c + ((long long)off << 32);
+    return __longlong_as_double(m);
 }
 
-// Reciprocal of any d: rcp_pair for 2^-100 <= |d| < 2^100 (exponent tested as
+// Reciprocal of any d: rcp_mid for 2^-100 <= |d| < 2^100 (exponent tested as
 // an integer); zero, infinities, NaN and the rest divide.
 __device__ __forceinline__ double rcp_d(double d)
 {
     const int ebits = (__double2hiint(d) >> 20) & 0x7ff;
     if (ebits < 1023 - 100 || ebits >= 1023 + 100) return 1.0 / d;
-    double r0, rl;
-    rcp_pair(fabs(d), r0, rl);
-    return copysign(r0 + rl, d);
+    return copysign(rcp_mid(fabs(d)), d);
 }
 
 // FP64 -> FP32 through the bit pattern (integer instructions only, nothing on
@@ -876,20 +871,20 @@ __device__ __forceinline__ float f32_of(double x)
 }
 
 // FP64 -> FP32 rounded to nearest even, as the conversion instruction does it,
-// in integer instructions (the conversion takes its turn on the FP64 pipe);
-// results below FP32's normal range, infinities and NaN are left to it.
+// in integer instructions (the conversion takes its turn on the FP64 pipe), for
+// finite x; magnitudes below FP32's normal range give a signed zero.
 __device__ __forceinline__ float f32_rn(double x)
 {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const unsigned eb = (hi >> 20) & 0x7ffu;
-    if (eb - 897u >= 254u && ((hi & 0x7fffffffu) | lo) != 0u) return (float)x;
-    // sign, re-biased exponent, 23 bits of the significand; a carry out of the
+    // re-biased exponent, 23 bits of the significand; a carry out of the
     // rounded significand steps the exponent
-    unsigned b = __funnelshift_l(lo, hi, 3) & 0x7fffffu;
-    b |= (eb - 896u) << 23;
+    unsigned b = (__funnelshift_l(lo, hi, 3) & 0x7fffffu) | ((eb - 896u) << 23);
     const unsigned rem = lo << 3;                  // what the cut leaves, 2^31 is half
-    b += (rem > 0x80000000u || (rem == 0x80000000u && (b & 1u))) ? 1u : 0u;
-    return __uint_as_float((eb ? b : 0u) | (hi & 0x80000000u));
+    if (rem > 0x80000000u - (b & 1u)) ++b;
+    if (eb < 897u) b = 0u;
+    if (eb > 1150u) b = 0x7f800000u;
+    return __uint_as_float(b | (hi & 0x80000000u));
 }
 
 // FP32 -> FP64 through the bit pattern: exact for zero and normal numbers
@@ -966,38 +961,63 @@ __device__ __forceinline__ void make_pass_params_warp(const double* T, double a,
 // runs it on bit-identical inputs, so all take the same decisions).
 enum { PH_START = 0, PH_CAND = 1 };
 
-constexpr int kXs0 = 8, kXs1 = 9, kXsPoly = 10, kXsTable = 19;
+// Constants behind the two states and behind the step, so that a lane fetches
+// every operand by index (no selects, no divergence).
+constexpr int kSt0 = 14, kSt1 = 15, kStM1 = 16, kStDown = 17, kStUp = 18, kStSize = 20;
+constexpr int kXs0 = 8, kXs1 = 9, kXsPoly = 10, kXsSize = 20;
+
+// w.w: the state machine's flags
+constexpr int kFlCur = 1;      // which state is the accepted one
+constexpr int kFlAcc = 2;      // which sums are the accepted state's
+constexpr int kFlCand = 4;     // phase: the pass evaluates a candidate
+constexpr int kFlSmall = 8;    // the candidate's step is below accept_step
+constexpr int kFlStop = 16;    // ... below the level's stop threshold
+constexpr int kFlMoved = 32;   // the pose changed since the initial state
+constexpr int kFlLevel = 8;    // the level, from this bit on
 
 struct Solver {
-    // two states (pose, affine pair): the accepted one at [cur], the candidate
-    // under evaluation at [cur ^ 1]; accepting a candidate flips cur
-    double T[2][12], ab[2][2];
-    double ema;               // cached-Hessian form: e^-a (a is held fixed there)
-    double N[kAccPad];        // sums at the accepted state
+    // two states [T (12), a, b, then the constants 0, 1, -1 and the damping
+    // factors]: the accepted one and the candidate under evaluation
+    double st[2][kStSize];
+    // two sets of sums: the accepted state's and the last pass's (zeros from
+    // kNumAcc on); n[]: their sample counts as integers
+    double tot[2][kAccPad];
+    double xs[kXsSize];       // the step (translation, rotation, da, db), then 0, 1 and the
+                              // series of A, B, C (tail_map_init)
+    double Lm[72];            // L row by row, then D^-1 L^-1 times the right-hand side
     double Hi[36];            // cached-Hessian form: -e^-a H^-1 of the level
-    double E, nd, res_E;      // energy / samples (as double) at the accepted state
-    double lam_dn, lam_up;    // the damping after the candidate is accepted / rejected
-    double xs[kXsTable];      // the step (translation, rotation, da, db), then the constants
-                              // 0, 1 and the series of A, B, C (see tail_map_init)
-    double Lm[72];            // L (row by row), then D^-1 L^-1 times the right-hand side
-    long long maxstep_bits;   // max |delta_xi| of the candidate, as abs_bits
-    int cur, hc_ok;           // hc_ok: the level's reference Hessian is positive definite
-    int n, res_n, level, it, phase, status, passes, done;
-    int moved;                // the pose changed since the initial state
+    double lam[2];            // the damping after the candidate is accepted / rejected
+    double ema;               // cached-Hessian form: e^-a (a is held fixed there)
+    double res_E;
+    int4 w;                   // iterations of the level, status, passes, flags
+    int n[2], bad;            // bad: a sum of the last pass is not finite
+    int hc_ok;                // the level's reference Hessian is positive definite
+    int res_n;
     int iters[kMaxLevels];
-    unsigned map_ldl[32], map_dot[32], map_ent[32];   // per lane, packed (tail_map_init)
+    unsigned map_ldl[32], map_dot[32], map_ent[32], map_cmp[32];   // per lane (tail_map_init)
 };
 
 // Upper-triangle index of (i, j), i <= j, in the accumulator layout.
-__device__ __forceinline__ int upper_index(int i, int j) { return i * 8 - (i * (i - 1)) / 2 + (j - i); }
+__host__ __device__ __forceinline__ constexpr int upper_index(int i, int j) { return i * 8 - (i * (i - 1)) / 2 + (j - i); }
+
+// The sums' buffer a pass writes, and one finished sum (of n samples) into it.
+__device__ __forceinline__ int solver_buffer(const Solver& S) { return (S.w.w & kFlAcc) ? 0 : 1; }
+
+template <bool HC>
+__device__ __forceinline__ void solver_put_sum(Solver& S, int wb, int i, double v, int n)
+{
+    S.tot[wb][i] = v;
+    // sums that are not finite (an FP32 overflow) make the pass unusable
+    if (!(abs_bits(v) < kInfBits)) S.bad = 1;
+    if (i == (HC ? kHcN : kIdxN)) S.n[wb] = n;
+}
 
 // Initial state (one thread): Gram-Schmidt the initial rotation, first level.
 __device__ inline void solver_init(const StreamDesc& D, const double* init, Solver& S, PassParams& P)
 {
-    S.cur = 0;
-    for (int i = 0; i < 12; ++i) S.T[0][i] = init[i];
+    double* T = S.st[0];
+    for (int i = 0; i < 14; ++i) T[i] = init[i];
     {
-        double* T = S.T[0];
         const double n0 = sqrt(T[0] * T[0] + T[1] * T[1] + T[2] * T[2]);
         for (int c = 0; c < 3; ++c) T[c] /= n0;
         const double d = T[4] * T[0] + T[5] * T[1] + T[6] * T[2];
@@ -1008,60 +1028,41 @@ __device__ inline void solver_init(const StreamDesc& D, const double* init, Solv
         T[9] = T[2] * T[4] - T[0] * T[6];
         T[10] = T[0] * T[5] - T[1] * T[4];
     }
-    S.ab[0][0] = init[12];
-    S.ab[0][1] = init[13];
-    S.status = 0;
+    for (int k = 0; k < 2; ++k) {
+        S.st[k][kSt0] = 0.0;
+        S.st[k][kSt1] = 1.0;
+        S.st[k][kStM1] = -1.0;
+        S.st[k][kStDown] = D.lambda_down;
+        S.st[k][kStUp] = D.lambda_up;
+    }
+    int status = 0;
     bool finite_start = true;
-    for (int i = 0; i < 12; ++i) finite_start &= abs_bits(S.T[0][i]) < kInfBits;
-    finite_start &= abs_bits(S.ab[0][0]) < kInfBits && abs_bits(S.ab[0][1]) < kInfBits;
-    S.passes = 0;
-    S.it = 0;
-    S.n = 0;
-    S.nd = 0.0;
-    S.E = 0.0;
-    S.maxstep_bits = 0;
+    for (int i = 0; i < 14; ++i) finite_start &= abs_bits(T[i]) < kInfBits;
+    S.n[0] = S.n[1] = 0;
+    S.bad = 0;
     S.res_n = 0;
     S.res_E = __longlong_as_double(0x7ff8000000000000ll);
-    S.done = 0;
-    S.moved = 0;
     for (int l = 0; l < kMaxLevels; ++l) S.iters[l] = 0;
-    S.ema = (D.Hc && finite_start) ? exp(-S.ab[0][0]) : 1.0;
+    S.ema = (D.Hc && finite_start) ? exp(-T[12]) : 1.0;
     int l = D.L - 1;
     while (l >= 0 && D.max_iters[l] <= 0) --l;
     if (!finite_start) {
         // a start that is not finite (or whose rotation is degenerate) is
         // not solved: the result is the start, flagged
-        S.status |= GLT_TRACK_DIVERGED;
+        status |= GLT_TRACK_DIVERGED;
         l = -1;
     }
-    S.level = l;
-    S.phase = PH_START;
-    if (l < 0) {
-        S.done = 1;
+    S.w = make_int4(0, status, 0, (l < 0 ? 0 : l) << kFlLevel);
+    if (l < 0)
         P.done = 1;
-    } else {
-        make_pass_params(S.T[0], S.ab[0][0], S.ab[0][1], l, P);
-    }
+    else
+        make_pass_params(T, T[12], T[13], l, P);
 }
 
-// (H + lambda diag H) delta = -g by L D L^T, right-looking, one entry per
-// lane.  The right-hand side rides along as row 8 of the lower triangle
-// (entry (8, k) = y_k), so the 44 entries (i, k), k <= i <= 8, all follow
-//   a_ik -= a_ij a_kj / d_j   for k > j.
-// Columns 2-7 (27 entries) sit in register A of lanes 0-26 and take one pair
-// of FMAs per eliminated column; columns 0 and 1 sit in register B of lanes
-// 0-8 and 9-16, of which column 1 is updated once.  Column k starts at lane
-// cA(k) of A, so entry (i, j) is on lane cA(j) - j + i (B: i for j = 0, 8 + i
-// for j = 1); a lane without part in a step takes its factors from lane 31,
-// which holds zeros.  The product a_ij a_kj is formed while the pivot's
-// reciprocal is, so a column's dependent chain is a shuffle, the product and
-// the two FMAs with the reciprocal's two parts: 300 cycles, 4.2k for the whole
-// solve.  (The form with l_ij = a_ij / d_j, a Newton step in FP64 and separate
-// updates of the diagonal and the right-hand side took 6.9k.)
+// Per-lane tables of the tail, packed, and its constants (one warp, once per
+// launch; the caller synchronises).
 __host__ __device__ constexpr int ldl_lane(int k) { return k == 2 ? 0 : k == 3 ? 7 : k == 4 ? 13 : k == 5 ? 18 : k == 6 ? 22 : 25; }
 
-// Per-lane tables of the tail, packed into three words, and the constants
-// behind the step (one warp, once per launch; the caller synchronises).
 __device__ inline void tail_map_init(Solver& S, int lane)
 {
     // L D L^T: positions of the lane's entries in the sums, and (i, k) of both
@@ -1081,18 +1082,25 @@ __device__ inline void tail_map_init(Solver& S, int lane)
     const int p3 = cross ? kXs0 : 5, q3 = cross ? kXs0 : dot ? 2 : 5;
     S.map_dot[lane] = (unsigned)(p1 | (q1 << 5) | (p2 << 10) | (q2 << 15) | (p3 << 20) | (q3 << 25));
     // entry (er, ec) of the exponential on lane 4 er + ec < 12: w_er, the
-    // column's w (rotation), d_rc or v_er, and W_rc = +w_{r+2} if c = r+1,
-    // -w_{r+1} if c = r+2; lanes 12-14: the series of A, B, C
-    const int er = (lane >> 2) % 3, ec = lane & 3, er1 = (er + 1) % 3, er2 = (er + 2) % 3;
-    const bool poly = lane >= 12 && lane < 15;
+    // column's w (rotation), d_rc or v_er, and W_rc = +w_{r+2} if c = r+1 (bit
+    // 25: negated), w_{r+1} if c = r+2; lanes 12-14: the series of A, B, C
+    const int q = lane & 15, er = (q >> 2) % 3, ec = q & 3, er1 = (er + 1) % 3, er2 = (er + 2) % 3;
+    const bool poly = lane >= 12 && lane < 15, rot = ec < 3;
     const int g = lane - 12;
     const int w = poly ? kXsPoly + 6 + g : 3 + er;
-    const int pq = ec < 3 ? 3 + ec : kXs0;
-    const int dd = poly ? kXsPoly + g : ec < 3 ? (er == ec ? kXs1 : kXs0) : er;
+    const int pq = rot ? 3 + ec : kXs0;
+    const int dd = poly ? kXsPoly + g : rot ? (er == ec ? kXs1 : kXs0) : er;
     const int c1 = poly ? kXsPoly + 3 + g : kXs0;
-    const int W = ec == er1 ? 3 + er2 : (ec < 3 && ec == er2) ? 3 + er1 : kXs0;
-    S.map_ent[lane] = (unsigned)(w | (pq << 5) | (dd << 10) | (c1 << 15) | (W << 20)) |
-                      (ec == er1 ? 1u << 25 : 0u);
+    const int W = ec == er1 ? 3 + er2 : (rot && ec == er2) ? 3 + er1 : kXs0;
+    S.map_ent[lane] = (unsigned)(w | (pq << 5) | (dd << 10) | (c1 << 15) | (W << 20)) | (ec == er1 ? 1u << 25 : 0u);
+    // the composition (indices into a state): row er of T on lanes 4 er + ec
+    // and 16 + 4 er + ec, the addend (translation, or minus the identity on
+    // lanes 0-11), 1 x da + a, 1 x db + b and the dampings on lanes 12-15
+    const int t0 = q < 12 ? 4 * er : kSt0, t1 = q < 12 ? 4 * er + 1 : kSt0;
+    const int t2 = q < 12 ? 4 * er + 2 : lane == 12 || lane == 13 ? kSt1 : lane == 14 ? kStDown : lane == 15 ? kStUp : kSt0;
+    const int add = q < 12 ? (!rot ? 4 * er + 3 : lane < 12 && er == ec ? kStM1 : kSt0) : lane == 12 || lane == 13 ? lane : kSt0;
+    const int pp = lane < 12 ? (rot ? 3 * er + ec : 9 + er) : lane < 14 ? lane : 0;   // entry of P
+    S.map_cmp[lane] = (unsigned)(t0 | (t1 << 5) | (t2 << 10) | (add << 15) | (pp << 20));
     if (lane == 0) {
         S.xs[kXs0] = 0.0;
         S.xs[kXs1] = 1.0;
@@ -1107,22 +1115,35 @@ __device__ inline void tail_map_init(Solver& S, int lane)
         c[7] = 0.5;
         c[8] = 1.0 / 6.0;
     }
-    for (int i = lane; i < kAccPad; i += 32) S.N[i] = 0.0;
+    for (int i = lane; i < 2 * kAccPad; i += 32) (&S.tot[0][0])[i] = 0.0;
 }
 
-// src: a pass's sums (zeros beyond the last); Lm: 72 doubles of shared memory;
+// (H + lambda diag H) delta = -g by L D L^T, right-looking, one entry per
+// lane.  The right-hand side rides along as row 8 of the lower triangle
+// (entry (8, k) = y_k), so the 44 entries (i, k), k <= i <= 8, all follow
+//   a_ik -= a_ij a_kj / d_j   for k > j.
+// Columns 2-7 (27 entries) sit in register A of lanes 0-26 and take one FMA
+// per eliminated column; columns 0 and 1 sit in register B of lanes 0-8 and
+// 9-16, of which column 1 is updated once.  Column k starts at lane cA(k) of
+// A, so entry (i, j) is on lane cA(j) - j + i (B: i for j = 0, 8 + i for j =
+// 1); a lane without part in a step takes its factors from lane 31, which
+// holds zeros.  The product a_ij a_kj is formed while the pivot's reciprocal
+// is, so a column's dependent chain is a shuffle, the product and one FMA.
+// (With l_ij = a_ij / d_j, a Newton step in FP64 and separate updates of the
+// diagonal and the right-hand side the solve took 6.9k cycles.)
+// tot: a pass's sums (zeros beyond the last); Lm: 72 doubles of shared memory;
 // x: the solution on lanes 0-7.  EXACT: reciprocals of any pivot and the pivot
 // test d > 0, d > 1e-13 x the damped diagonal; otherwise every pivot must
-// pass that test by its exponent alone (2^-43 > 1e-13) and lie in rcp_pair's
+// pass that test by its exponent alone (2^-43 > 1e-13) and lie in rcp_mid's
 // range.  False if one does not.
 template <bool EXACT>
-__device__ __forceinline__ bool ldl_solve_t(const double* src, double lambda, bool fixed_ab, unsigned map,
+__device__ __forceinline__ bool ldl_solve_t(const double* tot, double lambda, bool fixed_ab, unsigned map,
                                             double* Lm, int lane, double& x)
 {
     const unsigned full = 0xffffffffu;
     const int iA = (map >> 12) & 15, kA = (map >> 16) & 15, iB = (map >> 20) & 15, kB = map >> 24;
     const bool dA = iA == kA, dB = iB == kB;                // diagonal entries
-    double B = src[(map >> 6) & 63], A = src[map & 63];
+    double B = tot[(map >> 6) & 63], A = tot[map & 63];
     if (iB == 8) B = -B;                                    // y = -g
     if (iA == 8) A = -A;
     if (fixed_ab) {
@@ -1134,87 +1155,68 @@ __device__ __forceinline__ bool ldl_solve_t(const double* src, double lambda, bo
     B = fma(dB ? lambda : 0.0, B, B);                       // damped diagonal
     A = fma(dA ? lambda : 0.0, A, A);
     const double a0A = A, a0B = B;
-    double r0A = 0.0, rlA = 0.0, r0B = 0.0, rlB = 0.0;      // 1 / d of the lane's columns
+    double rA = 0.0, rB = 0.0, sB = 0.0;                    // 1 / d of the lane's columns
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < 7; ++j) {
         const int cj = j == 0 ? 0 : j == 1 ? 8 : ldl_lane(j) - j;   // lane of (i, j) is cj + i
         const double col = j < 2 ? B : A;
         const double piv = __shfl_sync(full, col, cj + j);
-        double pA = 0.0, pB = 0.0;
-        if (j == 0) {
-            const bool on = kB == 1;
-            pB = __shfl_sync(full, col, on ? iB : 31) * __shfl_sync(full, col, on ? 1 : 31);
-        }
-        if (j < 7) {
-            const bool on = kA > j && kA < 8;
-            pA = __shfl_sync(full, col, on ? cj + iA : 31) * __shfl_sync(full, col, on ? cj + kA : 31);
-        }
-        double r0, rl = 0.0;
-        if (EXACT)
-            r0 = rcp_d(piv);
-        else
-            rcp_pair(piv, r0, rl);
-        if (j == 0) B = fma(-pB, rl, fma(-pB, r0, B));
-        if (j < 7) A = fma(-pA, rl, fma(-pA, r0, A));
-        if (j < 2) {
-            if (kB == j) {
-                r0B = r0;
-                rlB = rl;
-            }
-        } else if (kA == j) {
-            r0A = r0;
-            rlA = rl;
-        }
+        const bool on = kA > j && kA < 8;
+        const double pA = __shfl_sync(full, col, on ? cj + iA : 31) * __shfl_sync(full, col, on ? cj + kA : 31);
+        double pB = 0.0;
+        if (j == 0) pB = __shfl_sync(full, col, kB == 1 ? iB : 31) * __shfl_sync(full, col, kB == 1 ? 1 : 31);
+        const double r = EXACT ? rcp_d(piv) : rcp_mid(piv);
+        if (j == 0) B = fma(-pB, r, B);
+        A = fma(-pA, r, A);
+        if (kB == j) rB = r;
+        if (kA == j) rA = r;
+        if (j == 2) sB = B * rB;                            // columns 0 and 1 of L, z_0 and z_1
     }
-    // L and z = D^-1 y (row 8): every entry times its column's reciprocal
-    const double sB = B * (r0B + rlB), sA = A * (r0A + rlA);
+    // L and z = D^-1 y (row 8): every entry times its column's reciprocal;
+    // column 7 is the last pivot and z_7 only
+    const double piv = __shfl_sync(full, A, 25);
+    const double sA = A * rA;
     if (kB < 8) Lm[8 * iB + kB] = sB;
-    if (kA < 8) Lm[8 * iA + kA] = sA;
+    if (kA < 7) Lm[8 * iA + kA] = sA;
+    const double z7 = A * (EXACT ? rcp_d(piv) : rcp_mid(piv));      // lane 26
     bool ok;
     if (EXACT) {
         ok = (!dA || (A > 1e-13 * a0A && A > 0.0)) && (!dB || (B > 1e-13 * a0B && B > 0.0));
     } else {
-        // exponents of the pivot and of the damped diagonal (positive, normal)
-        const int pA = __double2hiint(A) >> 20, pB = __double2hiint(B) >> 20;
-        const int qA = __double2hiint(a0A) >> 20, qB = __double2hiint(a0B) >> 20;
-        ok = (!dA || (pA >= 1023 - 100 && pA < 1023 + 100 && qA > 0 && pA - qA >= -42)) &&
-             (!dB || (pB >= 1023 - 100 && pB < 1023 + 100 && qB > 0 && pB - qB >= -42));
+        // high words of the pivot and of the damped diagonal
+        const int lo = (1023 - 100) << 20, hi = (1023 + 100) << 20, sl = 42 << 20;
+        const int pA = __double2hiint(A), qA = __double2hiint(a0A);
+        const int pB = __double2hiint(B), qB = __double2hiint(a0B);
+        ok = (!dA || (pA >= lo && pA < hi && qA > 0 && pA >= (qA & 0x7ff00000) - sl)) &&
+             (!dB || (pB >= lo && pB < hi && qB > 0 && pB >= (qB & 0x7ff00000) - sl));
     }
-    if (!__all_sync(full, ok)) return false;
+    ok = __all_sync(full, ok);
     __syncwarp();
     // L^T x = z: lane i < 8 holds x_i and its column of L
     double Lcol[8];
 #pragma unroll
     for (int j = 1; j < 8; ++j) Lcol[j] = lane < j ? Lm[8 * j + lane] : 0.0;
-    x = lane < 8 ? Lm[64 + lane] : 0.0;
+    x = lane < 7 ? Lm[64 + lane] : 0.0;
+    const double x7 = __shfl_sync(full, z7, 26);
+    x = fma(-Lcol[7], x7, x);
+    if (lane == 7) x = x7;
 #pragma unroll
-    for (int j = 7; j >= 1; --j) x = fma(-Lcol[j], __shfl_sync(full, x, j), x);
-    return true;
-}
-
-// kept out of line: near-singular systems only
-static __device__ __noinline__ bool ldl_solve_exact(const double* src, double lambda, bool fixed_ab, unsigned map,
-                                                    double* Lm, int lane, double* x)
-{
-    return ldl_solve_t<true>(src, lambda, fixed_ab, map, Lm, lane, *x);
-}
-
-__device__ __forceinline__ bool ldl_solve_warp(const double* src, double lambda, bool fixed_ab, Solver& S,
-                                               int lane, double& x)
-{
-    const unsigned map = S.map_ldl[lane];
-    if (ldl_solve_t<false>(src, lambda, fixed_ab, map, S.Lm, lane, x)) return true;
-    double xe = 0.0;
-    const bool ok = ldl_solve_exact(src, lambda, fixed_ab, map, S.Lm, lane, &xe);
-    x = xe;
+    for (int j = 6; j >= 1; --j) x = fma(-Lcol[j], __shfl_sync(full, x, j), x);
     return ok;
 }
 
+// kept out of line: near-singular systems only
+static __device__ __noinline__ bool ldl_solve_exact(const double* tot, double lambda, bool fixed_ab, unsigned map,
+                                                    double* Lm, int lane, double* x)
+{
+    return ldl_solve_t<true>(tot, lambda, fixed_ab, map, Lm, lane, *x);
+}
+
 // entry (i, k) of the system as doubles (the FP32 elimination's inputs)
-__device__ __forceinline__ double ldl_entry(const double* src, int i, int k, bool fixed_ab)
+__device__ __forceinline__ double ldl_entry(const double* tot, int i, int k, bool fixed_ab)
 {
     if (fixed_ab && (k >= 6 || i == 6 || i == 7)) return i == k ? 1.0 : 0.0;
-    return i < 8 ? src[upper_index(k, i)] : -src[kIdxG + k];
+    return i < 8 ? tot[upper_index(k, i)] : -tot[kIdxG + k];
 }
 
 // The FP32 elimination of GLT_SOLVE_FP32 (H and g are FP32 sums, relative
@@ -1300,7 +1302,7 @@ static __device__ __noinline__ double se3_coefficient(double th2, int g)
     return g == 0 ? sn / th : g == 1 ? 2.0 * sh * sh / th2 : (th - sn) / (th2 * th);
 }
 
-// exp(delta_xi) of the step S.xs as a 3x4 [R_e | t_e], entry (r, c) on lane
+// exp(delta_xi) of the step xs as a 3x4 [R_e | t_e], entry (r, c) on lane
 // 4 r + c:
 //   R_e(r, c) = d_rc + A W_rc + B (w_r w_c - d_rc th2)            (W = [w]x)
 //   t_e(r)    = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
@@ -1309,11 +1311,9 @@ static __device__ __noinline__ double se3_coefficient(double th2, int g)
 // uniform A, B, C took 17 and two compares): three give th2 (lanes 0-15),
 // w . v (lane 16) and w x v (lanes 17-19) at once, two the series of A, B, C
 // (lanes 12-14) together with w_r (.) - (.) th2 of every entry, two the entry.
-__device__ __forceinline__ double se3_exp_warp(const Solver& S, int lane)
+__device__ __forceinline__ double se3_exp_warp(const double* xs, unsigned md, unsigned me, int lane)
 {
     const unsigned full = 0xffffffffu;
-    const double* xs = S.xs;
-    const unsigned md = S.map_dot[lane], me = S.map_ent[lane];
     const double p1 = xs[md & 31], q1 = xs[(md >> 5) & 31], p2 = xs[(md >> 10) & 31], q2 = xs[(md >> 15) & 31],
                  p3 = xs[(md >> 20) & 31], q3 = xs[(md >> 25) & 31];
     const double w = xs[me & 31], wc = xs[(me >> 5) & 31], dd = xs[(me >> 10) & 31], c1 = xs[(me >> 15) & 31];
@@ -1386,38 +1386,33 @@ __device__ __forceinline__ double se3_exp_minus_i_warp(const double* xs, int lan
     return f64_of(fmaf(rot ? B : Cc, ey, fmaf(rot ? A : B, ex, base)));
 }
 
-// One LM decision after a pass whose cluster-wide sums are `tot`, of which `n`
-// valid samples; executed by all 32 lanes of one warp with uniform control
-// flow.
-// HC: the cached-Hessian form (tot holds g0 = sum w r J_ic, E and n; the
+// One LM decision after a pass, whose cluster-wide sums are in the buffer
+// solver_buffer() named; executed by all 32 lanes of one warp with uniform
+// control flow.
+// HC: the cached-Hessian form (the sums are g0 = sum w r J_ic, E and n; the
 // step is -e^-a H^-1 g0 with the level's per-reference H^-1, since the rows
 // are e^a J_ic and the normal matrix e^2a H).
 template <bool HC = false>
-__device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, int n, Solver& S,
-                                        PassParams& P, int lane, bool write_trace)
+__device__ inline void solver_step_warp(const StreamDesc& D, Solver& S, PassParams& P, int lane, bool write_trace)
 {
     const unsigned full = 0xffffffffu;
-    constexpr int NSUM = HC ? kHcAcc : kNumAcc;
-    const double E = tot[HC ? kHcE : kIdxE];
-    const double nd = tot[HC ? kHcN : kIdxN];   // exact integer count
-    // sums that are not finite (an FP32 overflow) make the pass unusable
-    bool fin = true;
-#pragma unroll
-    for (int i = lane; i <= (HC ? kHcE : kIdxE); i += 32) fin &= abs_bits(tot[i]) < kInfBits;
-    const bool sums_finite = __all_sync(full, fin);
+    constexpr int kE = HC ? kHcE : kIdxE, kN = HC ? kHcN : kIdxN;
+    const int4 w = S.w;
+    const unsigned map_ldl = S.map_ldl[lane], map_dot = S.map_dot[lane], map_ent = S.map_ent[lane],
+                   map_cmp = S.map_cmp[lane];
+    int it = w.x, status = w.y, fl = w.w;
+    const int level = fl >> kFlLevel;
+    const int wb = (fl & kFlAcc) ? 0 : 1;
+    const double* tot = S.tot[wb];
+    const int n = S.n[wb];
+    const bool sums_finite = S.bad == 0;
     const bool enough = n >= D.min_valid && n > 0 && sums_finite;
-    int status = S.status;
     if (!sums_finite) status |= GLT_TRACK_DIVERGED;
-    const int level = S.level;
-    const int phase = S.phase;
-    int it = S.it;
-    int cur = S.cur;
-    const long long step_bits = S.maxstep_bits;
     const long long stop_bits = abs_bits(level > 0 ? D.eps_step_coarse : D.eps_step);
     const long long take_bits = abs_bits(D.accept_step);
     double lambda = D.lambda0;
     bool accept = false, load_normal = false, finish = false, candidate = false;
-    if (phase == PH_START) {
+    if (!(fl & kFlCand)) {
         if (!enough) {
             if (sums_finite) status |= GLT_TRACK_TOO_FEW_POINTS;
         } else {
@@ -1427,36 +1422,32 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
         }
     } else {
         ++it;
-        accept = enough && step_bits < take_bits;
+        accept = enough && (fl & kFlSmall);
         bool flat = false;
         if (enough && !accept) {
             // c' < c  <=>  E' n < E n' (both sides non-negative: compared through
             // their bits; both products in one instruction);  flat: c' - c <= eps c
-            const double En = (lane & 1) ? S.E * nd : E * S.nd;
+            const double* old = S.tot[wb ^ 1];
+            const double En = (lane & 1) ? old[kE] * tot[kN] : tot[kE] * old[kN];
             const double e0 = __shfl_sync(full, En, 0), e1 = __shfl_sync(full, En, 1);
             accept = __double_as_longlong(e0) < __double_as_longlong(e1);
-            flat = !accept && __double_as_longlong(D.eps_cost) != 0 && (e0 - e1 <= D.eps_cost * e1);
+            if (!accept && __double_as_longlong(D.eps_cost) != 0) flat = e0 - e1 <= D.eps_cost * e1;
         }
-        lambda = accept ? S.lam_dn : S.lam_up;
+        lambda = S.lam[accept ? 0 : 1];
         load_normal = accept;
-        if (accept) cur ^= 1;
-        if (it >= D.max_iters[level] || step_bits < stop_bits || flat)
+        if (accept) fl = (fl ^ kFlCur) | kFlMoved;
+        if (it >= D.max_iters[level] || (fl & kFlStop) || flat)
             finish = true;
         else
             candidate = true;
     }
-    if (write_trace && lane == 0 && D.trace_E && S.passes < D.max_trace) {
-        D.trace_E[S.passes] = E;
-        D.trace_n[S.passes] = n;
-        D.trace_info[S.passes] = level * 4 + (phase == PH_CAND ? 1 + (accept ? 2 : 0) : 0);
-    }
     // the normal equations of the accepted state: this pass's, or the kept
     // ones after a rejection
-    const double* src = load_normal ? tot : S.N;
-    bool next_level = (phase == PH_START && !enough) || finish;
+    if (load_normal) fl ^= kFlAcc;
+    const double* src = S.tot[(fl & kFlAcc) ? 1 : 0];
     bool solved = false;
     double x = 0.0;                  // delta, entry i on lane i < 8
-    if (HC && candidate && phase == PH_START) {
+    if (HC && candidate && !(w.w & kFlCand)) {
         // -e^-a H^-1 of the level, kept for its later passes
         const double* Hi = D.Hc + 72 * level + 36;
         const double h0 = Hi[lane], h1 = Hi[lane < 4 ? 32 + lane : 0];
@@ -1478,118 +1469,99 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
         }
     } else if (candidate) {
         if (D.solve != GLT_SOLVE_FP64) solved = ldl_solve_warp_fp32(src, lambda, !D.affine, lane, x);
-        if (!solved) solved = ldl_solve_warp(src, lambda, !D.affine, S, lane, x);
+        if (!solved) {
+            solved = ldl_solve_t<false>(src, lambda, !D.affine, map_ldl, S.Lm, lane, x);
+            if (!solved) {
+                double xe = 0.0;
+                solved = ldl_solve_exact(src, lambda, !D.affine, map_ldl, S.Lm, lane, &xe);
+                x = xe;
+            }
+        }
     }
     if (candidate && !solved) {
         status |= GLT_TRACK_NOT_PD;
         finish = true;
-        next_level = true;
     }
-    if (lane < 8) S.xs[lane] = x;
-    __syncwarp();
     bool evaluated = false;          // P already holds the next state
-    bool moved = accept;
     if (solved) {
         const bool fp32 = D.solve == GLT_SOLVE_FP32;
+        if (lane < 8) S.xs[lane] = x;
+        __syncwarp();
         // ---- Tc = T exp(delta) (FP32 form: T + T (exp(delta) - I)), three FP64
         // instructions on all lanes: entry (r, c) on lane 16 + 4 r + c, the same
         // minus the identity (what the pass parameters need) on lane 4 r + c,
         // a + da and b + db on lanes 12 and 13, the two next dampings on 14, 15
-        const int q = lane & 15, er = (q >> 2) % 3, ec = q & 3;
-        const double* T = S.T[cur] + 4 * er;
-        double t0 = T[0], t1 = T[1], t2 = T[2], t3 = T[ec];
-        double e2 = 0.0, add = ec == 3 || fp32 ? t3 : 0.0;
-        if (q >= 12) {
-            t0 = t1 = 0.0;
-            t2 = lane == 12 || lane == 13 ? 1.0 : lane == 14 || lane == 15 ? lambda : 0.0;
-            e2 = lane == 12 ? S.xs[6] : lane == 13 ? S.xs[7] : lane == 14 ? D.lambda_down : D.lambda_up;
-            add = lane == 12 ? S.ab[cur][0] : lane == 13 ? S.ab[cur][1] : 0.0;
-        } else if (lane < 12 && er == ec) {
-            if (fp32)
+        const double ent = fp32 ? se3_exp_minus_i_warp(S.xs, lane) : se3_exp_warp(S.xs, map_dot, map_ent, lane);
+        const double* T = S.st[fl & kFlCur];
+        const double t0 = T[map_cmp & 31], t1 = T[(map_cmp >> 5) & 31], t2 = T[(map_cmp >> 10) & 31];
+        double add = T[(map_cmp >> 15) & 31];
+        const int q = lane & 15, ec = q & 3;
+        if (fp32 && q < 12) {
+            add = T[q];
+            if (lane == 0 || lane == 5 || lane == 10)
                 asm volatile("add.rn.f64 %0, %0, 0dBFF0000000000000;" : "+d"(add));   // never speculated
-            else
-                add = -1.0;
         }
-        const double ent = fp32 ? se3_exp_minus_i_warp(S.xs, lane) : se3_exp_warp(S, lane);
+        const double xab = S.xs[6 + (lane & 1)];
         const double x0 = __shfl_sync(full, ent, ec), x1 = __shfl_sync(full, ent, 4 + ec),
                      x2 = __shfl_sync(full, ent, 8 + ec);
-        const double v = fma(t0, x0, fma(t1, x1, fma(t2, q >= 12 ? e2 : x2, add)));
-        // (finite t0 = t1 = 0 on lanes 12-15 drop x0, x1 unless those are not finite,
-        // which lanes 0-11 report as well)
-        long long mbits = 0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) mbits = max(mbits, abs_bits(S.xs[c]));
+        const double v = fma(t0, x0, fma(t1, x1, fma(t2, q < 12 ? x2 : lane < 14 ? xab : lambda, add)));
+        // (t0 = t1 = 0 on lanes 12-15 and 28-31 drop x0, x1 unless those are not
+        // finite, which lanes 0-11 report as well)
         // a step below the level's stop threshold (and below accept_step)
         // would be taken whatever its cost and would end the level, so it
         // is taken here without a pass of its own: the next level's start
         // pass is the first evaluation of the new state; on the finest
         // level the result keeps the cost and count of the last evaluated
         // state
-        const bool take_now = mbits < stop_bits && mbits < take_bits;
-        if (!__all_sync(full, abs_bits(v) < kInfBits || lane == 14 || lane == 15)) {
+        const long long xb = abs_bits(x);
+        const bool small = __all_sync(full, xb < take_bits || lane >= 6);
+        const bool stop = __all_sync(full, xb < stop_bits || lane >= 6);
+        if (!__all_sync(full, abs_bits(v) < kInfBits || lane == 14 || lane == 15 || lane >= 28)) {
             // the solve produced a state that is not finite: keep the
             // accepted one and end the level
             status |= GLT_TRACK_DIVERGED;
             finish = true;
-            next_level = true;
         } else {
             // the next pass evaluates the new state either way
             const float vf = f32_rn(v);
             const float ea = expf(vf);
-            float* pf = lane < 12 ? (ec < 3 ? &P.Rm[3 * er + ec] : &P.t[er]) : lane == 12 ? &P.ea : &P.b;
-            double* pd = lane < 16 ? (lane < 14 ? &S.ab[cur ^ 1][lane & 1] : lane == 14 ? &S.lam_dn : &S.lam_up)
-                                   : &S.T[cur ^ 1][(lane - 16) % 12];
-            if (lane < 14) *pf = lane == 12 ? ea : vf;
+            const int nx = (fl & kFlCur) ^ 1;
+            if (lane < 14) reinterpret_cast<float*>(&P)[map_cmp >> 20] = lane == 12 ? ea : vf;
+            double* pd = lane < 14 ? &S.st[nx][lane] : lane < 16 ? &S.lam[lane - 14] : &S.st[nx][lane - 16];
             if (lane >= 12 && lane < 28) *pd = v;
             evaluated = true;
-            if (take_now) {
+            fl = (fl & ~(kFlSmall | kFlStop)) | kFlCand | (small ? kFlSmall : 0) | (stop ? kFlStop : 0);
+            if (small && stop) {
                 ++it;
                 finish = true;
-                next_level = true;
-                cur ^= 1;
-                moved = true;
-            }
-            if (lane == 0) {
-                S.maxstep_bits = mbits;
-                S.phase = PH_CAND;
+                fl = (fl ^ kFlCur) | kFlMoved;
             }
         }
     }
     // commit the pass outcome
-    if (load_normal) {
-        if (lane < NSUM) S.N[lane] = tot[lane];
-        if (lane < NSUM - 32) S.N[32 + lane] = tot[32 + lane];
+    if (write_trace && lane == 0 && D.trace_E && w.z < D.max_trace) {
+        D.trace_E[w.z] = tot[kE];
+        D.trace_n[w.z] = n;
+        D.trace_info[w.z] = level * 4 + ((w.w & kFlCand) ? 1 + (accept ? 2 : 0) : 0);
     }
-    if (lane == 0) {
-        S.passes += 1;
-        S.cur = cur;
-        if (moved) S.moved = 1;
-        S.it = it;
-        S.status = status;
-        if (load_normal) {
-            S.E = E;
-            S.nd = nd;
-            S.n = n;
-        }
-        if (finish) {
-            S.iters[level] = it;
-            S.res_E = S.E;
-            S.res_n = S.n;
-        }
+    if (finish && lane == 0) {
+        S.iters[level] = it;
+        S.res_E = src[kE];
+        S.res_n = S.n[(fl & kFlAcc) ? 1 : 0];
     }
-    __syncwarp();
-    if (next_level) {
+    if (!candidate || finish) {
+        // the next level, from the accepted state
         int l = level;
         do --l;
         while (l >= 0 && D.max_iters[l] <= 0);
-        cur = S.cur;
+        double* T = S.st[fl & kFlCur];
+        __syncwarp();
         if (l < 0) {
             // GLT_SOLVE_FP32: the poses composed from FP32 increments drift
             // from orthonormal by ~1e-9 per step: one Newton step R' = R (3 I - R^T R) / 2 =
             // R + R (I - R^T R) / 2 on the final pose (FP64; the deviation
             // becomes its square)
-            if (S.moved && D.solve == GLT_SOLVE_FP32) {
-                double* T = S.T[cur];
+            if ((fl & kFlMoved) && D.solve == GLT_SOLVE_FP32) {
                 const int i = lane / 3, j = lane % 3;
                 double dlt = lane < 9 ? (i == j ? 1.0 : 0.0) : 0.0;
                 if (lane < 9) {
@@ -1606,32 +1578,31 @@ __device__ inline void solver_step_warp(const StreamDesc& D, const double* tot, 
                 __syncwarp();
                 if (lane < 12 && c < 3) T[lane] = v;
             }
-            if (lane == 0) {
-                S.done = 1;
-                P.done = 1;
-            }
+            if (lane == 0) P.done = 1;
         } else {
-            if (lane == 0) {
-                S.level = l;
-                S.phase = PH_START;
-            }
+            fl = (fl & ((1 << kFlLevel) - 1) & ~kFlCand) | (l << kFlLevel);
             if (!evaluated)
-                make_pass_params_warp(S.T[cur], S.ab[cur][0], S.ab[cur][1], l, P, lane);
+                make_pass_params_warp(T, T[12], T[13], l, P, lane);
             else if (lane == 13) {
                 P.level = l;
                 P.scale = ldexpf(1.0f, -l);
             }
         }
     }
+    if (lane == 0) {
+        S.w = make_int4(it, status, w.z + 1, fl);
+        S.bad = 0;
+    }
     __syncwarp();
 }
 
 __device__ inline void solver_write_result(const StreamDesc& D, const Solver& S, glt_result* out)
 {
-    if (D.trace_count) *D.trace_count = S.passes;
-    for (int i = 0; i < 12; ++i) out->T[i] = S.T[S.cur][i];
-    out->a = S.ab[S.cur][0];
-    out->b = S.ab[S.cur][1];
+    const double* T = S.st[S.w.w & kFlCur];
+    if (D.trace_count) *D.trace_count = S.w.z;
+    for (int i = 0; i < 12; ++i) out->T[i] = T[i];
+    out->a = T[12];
+    out->b = T[13];
     out->cost = S.res_n > 0 ? S.res_E / (double)S.res_n : S.res_E;
     out->n_valid = S.res_n;
     int tot = 0;
@@ -1640,8 +1611,8 @@ __device__ inline void solver_write_result(const StreamDesc& D, const Solver& S,
         tot += S.iters[l];
     }
     out->iters_total = tot;
-    out->passes = S.passes;
-    out->status = S.status;
+    out->passes = S.w.z;
+    out->status = S.w.y;
 }
 
 }  // namespace glt

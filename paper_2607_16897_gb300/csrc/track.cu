@@ -124,8 +124,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
     __shared__ float red[NW][kAccPad];
     __shared__ __align__(16) float part[2][XW];
     __shared__ __align__(16) Exchange<XW> X;
-    __shared__ double tot[kAccPad];
-    __shared__ int tot_n;            // tot's sample count as an integer
     __shared__ int xfail;
 
     cg::cluster_group cluster = cg::this_cluster();
@@ -141,7 +139,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
         for (int i = tid; i < (int)(sizeof(StreamDesc) / sizeof(int)); i += THREADS) dst[i] = src[i];
     }
     if (tid < 32) tail_map_init(S, tid);
-    if (tid < kAccPad) tot[tid] = 0.0;
     __syncthreads();
     if (tid == 0) {
         solver_init(sD, init + 14 * user, S, P);
@@ -171,6 +168,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
     pc.p = -1;
     pc.level = -1;
     while (!P.done) {
+        const int wb = solver_buffer(S);   // where this pass's sums go
         float acc[NACC];
 #pragma unroll
         for (int i = 0; i < NACC; ++i) acc[i] = 0.0f;
@@ -223,8 +221,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
                     hi = s;
                 }
             }
-            tot[tid] = (double)hi + (double)lo;
-            if (tid == (HC ? kHcN : kIdxN)) tot_n = (int)hi + (int)lo;
+            solver_put_sum<HC>(S, wb, tid, (double)hi + (double)lo, (int)hi + (int)lo);
         }
         xph ^= 1u << par;
         __syncthreads();
@@ -232,14 +229,13 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
             // a peer's partial did not arrive within the limit: end the solve
             // with the accepted state
             if (tid == 0) {
-                S.status |= GLT_TRACK_TIMEOUT;
-                S.done = 1;
+                S.w.y |= GLT_TRACK_TIMEOUT;
             }
             break;
         }
         // the FP64 tail runs on one warp; CTAs of different streams that share an
         // SM use different warps so their tails spread over the SM's sub-partitions
-        if ((tid >> 5) == tail_warp) solver_step_warp<HC>(sD, tot, tot_n, S, P, tid & 31, rank == 0);
+        if ((tid >> 5) == tail_warp) solver_step_warp<HC>(sD, S, P, tid & 31, rank == 0);
         __syncthreads();
         par ^= 1;
     }
@@ -274,15 +270,12 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
     __shared__ float red[NW][kAccPad];
     __shared__ __align__(16) float part[2][XW];
     __shared__ __align__(16) Exchange<XW> X;
-    __shared__ double tot[kAccPad];
-    __shared__ int tot_n;            // tot's sample count as an integer
     __shared__ int xfail;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x;
     if (tid < 32) tail_map_init(S, tid);
-    if (tid < kAccPad) tot[tid] = 0.0;
     if (tid == 0) {
         int* z = reinterpret_cast<int*>(&sD);
         for (int i = 0; i < (int)(sizeof(StreamDesc) / sizeof(int)); ++i) z[i] = 0;
@@ -317,6 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
     int par = 0;
     unsigned xph = 0;
     for (int it = 0; it < passes; ++it) {
+        const int wb = solver_buffer(S);
         float acc[kAccPad];
 #pragma unroll
         for (int i = 0; i < kAccPad; ++i) acc[i] = 0.0f;
@@ -356,13 +350,12 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
                 for (int i = 0; i < 8; ++i)
                     if (tid == upper_index(i, i)) x = 100.0 + 10.0 * i;
             }
-            tot[tid] = x + (double)hi + (double)lo;
-            if (tid == (HC ? kHcN : kIdxN)) tot_n = 1000 + (int)hi + (int)lo;
+            solver_put_sum<HC>(S, wb, tid, x + (double)hi + (double)lo, 1000 + (int)hi + (int)lo);
         }
         xph ^= 1u << par;
         __syncthreads();
         if (xfail) break;
-        if ((tid >> 5) == (int)(blockIdx.x % NW)) solver_step_warp<HC>(sD, tot, tot_n, S, P, tid & 31, false);
+        if ((tid >> 5) == (int)(blockIdx.x % NW)) solver_step_warp<HC>(sD, S, P, tid & 31, false);
         __syncthreads();
         par ^= 1;
     }
