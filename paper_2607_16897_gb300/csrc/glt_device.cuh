@@ -12,6 +12,7 @@
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include "glt.h"
@@ -1088,7 +1089,7 @@ __device__ inline void tail_map_init(Solver& S, int lane)
     const bool poly = lane >= 12 && lane < 15, rot = ec < 3;
     const int g = lane - 12;
     const int w = poly ? kXsPoly + 6 + g : 3 + er;
-    const int pq = rot ? 3 + ec : kXs0;
+    const int pq = poly ? kXs1 : rot ? 3 + ec : kXs0;
     const int dd = poly ? kXsPoly + g : rot ? (er == ec ? kXs1 : kXs0) : er;
     const int c1 = poly ? kXsPoly + 3 + g : kXs0;
     const int W = ec == er1 ? 3 + er2 : (rot && ec == er2) ? 3 + er1 : kXs0;
@@ -1104,10 +1105,10 @@ __device__ inline void tail_map_init(Solver& S, int lane)
     if (lane == 0) {
         S.xs[kXs0] = 0.0;
         S.xs[kXs1] = 1.0;
-        double* c = S.xs + kXsPoly;      // th^2 coefficients 2, 1, 0 of A, B, C
-        c[0] = 1.0 / 120.0;
-        c[1] = 1.0 / 720.0;
-        c[2] = 1.0 / 5040.0;
+        double* c = S.xs + kXsPoly;      // th^2 coefficients 2 (negated), 1, 0 of A, B, C
+        c[0] = -1.0 / 120.0;
+        c[1] = -1.0 / 720.0;
+        c[2] = -1.0 / 5040.0;
         c[3] = -1.0 / 6.0;
         c[4] = -1.0 / 24.0;
         c[5] = -1.0 / 120.0;
@@ -1116,6 +1117,13 @@ __device__ inline void tail_map_init(Solver& S, int lane)
         c[8] = 1.0 / 6.0;
     }
     for (int i = lane; i < 2 * kAccPad; i += 32) (&S.tot[0][0])[i] = 0.0;
+}
+
+// -x where `on`, through the sign bit (a conditional negation of an FP64 operand
+// otherwise becomes two FP64 instructions and a select)
+__device__ __forceinline__ double flip_sign(double x, bool on)
+{
+    return __hiloint2double(__double2hiint(x) ^ (on ? (int)0x80000000 : 0), __double2loint(x));
 }
 
 // (H + lambda diag H) delta = -g by L D L^T, right-looking, one entry per
@@ -1144,8 +1152,8 @@ __device__ __forceinline__ bool ldl_solve_t(const double* tot, double lambda, bo
     const int iA = (map >> 12) & 15, kA = (map >> 16) & 15, iB = (map >> 20) & 15, kB = map >> 24;
     const bool dA = iA == kA, dB = iB == kB;                // diagonal entries
     double B = tot[(map >> 6) & 63], A = tot[map & 63];
-    if (iB == 8) B = -B;                                    // y = -g
-    if (iA == 8) A = -A;
+    B = flip_sign(B, iB == 8);                              // y = -g
+    A = flip_sign(A, iA == 8);
     if (fixed_ab) {
         // with (a, b) held fixed their rows and columns become the identity and
         // their right-hand side zero, so the solve gives da = db = 0
@@ -1155,6 +1163,13 @@ __device__ __forceinline__ bool ldl_solve_t(const double* tot, double lambda, bo
     B = fma(dB ? lambda : 0.0, B, B);                       // damped diagonal
     A = fma(dA ? lambda : 0.0, A, A);
     const double a0A = A, a0B = B;
+    // the smallest high word of a pivot that passes by its exponent (a damped
+    // diagonal that is not positive: none), or any
+    const int lo = (1023 - 100) << 20, hi = (1023 + 100) << 20, sl = 42 << 20;
+    const int qA = __double2hiint(a0A), qB = __double2hiint(a0B);
+    const int loA = !dA ? INT_MIN : qA > 0 ? max(lo, (qA & 0x7ff00000) - sl) : INT_MAX;
+    const int loB = !dB ? INT_MIN : qB > 0 ? max(lo, (qB & 0x7ff00000) - sl) : INT_MAX;
+    const int hiA = dA ? hi : INT_MAX, hiB = dB ? hi : INT_MAX;
     double rA = 0.0, rB = 0.0, sB = 0.0;                    // 1 / d of the lane's columns
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
@@ -1162,9 +1177,9 @@ __device__ __forceinline__ bool ldl_solve_t(const double* tot, double lambda, bo
         const double col = j < 2 ? B : A;
         const double piv = __shfl_sync(full, col, cj + j);
         const bool on = kA > j && kA < 8;
-        const double pA = __shfl_sync(full, col, on ? cj + iA : 31) * __shfl_sync(full, col, on ? cj + kA : 31);
-        double pB = 0.0;
+        double pB = 0.0;                                    // column 1 first: the next pivot's
         if (j == 0) pB = __shfl_sync(full, col, kB == 1 ? iB : 31) * __shfl_sync(full, col, kB == 1 ? 1 : 31);
+        const double pA = __shfl_sync(full, col, on ? cj + iA : 31) * __shfl_sync(full, col, on ? cj + kA : 31);
         const double r = EXACT ? rcp_d(piv) : rcp_mid(piv);
         if (j == 0) B = fma(-pB, r, B);
         A = fma(-pA, r, A);
@@ -1183,12 +1198,8 @@ __device__ __forceinline__ bool ldl_solve_t(const double* tot, double lambda, bo
     if (EXACT) {
         ok = (!dA || (A > 1e-13 * a0A && A > 0.0)) && (!dB || (B > 1e-13 * a0B && B > 0.0));
     } else {
-        // high words of the pivot and of the damped diagonal
-        const int lo = (1023 - 100) << 20, hi = (1023 + 100) << 20, sl = 42 << 20;
-        const int pA = __double2hiint(A), qA = __double2hiint(a0A);
-        const int pB = __double2hiint(B), qB = __double2hiint(a0B);
-        ok = (!dA || (pA >= lo && pA < hi && qA > 0 && pA >= (qA & 0x7ff00000) - sl)) &&
-             (!dB || (pB >= lo && pB < hi && qB > 0 && pB >= (qB & 0x7ff00000) - sl));
+        const int pA = __double2hiint(A), pB = __double2hiint(B);
+        ok = (pA >= loA) & (pA < hiA) & (pB >= loB) & (pB < hiB);
     }
     ok = __all_sync(full, ok);
     __syncwarp();
@@ -1307,28 +1318,29 @@ static __device__ __noinline__ double se3_coefficient(double th2, int g)
 //   R_e(r, c) = d_rc + A W_rc + B (w_r w_c - d_rc th2)            (W = [w]x)
 //   t_e(r)    = v_r + B (w x v)_r + C (w_r (w . v) - v_r th2)
 // with A = sin th / th, B = (1 - cos th) / th^2, C = (th - sin th) / th^3.
-// Seven FP64 instructions on the chain (the one-entry-per-lane form with
-// uniform A, B, C took 17 and two compares): three give th2 (lanes 0-15),
-// w . v (lane 16) and w x v (lanes 17-19) at once, two the series of A, B, C
-// (lanes 12-14) together with w_r (.) - (.) th2 of every entry, two the entry.
+// Eight FP64 instructions, seven of them on the chain (the one-entry-per-lane
+// form with uniform A, B, C took 17 and two compares): three give th2 (lanes
+// 0-15), w . v (lane 16) and w x v (lanes 17-19) at once; u = c1 + c2 th2 of
+// the series (lanes 12-14) is also -d_rc th2 or -v_r th2 of the entries, and
+// u Y + Z the series (Y = th2, Z = c0) and w_r (.) - (.) th2 (Y = 1, Z = w_r
+// (.)); two more give the entry.  No select stands between two FP64
+// instructions of the chain: a result costs ~50 cycles more on the way out of
+// the FP64 pipe than to its next instruction.
 __device__ __forceinline__ double se3_exp_warp(const double* xs, unsigned md, unsigned me, int lane)
 {
     const unsigned full = 0xffffffffu;
     const double p1 = xs[md & 31], q1 = xs[(md >> 5) & 31], p2 = xs[(md >> 10) & 31], q2 = xs[(md >> 15) & 31],
                  p3 = xs[(md >> 20) & 31], q3 = xs[(md >> 25) & 31];
     const double w = xs[me & 31], wc = xs[(me >> 5) & 31], dd = xs[(me >> 10) & 31], c1 = xs[(me >> 15) & 31];
-    double W = xs[(me >> 20) & 31];
-    if (me >> 25) W = -W;
+    const double W = flip_sign(xs[(me >> 20) & 31], (me >> 25) != 0);
     const bool poly = lane >= 12 && lane < 15, rot = (lane & 3) < 3;
-    double s = p1 * q1;
-    s = fma(lane >= 17 && lane < 20 ? -p2 : p2, q2, s);
-    s = fma(p3, q3, s);                                      // th2 on lanes 0-15
+    const double s = fma(p3, q3, fma(flip_sign(p2, lane >= 17 && lane < 20), q2, p1 * q1));   // th2 on lanes 0-15
+    const double u = fma(-s, dd, c1);
     const double wv = __shfl_sync(full, s, 16);
     const double cr = __shfl_sync(full, s, 17 + (lane >> 2) % 3);
-    const double pq = rot ? wc : wv;
-    const double u = fma(s, dd, c1);                         // (.) th2, or the series' first step
-    double ey = fma(poly ? u : w, poly ? s : pq, poly ? w : -u);
     const double th2 = __shfl_sync(full, s, 0);
+    const double Z = w * (rot ? wc : wv);
+    double ey = fma(u, poly ? s : 1.0, Z);
     if (!(__double_as_longlong(th2) < 0x3f1a36e2eb1c432dll)) {   // th2 >= 1e-4 (or NaN)
         const double co = se3_coefficient(th2, lane >= 12 ? lane - 12 : 0);
         if (poly) ey = co;
