@@ -135,7 +135,6 @@ namespace glt {
 
 void set_error(const std::string& msg);
 int invalid_arg_msg(const char* msg);
-cudaError_t nn_forward(glt_nn* n, const float* x, const float* mo, int B, cudaStream_t s);
 cudaError_t launch_proposal(glt_batch* b, const double* init_dev, cudaStream_t s);
 int cuda_fail(cudaError_t e, const char* what);
 
