@@ -74,89 +74,152 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 
+// Two FP32 FMAs in one instruction (fma.rn.f32x2, each half rounded as fmaf
+// does): the pipe's rate is the same, but one issue slot serves both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 __device__ __forceinline__ float2 bf2(unsigned v) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v)); }
+
+__device__ __forceinline__ f32x2 bfx2(unsigned v)
+{
+    return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
 
 // ---------------------------------------------------------------------------
 // Forward pass, convolutions: one persistent block per SM runs conv1-conv3 of
 // S samples at a time with all activations and the BF16 weights in shared
 // memory, so a sample costs its 4.8 KB of input and 5 KB of features in HBM.
 // Bound by FP32 issue: conv2 and conv3 are 5-pixel x CH-channel register tiles
-// (per tap and input channel 5 + 1 shared loads for 5 CH FMAs; the lanes of a
-// warp share their weights), conv1 8 channels of one pixel.  S = 4 fills the
+// (a window row's 11 values loaded once for its 15 uses, 3 weight loads; the
+// lanes of a warp share their weights), conv3 in two halves of its input
+// channels, conv1 8 channels of one pixel.  S = 4 fills the
 // shared memory and has the larger tiles; S = 2 has twice the blocks, and is
-// taken while those still fit one round (kFwdSmall).  Per output the sum runs
-// over the input channels and taps in order, from the bias.  Training also
+// taken while those still fit one round (kFwdSmall).  Training also
 // stores the activations (a1, a2) that the backward pass reads.  5000 samples:
 // 2.03 ms by one thread per output on global memory, 0.27 ms here; 256: 139 ->
 // 24 us (caches flushed).
 // ---------------------------------------------------------------------------
-constexpr int kFwdThreads = 256;
-constexpr int kXs = 32 * 42 + 16, kA1s = 16 * 17 * 22 + 16, kA2s = 32 * 10 * 12 + 4;   // per sample: banks staggered
+constexpr int kFwdThreads = 512;
+constexpr int kXs = 32 * 42 + 16, kA1s = 16 * 17 * 22 + 2, kA2s = 32 * 10 * 12 + 1;   // per sample (banks: conv_tiles)
 constexpr int kFwdSmall = 2;        // samples per block of the small form
 
 template <int S>
 struct FwdSmem {
     float x[S * kXs], a1[S * kA1s], a2[S * kA2s];
-    float w1[9 * 16], b1[16], b2[32], b3[64];
-    __nv_bfloat16 w2[kW2], w3[kW3];
+    alignas(16) float w1[9 * 16];
+    float b1[16], b2[32], b3[64];
+    alignas(16) __nv_bfloat16 w2[kW2], w3[kW3];
 };
+static_assert(5 * 256 <= kXs, "conv3's partial sums (5 S x 256 floats) go over x, which is no longer needed");
+static_assert(offsetof(FwdSmem<2>, w3) == offsetof(FwdSmem<2>, w2) + kW2 * sizeof(__nv_bfloat16) &&
+                  offsetof(FwdSmem<4>, w3) == offsetof(FwdSmem<4>, w2) + kW2 * sizeof(__nv_bfloat16) &&
+                  offsetof(FwdSmem<2>, w3) % 16 == 0 && offsetof(FwdSmem<4>, w3) % 16 == 0 &&
+                  offsetof(FwdSmem<4>, a2) == (size_t)4 * (kXs + kA1s) * sizeof(float),
+              "one 16-byte aligned weight copy; contiguous planes");
 
 // stride-2 3x3 conv + bias + ReLU of S samples from bordered, column-split
-// planes: thread t computes pixels pg + u PG (u < 5) x CH channels of sample s
-template <int S, int C, int W, int HO, int WO, int O, int CH, int IN, class Out>
+// planes: a thread computes 5 neighbouring pixels of a row x CH channels of one
+// sample.  Their 15 window values of a row are 11 different ones, loaded once;
+// the lanes of a warp take the rows (two halves of a row for the 10-pixel
+// ones) of two or more samples, and the sample strides place their words in
+// different banks (rows 24 or 44 words apart, halves 5, samples 1 or 2).
+// KS: the input channels in KS parts, one per thread group; part 0 adds the
+// others' sums through `red` (shared memory).
+template <int S, int C, int W, int HO, int WO, int O, int CH, int IN, int KS, class Out>
 __device__ __forceinline__ void conv_tiles(const float* __restrict__ in, const __nv_bfloat16* __restrict__ w,
-                                           const float* __restrict__ bias, Out out)
+                                           const float* __restrict__ bias, float* __restrict__ red, Out out)
 {
     constexpr int Wp = W + 2, plane = (2 * HO + (W == 20 ? 1 : 2)) * Wp, half = Wp / 2;
-    constexpr int PT = 5, PG = HO * WO / PT;
-    static_assert(S * PG * (O / CH) == kFwdThreads, "one tile per thread");
-    const int t = threadIdx.x;
+    constexpr int PT = 5, PR = WO / PT, PG = HO * PR;
+    constexpr int NT = S * PG * (O / CH);
+    static_assert(NT * KS == kFwdThreads, "one tile per thread");
+    const int t = threadIdx.x % NT, ks = threadIdx.x / NT;
     const int pg = t % PG, s = (t / PG) % S, cg = t / (PG * S);
-    int base[PT];
+    const int i = pg / PR, j = (pg % PR) * PT;
+    const float* xb = in + s * IN + 2 * i * Wp + j;          // window row 2i, split column of 2j
+    f32x2 acc[PT][CH / 2];
 #pragma unroll
-    for (int u = 0; u < PT; ++u) {
-        const int p = pg + u * PG;
-        base[u] = s * IN + 2 * (p / WO) * Wp + (p % WO);     // window row 2i, split column of 2j
-    }
-    float acc[PT][CH];
-#pragma unroll
-    for (int k = 0; k < CH; ++k) {
-        const float b = bias[cg * CH + k];
+    for (int k = 0; k < CH / 2; ++k) {
+        const f32x2 b = ks ? 0ull : pack2(bias[cg * CH + 2 * k], bias[cg * CH + 2 * k + 1]);
 #pragma unroll
         for (int u = 0; u < PT; ++u) acc[u][k] = b;
     }
 #pragma unroll 1
-    for (int c = 0; c < C; ++c) {
+    for (int c = ks * (C / KS); c < (ks + 1) * (C / KS); ++c) {
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const __nv_bfloat16* wq = w + (c * 9 + q) * O + cg * CH;
-            float wf[CH];
-            if (CH == 8) {
-                const uint4 r = *reinterpret_cast<const uint4*>(wq);
-                const float2 a = bf2(r.x), b = bf2(r.y), d = bf2(r.z), e = bf2(r.w);
-                wf[0] = a.x, wf[1] = a.y, wf[2 % CH] = b.x, wf[3 % CH] = b.y;
-                wf[4 % CH] = d.x, wf[5 % CH] = d.y, wf[6 % CH] = e.x, wf[7 % CH] = e.y;
-            } else if (CH == 4) {
-                const uint2 r = *reinterpret_cast<const uint2*>(wq);
-                const float2 a = bf2(r.x), b = bf2(r.y);
-                wf[0] = a.x, wf[1] = a.y, wf[2 % CH] = b.x, wf[3 % CH] = b.y;
-            } else {
-                const float2 a = bf2(*reinterpret_cast<const unsigned*>(wq));
-                wf[0] = a.x, wf[1] = a.y;
-            }
-            const int off = c * plane + (q / 3) * Wp + ((q % 3) & 1) * half + ((q % 3) >> 1);   // column 2j + dj
+        for (int di = 0; di < 3; ++di) {
+            const float* xr = xb + c * plane + di * Wp;
+            f32x2 ev[PT + 1], od[PT];
 #pragma unroll
-            for (int u = 0; u < PT; ++u) {
-                const float a = in[base[u] + off];
+            for (int u = 0; u <= PT; ++u) ev[u] = pack2(xr[u], xr[u]);                 // columns 2j, 2j + 2, ..
 #pragma unroll
-                for (int k = 0; k < CH; ++k) acc[u][k] = fmaf(wf[k], a, acc[u][k]);
+            for (int u = 0; u < PT; ++u) od[u] = pack2(xr[half + u], xr[half + u]);    // columns 2j + 1, ..
+#pragma unroll
+            for (int dj = 0; dj < 3; ++dj) {
+                const __nv_bfloat16* wq = w + (c * 9 + di * 3 + dj) * O + cg * CH;
+                f32x2 wf[CH / 2];
+                if constexpr (CH == 8) {
+                    const uint4 r = *reinterpret_cast<const uint4*>(wq);
+                    wf[0] = bfx2(r.x), wf[1] = bfx2(r.y), wf[2] = bfx2(r.z), wf[3] = bfx2(r.w);
+                } else if constexpr (CH == 4) {
+                    const uint2 r = *reinterpret_cast<const uint2*>(wq);
+                    wf[0] = bfx2(r.x), wf[1] = bfx2(r.y);
+                } else {
+                    wf[0] = bfx2(*reinterpret_cast<const unsigned*>(wq));
+                }
+#pragma unroll
+                for (int u = 0; u < PT; ++u) {
+                    const f32x2 a = dj == 0 ? ev[u] : dj == 1 ? od[u] : ev[u + 1];
+#pragma unroll
+                    for (int k = 0; k < CH / 2; ++k) acc[u][k] = fma2(wf[k], a, acc[u][k]);
+                }
             }
         }
+    }
+    if constexpr (KS == 2) {
+        if (ks) {
+#pragma unroll
+            for (int u = 0; u < PT; ++u)
+#pragma unroll
+                for (int k = 0; k < CH / 2; ++k) {
+                    const float2 r = unpack2(acc[u][k]);
+                    red[(u * CH + 2 * k) * NT + t] = r.x;
+                    red[(u * CH + 2 * k + 1) * NT + t] = r.y;
+                }
+        }
+        __syncthreads();
+        if (ks) return;
     }
 #pragma unroll
     for (int u = 0; u < PT; ++u)
 #pragma unroll
-        for (int k = 0; k < CH; ++k) out(s, cg * CH + k, pg + u * PG, fmaxf(acc[u][k], 0.0f));
+        for (int k = 0; k < CH / 2; ++k) {
+            float2 r = unpack2(acc[u][k]);
+            if constexpr (KS == 2) {
+                r.x += red[(u * CH + 2 * k) * NT + t];
+                r.y += red[(u * CH + 2 * k + 1) * NT + t];
+            }
+            out(s, cg * CH + 2 * k, i * WO + j + u, fmaxf(r.x, 0.0f));
+            out(s, cg * CH + 2 * k + 1, i * WO + j + u, fmaxf(r.y, 0.0f));
+        }
 }
 
 template <int S, bool TRAIN>
@@ -177,12 +240,31 @@ conv_forward(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w, c
     for (int i = tid; i < S * (kXs + kA1s + kA2s); i += kFwdThreads) M.x[i] = 0.0f;
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
+    // a group's inputs, loaded while the group before it is computed
+    constexpr int NX = (S * kIn + kFwdThreads - 1) / kFwdThreads;
+    float xv[NX];
+    auto load = [&](int b0) {
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+            const int i = tid + q * kFwdThreads;
+            xv[q] = i < S * kIn && (size_t)b0 * kIn + i < (size_t)B * kIn ? x[(size_t)b0 * kIn + i] : 0.0f;
+        }
+    };
+    load(blockIdx.x * S);
     for (int b0 = blockIdx.x * S; b0 < B; b0 += gridDim.x * S) {
-        for (int i = tid; i < S * kIn; i += kFwdThreads) {
-            const int s = i / kIn, p = i - s * kIn, r = p / 40, c = p - r * 40;
-            M.x[s * kXs + (r + 1) * 42 + split_col(c + 1, 42)] = b0 + s < B ? x[(size_t)(b0 + s) * kIn + p] : 0.0f;
+        // (conv3's partial sums went over the planes' borders)
+        for (int i = tid; i < S * 144; i += kFwdThreads) {
+            const int s = i / 144, e = i % 144;
+            const int r = e < 84 ? (e / 42) * 31 : 1 + (e - 84) / 2, c = e < 84 ? e % 42 : ((e - 84) & 1) * 41;
+            M.x[s * kXs + r * 42 + split_col(c, 42)] = 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+            const int i = tid + q * kFwdThreads, s = i / kIn, p = i - s * kIn, r = p / 40, c = p - r * 40;
+            if (i < S * kIn) M.x[s * kXs + (r + 1) * 42 + split_col(c + 1, 42)] = xv[q];
         }
         __syncthreads();
+        if (b0 + (int)gridDim.x * S < B) load(b0 + gridDim.x * S);
         for (int t = tid; t < S * 600; t += kFwdThreads) {
             const int p = t % 300, s = (t / 300) % S, og = t / (300 * S), i = p / 20, j = p % 20;
             const float* xb = M.x + s * kXs + 2 * i * 42 + j;
@@ -208,12 +290,12 @@ conv_forward(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w, c
             }
         }
         __syncthreads();
-        conv_tiles<S, 16, 20, 8, 10, 32, 2 * S, kA1s>(M.a1, M.w2, M.b2, [&](int s, int o, int p, float r) {
+        conv_tiles<S, 16, 20, 8, 10, 32, S, kA1s, 1>(M.a1, M.w2, M.b2, nullptr, [&](int s, int o, int p, float r) {
             M.a2[s * kA2s + o * 120 + (p / 10 + 1) * 12 + split_col(p % 10 + 1, 12)] = r;
             if (TRAIN && b0 + s < B) a2g[((size_t)(b0 + s) * 32 + o) * 80 + p] = r;
         });
         __syncthreads();
-        conv_tiles<S, 32, 10, 4, 5, 64, S, kA2s>(M.a2, M.w3, M.b3, [&](int s, int o, int p, float r) {
+        conv_tiles<S, 32, 10, 4, 5, 64, S, kA2s, 2>(M.a2, M.w3, M.b3, M.x, [&](int s, int o, int p, float r) {
             if (b0 + s < B) a3g[(size_t)(b0 + s) * kFlat + o * 20 + p] = r;
         });
         __syncthreads();
@@ -221,241 +303,449 @@ conv_forward(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w, c
 }
 
 // ---------------------------------------------------------------------------
-// Fully connected layers of kFcS samples per block: fc1 as 2 outputs x kFcS
-// samples per thread, the 1286 inputs split over 8 thread groups (their sums
-// added in group order), weights read coalesced from the transposed copy and
-// features broadcast from shared memory; then fc2.  In training also the loss
-// terms, dy = (y - t) / B, and fc2's input gradient dh (with fc1's ReLU mask).
-// Bound by the latency of the weights: 5000 samples 0.67 -> 0.11 ms, 256 52 ->
-// 45 us (caches flushed).
+// Fully connected layers.  fc1 tiles 4 samples x 4 outputs (or 8 x 4) per
+// thread over the transposed BF16 weights and the features in shared memory;
+// then fc2 and, in training, the loss terms, dy = (y - t) / B and fc2's input
+// gradient dh (with fc1's ReLU mask).  Two forms:
+//  * fc_forward_split, for few samples (a chip's worth of blocks matters more
+//    than reuse): a cluster of 8 blocks shares 8 samples, each block summing an
+//    eighth of the 1286 inputs; the partial sums meet through distributed
+//    shared memory in rank order and each block finishes one sample;
+//  * fc_forward_tile, for many: 32 samples per block, the inputs staged 64 at
+//    a time with two stages of asynchronous copies.
 // ---------------------------------------------------------------------------
-constexpr int kFcS = 8, kFcThreads = 512, kFcSplit = 8;
+constexpr int kFcS = 8;
 
+// fc2 of one sample from its hidden vector hs: 8 warps, one output each
 template <bool TRAIN>
-__global__ void __launch_bounds__(kFcThreads)
-fc_forward(const float* __restrict__ a3, const float* __restrict__ mo, const __nv_bfloat16* __restrict__ w,
-           const __nv_bfloat16* __restrict__ wt, int B, float* __restrict__ y, const float* __restrict__ t,
-           float* __restrict__ h, float* __restrict__ dy, float* __restrict__ dh, float* __restrict__ loss_b)
+__device__ __forceinline__ void fc2_sample(const float* __restrict__ hs, float* __restrict__ ys, const __nv_bfloat16* __restrict__ w,
+                                           int b, int B, float* __restrict__ y, const float* __restrict__ t)
 {
-    extern __shared__ __align__(16) float smf[];
-    float* f = smf;                              // [kFcS][kF + 2]
-    float* part = f + kFcS * (kF + 2);           // [kFcSplit][kFcS][kHid]
-    __shared__ float hs[kFcS][kHid], ys[kFcS][kOut];
-    const int tid = threadIdx.x, b0 = blockIdx.x * kFcS, nb = min(kFcS, B - b0);
-    for (int i = tid; i < kFcS * (kF + 2); i += kFcThreads) {
-        const int s = i / (kF + 2), k = i - s * (kF + 2);
-        float v = 0.0f;
-        if (s < nb && k < kF)
-            v = k < kFlat ? a3[(size_t)(b0 + s) * kFlat + k] : mo[(size_t)(b0 + s) * kMotion + (k - kFlat)];
-        f[i] = v;
-    }
-    __syncthreads();
-    {
-        const int o2 = tid & 63, ks = tid >> 6;
-        float acc[kFcS][2];
+    const int lane = threadIdx.x & 31, o = threadIdx.x >> 5;
+    float v = 0.0f;
 #pragma unroll
-        for (int s = 0; s < kFcS; ++s) acc[s][0] = acc[s][1] = 0.0f;
-        const __nv_bfloat16* wo = wt + kT4 + 2 * o2;
-#pragma unroll 4
-        for (int k = 2 * ks; k < kF; k += 2 * kFcSplit) {
-            const float2 w0 = bf2(*reinterpret_cast<const unsigned*>(wo + k * kHid));
-            const float2 w1 = bf2(*reinterpret_cast<const unsigned*>(wo + (k + 1) * kHid));
+    for (int i = 0; i < kHid / 32; ++i) v = fmaf(wv(w, kF2.w + o * kHid + lane + 32 * i), hs[lane + 32 * i], v);
 #pragma unroll
-            for (int s = 0; s < kFcS; ++s) {
-                const float2 v = *reinterpret_cast<const float2*>(&f[s * (kF + 2) + k]);
-                acc[s][0] = fmaf(w1.x, v.y, fmaf(w0.x, v.x, acc[s][0]));
-                acc[s][1] = fmaf(w1.y, v.y, fmaf(w0.y, v.x, acc[s][1]));
-            }
-        }
-#pragma unroll
-        for (int s = 0; s < kFcS; ++s)
-            *reinterpret_cast<float2*>(&part[(ks * kFcS + s) * kHid + 2 * o2]) = make_float2(acc[s][0], acc[s][1]);
-    }
-    __syncthreads();
-    for (int i = tid; i < kFcS * kHid; i += kFcThreads) {
-        float v = 0.0f;
-#pragma unroll
-        for (int ks = 0; ks < kFcSplit; ++ks) v += part[ks * kFcS * kHid + i];
-        v = fmaxf(v + wv(w, kF1.b + i % kHid), 0.0f);
-        hs[i / kHid][i % kHid] = v;
-        if (TRAIN && i / kHid < nb) h[(size_t)b0 * kHid + i] = v;
-    }
-    __syncthreads();
-    // fc2: warp w computes outputs 4 w .. 4 w + 3 of the 64 (sample, output) pairs
-    const int lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-    for (int q = 0; q < kFcS * kOut / (kFcThreads / 32); ++q) {
-        const int e = warp * (kFcS * kOut / (kFcThreads / 32)) + q, s = e / kOut, o = e % kOut;
-        float v = 0.0f;
-#pragma unroll
-        for (int i = 0; i < kHid / 32; ++i) v = fmaf(wv(w, kF2.w + o * kHid + lane + 32 * i), hs[s][lane + 32 * i], v);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        v += wv(w, kF2.b + o);
-        if (lane == 0) {
-            if (!TRAIN) {
-                if (s < nb) y[(size_t)(b0 + s) * kOut + o] = v;
-            } else {
-                ys[s][o] = s < nb ? v - t[(size_t)(b0 + s) * kOut + o] : 0.0f;
-            }
-        }
-    }
-    if (!TRAIN) return;
-    __syncthreads();
-    if (tid < nb) {
-        float e = 0.0f;
-#pragma unroll
-        for (int o = 0; o < kOut; ++o) e = fmaf(ys[tid][o], ys[tid][o], e);
-        loss_b[b0 + tid] = e;
-    }
-    if (tid < nb * kOut) dy[(size_t)b0 * kOut + tid] = ys[tid / kOut][tid % kOut] / (float)B;
-    for (int i = tid; i < nb * kHid; i += kFcThreads) {
-        const int s = i / kHid, k = i % kHid;
-        float v = 0.0f;
-#pragma unroll
-        for (int o = 0; o < kOut; ++o) v = fmaf(wv(w, kF2.w + o * kHid + k), ys[s][o] / (float)B, v);
-        dh[(size_t)b0 * kHid + i] = hs[s][k] > 0.0f ? v : 0.0f;
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    v += wv(w, kF2.b + o);
+    if (lane == 0) {
+        if (!TRAIN)
+            y[(size_t)b * kOut + o] = v;
+        else
+            ys[o] = v - t[(size_t)b * kOut + o];
     }
 }
 
-// d3[b,i] = (sum_o fc1.w[o,i] dh[b,o]) (a3[b,i] > 0) for the 1280 conv3
-// features: 8 samples x 2 features per thread, 256 features per block.
-constexpr int kD3Threads = 128;
-
-__global__ void __launch_bounds__(kD3Threads)
-fc1_input_grad(const float* __restrict__ dh, const __nv_bfloat16* __restrict__ w, const float* __restrict__ a3, int B,
-               float* __restrict__ d3)
+// loss term, dy and dh of one sample from its errors ys (256 threads; after a barrier)
+__device__ __forceinline__ void fc2_backward(const float* __restrict__ hs, const float* __restrict__ ys,
+                                             const __nv_bfloat16* __restrict__ w, int b, int B, float* __restrict__ h,
+                                             float* __restrict__ dy, float* __restrict__ dh, float* __restrict__ loss_b)
 {
-    __shared__ __align__(16) float d[kFcS][kHid];
-    const int tid = threadIdx.x, b0 = blockIdx.x * kFcS, nb = min(kFcS, B - b0);
-    for (int i = tid; i < kFcS * kHid; i += kD3Threads) d[i / kHid][i % kHid] = i / kHid < nb ? dh[(size_t)b0 * kHid + i] : 0.0f;
+    const int tid = threadIdx.x;
+    if (tid < kHid) {
+        float v = 0.0f;
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) v = fmaf(wv(w, kF2.w + o * kHid + tid), ys[o] / (float)B, v);
+        h[(size_t)b * kHid + tid] = hs[tid];
+        dh[(size_t)b * kHid + tid] = hs[tid] > 0.0f ? v : 0.0f;
+    } else if (tid < kHid + kOut) {
+        dy[(size_t)b * kOut + tid - kHid] = ys[tid - kHid] / (float)B;
+    } else if (tid == kHid + kOut) {
+        float e = 0.0f;
+#pragma unroll
+        for (int o = 0; o < kOut; ++o) e = fmaf(ys[o], ys[o], e);
+        loss_b[b] = e;
+    }
+}
+
+constexpr int kSpC = 8, kSpK = 162, kSpThreads = 256;       // cluster, inputs per block
+static_assert(kSpC * kSpK >= kF && kSpC == kFcS && kSpThreads / 32 == kOut, "one sample per block, one output per warp");
+
+struct SplitSmem {
+    __nv_bfloat16 w[kSpK * kHid];
+    float f[kSpK * kFcS];                        // [input][sample]
+    float part[kSpThreads / 32][kFcS][kHid];     // the warps' sums
+    float sum[kFcS][kHid];                       // the block's
+    float hs[kHid], ys[kOut];
+};
+
+static_assert(offsetof(SplitSmem, f) % 16 == 0 && offsetof(SplitSmem, part) % 16 == 0, "16-byte accesses");
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kSpThreads)
+fc_forward_split(const float* __restrict__ a3, const float* __restrict__ mo, const __nv_bfloat16* __restrict__ w,
+                 const __nv_bfloat16* __restrict__ wt, int B, float* __restrict__ y, const float* __restrict__ t,
+                 float* __restrict__ h, float* __restrict__ dy, float* __restrict__ dh, float* __restrict__ loss_b)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char raw[];
+    SplitSmem& M = *reinterpret_cast<SplitSmem*>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)cluster.block_rank(), b0 = (blockIdx.x / kSpC) * kFcS;
+    const int k0 = rank * kSpK, nk = min(kSpK, kF - k0);
+    for (int i = tid; i < nk * (kHid / 8); i += kSpThreads) cp_async16(M.w + 8 * i, wt + kT4 + k0 * kHid + 8 * i);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < (kFcS * kSpK + kSpThreads - 1) / kSpThreads; ++q) {
+        const int i = tid + q * kSpThreads, s = i / kSpK, kk = i - s * kSpK, k = k0 + kk;
+        if (i < kFcS * kSpK) {
+            float v = 0.0f;
+            if (b0 + s < B && k < kF)
+                v = k < kFlat ? a3[(size_t)(b0 + s) * kFlat + k] : mo[(size_t)(b0 + s) * kMotion + (k - kFlat)];
+            M.f[kk * kFcS + s] = v;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    const int i = 2 * (blockIdx.y * kD3Threads + tid);
-    float acc[kFcS][2];
+    // 4 outputs x 8 samples per thread, the warps on consecutive eighths of the block's inputs
+    f32x2 acc[kFcS][2];
 #pragma unroll
-    for (int s = 0; s < kFcS; ++s) acc[s][0] = acc[s][1] = 0.0f;
-#pragma unroll 2
-    for (int o = 0; o < kHid; o += 4) {
-        float2 wf[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) wf[q] = bf2(*reinterpret_cast<const unsigned*>(w + kF1.w + (o + q) * kF + i));
+    for (int s = 0; s < kFcS; ++s) acc[s][0] = acc[s][1] = 0ull;
+    constexpr int KW = (kSpK + 7) / 8;
+    const int ke = min(nk, (warp + 1) * KW);
+#pragma unroll 3
+    for (int k = warp * KW; k < ke; ++k) {
+        const uint2 r = *reinterpret_cast<const uint2*>(M.w + k * kHid + 4 * lane);
+        const f32x2 wa = bfx2(r.x), wb = bfx2(r.y);
+        const float4 fa = *reinterpret_cast<const float4*>(M.f + k * kFcS);
+        const float4 fb = *reinterpret_cast<const float4*>(M.f + k * kFcS + 4);
+        const float fs[kFcS] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
 #pragma unroll
         for (int s = 0; s < kFcS; ++s) {
-            const float4 v = *reinterpret_cast<const float4*>(&d[s][o]);
-            const float vq[4] = {v.x, v.y, v.z, v.w};
+            const f32x2 v = pack2(fs[s], fs[s]);
+            acc[s][0] = fma2(wa, v, acc[s][0]);
+            acc[s][1] = fma2(wb, v, acc[s][1]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < kFcS; ++s) {
+        const float2 a = unpack2(acc[s][0]), b = unpack2(acc[s][1]);
+        *reinterpret_cast<float4*>(&M.part[warp][s][4 * lane]) = make_float4(a.x, a.y, b.x, b.y);
+    }
+    __syncthreads();
+    for (int i = tid; i < kFcS * kHid; i += kSpThreads) {
+        float v = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kSpThreads / 32; ++q) v += (&M.part[q][0][0])[i];
+        (&M.sum[0][0])[i] = v;
+    }
+    cluster.sync();
+    const int b = b0 + rank;                     // this block's sample
+    if (tid < kHid) {
+        float p[kSpC], v = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kSpC; ++q) p[q] = cluster.map_shared_rank(&M.sum[rank][0], q)[tid];
+#pragma unroll
+        for (int q = 0; q < kSpC; ++q) v += p[q];
+        M.hs[tid] = fmaxf(v + wv(w, kF1.b + tid), 0.0f);
+    }
+    // every partial has been read: a block may leave
+    cluster.sync();
+    if (b >= B) return;
+    fc2_sample<TRAIN>(M.hs, M.ys, w, b, B, y, t);
+    if (!TRAIN) return;
+    __syncthreads();
+    fc2_backward(M.hs, M.ys, w, b, B, h, dy, dh, loss_b);
+}
+
+constexpr int kTlS = 32, kTlK = 64, kTlThreads = 256;
+
+struct TileSmem {
+    __nv_bfloat16 w[2][kTlK * kHid];
+    float f[2][kTlS * kTlK];                     // [sample][input]
+    float hs[kTlS][kHid], ys[kTlS][kOut];
+};
+
+static_assert(offsetof(TileSmem, f) % 16 == 0, "16-byte accesses");
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kTlThreads)
+fc_forward_tile(const float* __restrict__ a3, const float* __restrict__ mo, const __nv_bfloat16* __restrict__ w,
+                const __nv_bfloat16* __restrict__ wt, int B, float* __restrict__ y, const float* __restrict__ t,
+                float* __restrict__ h, float* __restrict__ dy, float* __restrict__ dh, float* __restrict__ loss_b)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    TileSmem& M = *reinterpret_cast<TileSmem*>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b0 = blockIdx.x * kTlS, nb = min(kTlS, B - b0);
+    auto stage = [&](int st, int k0) {
+#pragma unroll
+        for (int q = 0; q < kTlK * kHid / 8 / kTlThreads; ++q) {
+            const int i = tid + q * kTlThreads;
+            cp_async16(M.w[st] + 8 * i, wt + kT4 + k0 * kHid + 8 * i);
+        }
+#pragma unroll
+        for (int q = 0; q < kTlS * kTlK / 4 / kTlThreads; ++q) {
+            const int i = tid + q * kTlThreads, s = i / (kTlK / 4), c = i % (kTlK / 4);
+            cp_async16(M.f[st] + s * kTlK + 4 * c, a3 + (size_t)(b0 + min(s, nb - 1)) * kFlat + k0 + 4 * c);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    // samples 4 warp .. + 3, outputs 4 lane .. + 3
+    f32x2 acc[4][2];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) acc[s][0] = acc[s][1] = 0ull;
+    stage(0, 0);
+    for (int k0 = 0, st = 0; k0 < kFlat; k0 += kTlK, st ^= 1) {
+        if (k0 + kTlK < kFlat) {
+            stage(st ^ 1, k0 + kTlK);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
+        __syncthreads();
+        const float* f = M.f[st] + 4 * warp * kTlK;
+        const __nv_bfloat16* wk = M.w[st] + 4 * lane;
+        // the stage's own sums, then added: chains of 64 and 21 instead of 1286
+        f32x2 part[4][2];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) part[s][0] = part[s][1] = 0ull;
+#pragma unroll 4
+        for (int k = 0; k < kTlK; k += 4) {
+            f32x2 wa[4], wb[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                acc[s][0] = fmaf(wf[q].x, vq[q], acc[s][0]);
-                acc[s][1] = fmaf(wf[q].y, vq[q], acc[s][1]);
+                const uint2 r = *reinterpret_cast<const uint2*>(wk + (k + q) * kHid);
+                wa[q] = bfx2(r.x), wb[q] = bfx2(r.y);
             }
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const float4 v = *reinterpret_cast<const float4*>(f + s * kTlK + k);
+                const float vq[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const f32x2 vv = pack2(vq[q], vq[q]);
+                    part[s][0] = fma2(wa[q], vv, part[s][0]);
+                    part[s][1] = fma2(wb[q], vv, part[s][1]);
+                }
+            }
+        }
+        const f32x2 one = pack2(1.0f, 1.0f);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            acc[s][0] = fma2(part[s][0], one, acc[s][0]);
+            acc[s][1] = fma2(part[s][1], one, acc[s][1]);
+        }
+        __syncthreads();
+    }
+    // the motion inputs, then bias and ReLU
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int ls = 4 * warp + s, b = b0 + min(ls, nb - 1);
+#pragma unroll
+        for (int k = 0; k < kMotion; ++k) {
+            const uint2 r = *reinterpret_cast<const uint2*>(wt + kT4 + (kFlat + k) * kHid + 4 * lane);
+            const float m = mo[(size_t)b * kMotion + k];
+            acc[s][0] = fma2(bfx2(r.x), pack2(m, m), acc[s][0]);
+            acc[s][1] = fma2(bfx2(r.y), pack2(m, m), acc[s][1]);
+        }
+        const float2 a = unpack2(acc[s][0]), c = unpack2(acc[s][1]);
+        const float v[4] = {a.x, a.y, c.x, c.y};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) M.hs[ls][4 * lane + k] = fmaxf(v[k] + wv(w, kF1.b + 4 * lane + k), 0.0f);
+    }
+    __syncthreads();
+    for (int s = 0; s < nb; ++s) fc2_sample<TRAIN>(M.hs[s], M.ys[s], w, b0 + s, B, y, t);
+    if (!TRAIN) return;
+    __syncthreads();
+    for (int s = 0; s < nb; ++s) fc2_backward(M.hs[s], M.ys[s], w, b0 + s, B, h, dy, dh, loss_b);
+}
+
+// d3[b,i] = (sum_o fc1.w[o,i] dh[b,o]) (a3[b,i] > 0) for the 1280 conv3
+// features: one feature x 8 samples per thread, 256 features per block, whose
+// weights (contiguous in the transposed copy) are staged once; their rows are
+// padded to 272 bytes so that the lanes' 16-byte reads meet different banks.
+constexpr int kD3Threads = 256, kD3Pitch = kHid + 8;
+constexpr size_t kD3Smem = (size_t)kD3Threads * kD3Pitch * sizeof(__nv_bfloat16);
+
+__global__ void __launch_bounds__(kD3Threads)
+fc1_input_grad(const float* __restrict__ dh, const __nv_bfloat16* __restrict__ wt, const float* __restrict__ a3, int B,
+               float* __restrict__ d3)
+{
+    extern __shared__ __align__(16) __nv_bfloat16 ws[];
+    __shared__ __align__(16) float d[kHid][kFcS];
+    const int tid = threadIdx.x, b0 = blockIdx.x * kFcS, nb = min(kFcS, B - b0), i0 = blockIdx.y * kD3Threads;
+#pragma unroll
+    for (int q = 0; q < kHid / 8; ++q) {
+        const int v = tid + q * kD3Threads, r = v / (kHid / 8), c = v % (kHid / 8);
+        cp_async16(ws + r * kD3Pitch + 8 * c, wt + kT4 + (size_t)(i0 + r) * kHid + 8 * c);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < kFcS * kHid / kD3Threads; ++q) {
+        const int i = tid + q * kD3Threads, s = i / kHid, o = i % kHid;
+        d[o][s] = s < nb ? dh[(size_t)b0 * kHid + i] : 0.0f;
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    f32x2 acc[kFcS / 2];
+#pragma unroll
+    for (int s = 0; s < kFcS / 2; ++s) acc[s] = 0ull;
+#pragma unroll 4
+    for (int o = 0; o < kHid; o += 8) {
+        const uint4 r = *reinterpret_cast<const uint4*>(ws + tid * kD3Pitch + o);
+        const unsigned rw[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float wq = __uint_as_float((q & 1) ? rw[q / 2] & 0xffff0000u : rw[q / 2] << 16);
+            const f32x2 ww = pack2(wq, wq);
+            const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(&d[o + q][0]);
+            const ulonglong2 vb = *reinterpret_cast<const ulonglong2*>(&d[o + q][4]);
+            acc[0] = fma2(ww, va.x, acc[0]);
+            acc[1] = fma2(ww, va.y, acc[1]);
+            acc[2] = fma2(ww, vb.x, acc[2]);
+            acc[3] = fma2(ww, vb.y, acc[3]);
         }
     }
 #pragma unroll
     for (int s = 0; s < kFcS; ++s) {
         if (s >= nb) break;
-        const size_t at = (size_t)(b0 + s) * kFlat + i;
-        const float2 a = *reinterpret_cast<const float2*>(a3 + at);
-        *reinterpret_cast<float2*>(d3 + at) = make_float2(a.x > 0.0f ? acc[s][0] : 0.0f, a.y > 0.0f ? acc[s][1] : 0.0f);
+        const size_t at = (size_t)(b0 + s) * kFlat + i0 + tid;
+        const float2 v = unpack2(acc[s / 2]);
+        d3[at] = a3[at] > 0.0f ? ((s & 1) ? v.y : v.x) : 0.0f;
     }
 }
 
 // Weight and bias gradients of the fully connected layers: dW[o,i] = sum_b
-// dz[b,o] in[b,i], the bias as one more input of ones.  32 x 32 output tiles,
-// 4 x 4 per thread, 32 samples staged at a time; the tiles of fc1 (4 x 41)
-// come first, then fc2's (1 x 5).
-constexpr int kGwThreads = 64, kGwT = 32;
-constexpr int kGwI1 = (kF + 1 + kGwT - 1) / kGwT, kGwI2 = (kHid + 1 + kGwT - 1) / kGwT;
-constexpr int kGwBlocks = (kHid / kGwT) * kGwI1 + kGwI2;
+// dz[b,o] in[b,i], the bias as one more input of ones.  A block takes 16
+// inputs of fc1 and all 128 outputs (4 outputs x 2 inputs per thread), the
+// samples staged 64 at a time in two stages; blocks past those take fc2's.
+constexpr int kGwThreads = 256, kGwK = 64, kGwI = 16;
+constexpr int kGwB1 = (kF + 1 + kGwI - 1) / kGwI, kGwB2 = (kHid + 1 + 31) / 32, kGwBlocks = kGwB1 + kGwB2;
 
 __global__ void __launch_bounds__(kGwThreads)
 fc_weight_grad(const float* __restrict__ dh, const float* __restrict__ dy, const float* __restrict__ a3,
                const float* __restrict__ mo, const float* __restrict__ h, int B, float* __restrict__ grad)
 {
-    __shared__ __align__(16) float zs[kGwT][kGwT], is[kGwT][kGwT];
-    const bool first = blockIdx.x < (kHid / kGwT) * kGwI1;
-    const int tile = first ? blockIdx.x : blockIdx.x - (kHid / kGwT) * kGwI1;
-    const int O = first ? kHid : kOut, n = first ? kF : kHid;
-    const int o0 = first ? (tile / kGwI1) * kGwT : 0, i0 = (first ? tile % kGwI1 : tile) * kGwT;
-    const float* dz = first ? dh : dy;
-    const int tid = threadIdx.x, to = (tid / 8) * 4, ti = (tid % 8) * 4;
-    float acc[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = 0.0f;
-    for (int b0 = 0; b0 < B; b0 += kGwT) {
+    extern __shared__ __align__(16) float smw[];
+    const int tid = threadIdx.x;
+    if (blockIdx.x >= kGwB1) {
+        // fc2: 8 outputs x 32 inputs, one per thread
+        const int o = tid >> 5, i = (blockIdx.x - kGwB1) * 32 + (tid & 31);
+        float s = 0.0f;
 #pragma unroll 8
-        for (int e = tid; e < kGwT * kGwT; e += kGwThreads) {
-            const int b = b0 + e / kGwT, o = o0 + e % kGwT, i = i0 + e % kGwT;
-            float z = 0.0f, v = 0.0f;
-            if (b < B) {
-                if (o < O) z = dz[(size_t)b * O + o];
-                if (i == n)
-                    v = 1.0f;
-                else if (i < n)
-                    v = !first ? h[(size_t)b * kHid + i] : i < kFlat ? a3[(size_t)b * kFlat + i]
-                                                                   : mo[(size_t)b * kMotion + (i - kFlat)];
+        for (int b = 0; b < B; ++b)
+            s = fmaf(dy[(size_t)b * kOut + o], i < kHid ? h[(size_t)b * kHid + i] : 1.0f, s);
+        if (i <= kHid) grad[i == kHid ? kF2.b + o : kF2.w + o * kHid + i] = s;
+        return;
+    }
+    float* zs = smw;                              // [2][kGwK][kHid]
+    float* is = smw + 2 * kGwK * kHid;            // [2][kGwK][kGwI]
+    const int i0 = blockIdx.x * kGwI;
+    auto stage = [&](int st, int b0) {
+#pragma unroll
+        for (int q = 0; q < kGwK * kHid / 4 / kGwThreads; ++q) {
+            const int e = tid + q * kGwThreads, b = b0 + e / (kHid / 4);
+            float* to = zs + st * kGwK * kHid + 4 * e;
+            if (b < B)
+                cp_async16(to, dh + (size_t)b0 * kHid + 4 * e);
+            else
+                *reinterpret_cast<float4*>(to) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        const int r = tid / (kGwI / 4), c = 4 * (tid % (kGwI / 4)), b = b0 + r;
+        float* to = is + (st * kGwK + r) * kGwI + c;
+        if (b < B && i0 + c < kFlat) {
+            cp_async16(to, a3 + (size_t)b * kFlat + i0 + c);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = i0 + c + q;
+                to[q] = b >= B || i > kF ? 0.0f : i == kF ? 1.0f : mo[(size_t)b * kMotion + (i - kFlat)];
             }
-            zs[e / kGwT][e % kGwT] = z;
-            is[e / kGwT][e % kGwT] = v;
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    static_assert(kGwK * kGwI / 4 == kGwThreads && kFlat % kGwI == 0, "one input quad per thread");
+    const int to = (tid & 31) * 4, ti = (tid >> 5) * 2;
+    f32x2 acc[2][2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) acc[q][0] = acc[q][1] = 0ull;
+    stage(0, 0);
+    for (int b0 = 0, st = 0; b0 < B; b0 += kGwK, st ^= 1) {
+        if (b0 + kGwK < B) {
+            stage(st ^ 1, b0 + kGwK);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         }
         __syncthreads();
+        const float* z = zs + st * kGwK * kHid + to;
+        const float* v = is + st * kGwK * kGwI + ti;
 #pragma unroll 8
-        for (int b = 0; b < kGwT; ++b) {
-            const float4 z = *reinterpret_cast<const float4*>(&zs[b][to]);
-            const float4 v = *reinterpret_cast<const float4*>(&is[b][ti]);
-            const float zq[4] = {z.x, z.y, z.z, z.w}, vq[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int p = 0; p < 4; ++p)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(zq[p], vq[q], acc[p][q]);
+        for (int b = 0; b < kGwK; ++b) {
+            const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(z + b * kHid);
+            const float2 vv = *reinterpret_cast<const float2*>(v + b * kGwI);
+            const f32x2 va = pack2(vv.x, vv.x), vb = pack2(vv.y, vv.y);
+            acc[0][0] = fma2(zz.x, va, acc[0][0]);
+            acc[0][1] = fma2(zz.y, va, acc[0][1]);
+            acc[1][0] = fma2(zz.x, vb, acc[1][0]);
+            acc[1][1] = fma2(zz.y, vb, acc[1][1]);
         }
         __syncthreads();
     }
-    const int woff = first ? kF1.w : kF2.w, boff = first ? kF1.b : kF2.b;
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int q = 0; q < 2; ++q) {
+        const int i = i0 + ti + q;
+        if (i > kF) continue;
+        const float2 a = unpack2(acc[q][0]), b = unpack2(acc[q][1]);
+        const float v[4] = {a.x, a.y, b.x, b.y};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int o = o0 + to + p, i = i0 + ti + q;
-            if (o >= O || i > n) continue;
-            grad[i == n ? boff + o : woff + o * n + i] = acc[p][q];
-        }
+        for (int k = 0; k < 4; ++k) grad[i == kF ? kF1.b + to + k : kF1.w + (to + k) * kF + i] = v[k];
+    }
 }
 
 // ---------------------------------------------------------------------------
-// Backward pass of the convolutions: a block takes whole samples, one at a
-// time, keeps their activations and gradients in shared memory, and carries
-// its weight-gradient sums in registers over all of them; the blocks' sums go
-// to `part` and are added in block order by adam_update.  Bound by FP32 issue
-// and the shared-memory pipe.
-//  * input gradients (d2 from d3, d1 from d2): a thread owns a 2 x 2 quad of
-//    input pixels x 4 channels, whose nine (pixel, tap) pairs use each weight
-//    once (36 FMAs per 9 + 4 shared loads); conv3's 64 channels are split over
-//    two thread groups;
-//  * weight gradients: a thread owns 8 output channels x the 9 taps of one
-//    input channel (72 sums; 72 FMAs per 2 + 9 shared loads): half of the
-//    block conv3's, the other half conv2's with the positions split over four
-//    thread groups; conv1 one (channel, row) per thread.
-// Input planes have an odd stride, so the lanes of a warp (channels) read
-// different banks.  256 samples: 82 us, against 1.43 ms of one block per weight
-// and one thread per input value on global memory.
+// Backward pass of the convolutions, in two kernels (together they would hold
+// 80 gradient sums a thread beside the input gradients' registers and spill):
+//  * conv_input_grad: d2 from d3 and d1 from d2, a sample per block at a time.
+//    A thread owns a 2 x 2 quad of input pixels x 4 channels, whose nine
+//    (pixel, tap) pairs use each weight once (36 FMAs per 9 + 4 shared loads);
+//    the lanes of a warp take the quads of one channel group, so its weight
+//    loads are broadcasts; the output channels are split over warp groups;
+//  * conv_weight_grad: a block takes whole samples and carries its sums in
+//    registers over all of them.  A thread owns 8 output channels x the 9 taps
+//    of one input channel (72 sums; 72 FMAs per 2 + 9 shared loads): half of
+//    the block conv3's, the other half conv2's with the positions split over
+//    four thread groups; conv1 one (channel, row) per thread.  Input planes
+//    have an odd stride, so the lanes of a warp (channels) read different
+//    banks.  The blocks' sums go to `part`; adam_update adds them in order.
+// Both bound by FP32 issue and the shared-memory pipe.
 // ---------------------------------------------------------------------------
 constexpr int kBwThreads = 512, kBwBlocks = 148;
 constexpr int kP1 = 375, kP2 = 121;                       // plane strides of a1 (17 x 22) and a2 (10 x 12)
+constexpr int kD3P = 68, kD2P = 36;                       // position strides of d3 and d2 (banks staggered)
 constexpr int kPart = kW3 + 64 + kW2 + 32 + 144 + 16;     // one block's sums: conv3, conv2, conv1 (w, b each)
 constexpr int kPt3 = 0, kPt2 = kW3 + 64, kPt1 = kPt2 + kW2 + 32;
 
-struct BwdSmem {
+// Place e of a block's sums ([tap][output channel][input channel], then the
+// biases, of conv3 and conv2; conv1 in file order) -> parameter.
+__device__ __forceinline__ int part_param(int e)
+{
+    if (e >= kPt1) return e - kPt1;
+    const bool third = e < kPt2;
+    const int C = third ? 32 : 16, O = third ? 64 : 32, q = third ? e : e - kPt2, base = third ? kC3.w : kC2.w;
+    if (q >= 9 * O * C) return base + q;                  // bias
+    const int c = q % C, o = (q / C) % O, tap = q / (C * O);
+    return base + (o * C + c) * 9 + tap;
+}
+
+struct IgSmem {
     float w3[kW3], w2[kW2];             // [output channel][tap][input channel]
-    float x[32 * 42], a1[16 * kP1], a2[32 * kP2];
-    float d3[20 * 64];                  // [position][channel]
     float d3p[64 * 30];                 // [channel][5 x 6], zero beyond 4 x 5
-    float d2[80 * 32];                  // [position][channel]
     float d2p[32 * 99];                 // [channel][9 x 11], zero beyond 8 x 10
-    float d1[16 * 301];                 // [channel][15 x 20]
-    float tmp[160 * 16];                // the second half of conv3's input gradient
+    float tmp[16 * 160];                // the other warp groups' part of a gradient
 };
+static_assert(offsetof(IgSmem, w2) % 16 == 0, "16-byte reads");
+
+struct WgSmem {
+    float x[32 * 42], a1[16 * kP1], a2[32 * kP2];
+    float d3[20 * kD3P];                // [position][channel]
+    float d2[80 * kD2P];                // [position][channel]
+    float d1[16 * 301];                 // [channel][15 x 20]
+    float red[4 * kW2], tmp[128];
+};
+static_assert(offsetof(WgSmem, d3) % 16 == 0 && offsetof(WgSmem, d2) % 16 == 0, "16-byte reads");
 
 // the quad (i0, j0) of an input gradient: acc[px][channel] over output
 // channels [o0, o1); dp: padded gradient planes of stride DP and row DW;
@@ -464,23 +754,21 @@ template <int C, int DP, int DW>
 __device__ __forceinline__ void quad_grad(const float* __restrict__ dp, const float* __restrict__ w, int o0, int o1,
                                           int i0, int j0, int c0, float (&acc)[4][4])
 {
+    f32x2 s[4][2];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[p][k] = 0.0f;
+    for (int p = 0; p < 4; ++p) s[p][0] = s[p][1] = 0ull;
 #pragma unroll 2
     for (int o = o0; o < o1; ++o) {
         const float* d = dp + o * DP + i0 * DW + j0;
-        const float d00 = d[0], d01 = d[1], d10 = d[DW], d11 = d[DW + 1];
+        const f32x2 d00 = pack2(d[0], d[0]), d01 = pack2(d[1], d[1]), d10 = pack2(d[DW], d[DW]),
+                    d11 = pack2(d[DW + 1], d[DW + 1]);
         const float* wo = w + o * 9 * C + c0;
         // input row 2 i0 takes tap row 1 of output row i0; row 2 i0 + 1 tap row
         // 2 of i0 and tap row 0 of i0 + 1; columns alike
-        auto tap = [&](int q, int px, float v) {
-            const float4 r = *reinterpret_cast<const float4*>(wo + q * C);
-            acc[px][0] = fmaf(r.x, v, acc[px][0]);
-            acc[px][1] = fmaf(r.y, v, acc[px][1]);
-            acc[px][2] = fmaf(r.z, v, acc[px][2]);
-            acc[px][3] = fmaf(r.w, v, acc[px][3]);
+        auto tap = [&](int q, int px, f32x2 v) {
+            const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(wo + q * C);
+            s[px][0] = fma2(r.x, v, s[px][0]);
+            s[px][1] = fma2(r.y, v, s[px][1]);
         };
         tap(4, 0, d00);
         tap(3, 1, d01);
@@ -492,122 +780,178 @@ __device__ __forceinline__ void quad_grad(const float* __restrict__ dp, const fl
         tap(6, 3, d01);
         tap(8, 3, d00);
     }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const float2 a = unpack2(s[p][0]), b = unpack2(s[p][1]);
+        acc[p][0] = a.x, acc[p][1] = a.y, acc[p][2] = b.x, acc[p][3] = b.y;
+    }
 }
 
 // weight-gradient sums of 8 output channels x 9 taps of one input plane over
 // positions [p0, p1)
-template <int WO, int Wp, int O>
+template <int WO, int Wp, int DP>
 __device__ __forceinline__ void tap_grad(const float* __restrict__ dpos, const float* __restrict__ plane, int p0, int p1,
-                                         int og, float (&acc)[8][9], float (&bias)[8])
+                                         int og, f32x2 (&acc)[4][9], f32x2 (&bias)[4])
 {
+    const f32x2 one = pack2(1.0f, 1.0f);
     for (int p = p0; p < p1; ++p) {
-        const float4 da = *reinterpret_cast<const float4*>(dpos + p * O + og * 8);
-        const float4 db = *reinterpret_cast<const float4*>(dpos + p * O + og * 8 + 4);
-        const float dv[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+        const ulonglong2 da = *reinterpret_cast<const ulonglong2*>(dpos + p * DP + og * 8);
+        const ulonglong2 db = *reinterpret_cast<const ulonglong2*>(dpos + p * DP + og * 8 + 4);
+        const f32x2 dv[4] = {da.x, da.y, db.x, db.y};
         const float* in = plane + 2 * (p / WO) * Wp + (p % WO);
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
             const float v = in[(q / 3) * Wp + ((q % 3) & 1) * (Wp / 2) + ((q % 3) >> 1)];
+            const f32x2 vv = pack2(v, v);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k][q] = fmaf(dv[k], v, acc[k][q]);
+            for (int k = 0; k < 4; ++k) acc[k][q] = fma2(dv[k], vv, acc[k][q]);
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) bias[k] += dv[k];
+        for (int k = 0; k < 4; ++k) bias[k] = fma2(dv[k], one, bias[k]);
     }
 }
 
 __global__ void __launch_bounds__(kBwThreads, 1)
-conv_backward(const float* __restrict__ x, const float* __restrict__ a1, const float* __restrict__ a2,
-              const float* __restrict__ d3, const __nv_bfloat16* __restrict__ wt, int B, float* __restrict__ part)
+conv_input_grad(const float* __restrict__ d3, const float* __restrict__ a1, const float* __restrict__ a2,
+                const __nv_bfloat16* __restrict__ wt, int B, float* __restrict__ d2, float* __restrict__ d1)
 {
     extern __shared__ __align__(16) unsigned char raw[];
-    BwdSmem& M = *reinterpret_cast<BwdSmem*>(raw);
-    const int tid = threadIdx.x;
-    for (int i = tid; i < kW3; i += kBwThreads) M.w3[i] = wv(wt, kB3 + i);
-    for (int i = tid; i < kW2; i += kBwThreads) M.w2[i] = wv(wt, kB2 + i);
-    for (int i = tid; i < (int)((sizeof(BwdSmem) - offsetof(BwdSmem, x)) / sizeof(float)); i += kBwThreads) M.x[i] = 0.0f;
-    // weight-gradient roles: threads 0-255 conv3 (8 output groups x 32 input
-    // channels), the others conv2 (4 position groups x 4 x 16)
-    const bool third = tid < 256;
-    const int u = tid & 255, gc = third ? u & 31 : u & 15, gg = third ? u >> 5 : (u >> 4) & 3, gs = u >> 6;
-    const int o1 = tid & 15, r1 = tid >> 4;               // conv1: channel, row (r1 < 15)
-    float wg[8][9], bg[8], w1g[9], b1g = 0.0f;
+    IgSmem& M = *reinterpret_cast<IgSmem*>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // BF16 weights, 8 at a time: conv2's part, then conv3's
+    static_assert(kB3 == kB2 + kW2, "one contiguous copy");
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        bg[k] = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) wg[k][q] = 0.0f;
+    for (int q = 0; q < ((kW2 + kW3) / 8 + kBwThreads - 1) / kBwThreads; ++q) {
+        const int e = 8 * (tid + q * kBwThreads);
+        if (e < kW2 + kW3) {
+            const uint4 r = *reinterpret_cast<const uint4*>(wt + kB2 + e);
+            float* to = e < kW2 ? M.w2 + e : M.w3 + e - kW2;
+            const float2 a = bf2(r.x), b = bf2(r.y), c = bf2(r.z), d = bf2(r.w);
+            *reinterpret_cast<float4*>(to) = make_float4(a.x, a.y, b.x, b.y);
+            *reinterpret_cast<float4*>(to + 4) = make_float4(c.x, c.y, d.x, d.y);
+        }
     }
-#pragma unroll
-    for (int q = 0; q < 9; ++q) w1g[q] = 0.0f;
+    for (int i = tid; i < 64 * 30 + 32 * 99; i += kBwThreads) M.d3p[i] = 0.0f;
     __syncthreads();
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
-        for (int i = tid; i < kIn; i += kBwThreads) M.x[(i / 40 + 1) * 42 + split_col(i % 40 + 1, 42)] = x[(size_t)b * kIn + i];
-        for (int i = tid; i < 4800; i += kBwThreads) {
-            const int c = i / 300, p = i % 300;
-            M.a1[c * kP1 + (p / 20 + 1) * 22 + split_col(p % 20 + 1, 22)] = a1[(size_t)b * 4800 + i];
-        }
-        for (int i = tid; i < 2560; i += kBwThreads) {
-            const int c = i / 80, p = i % 80;
-            M.a2[c * kP2 + (p / 10 + 1) * 12 + split_col(p % 10 + 1, 12)] = a2[(size_t)b * 2560 + i];
-        }
-        for (int i = tid; i < kFlat; i += kBwThreads) {
-            const int o = i / 20, p = i % 20;
-            const float v = d3[(size_t)b * kFlat + i];
-            M.d3[p * 64 + o] = v;
-            M.d3p[o * 30 + (p / 5) * 6 + p % 5] = v;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int i = tid + q * kBwThreads, o = i / 20, p = i % 20;
+            if (i < kFlat) M.d3p[o * 30 + (p / 5) * 6 + p % 5] = d3[(size_t)b * kFlat + i];
         }
         __syncthreads();
-        // d2, in two halves of conv3's channels
+        // d2: warp = half of conv3's channels x channel group of 4, lanes 0-19 the quads
         {
-            const int half = tid / 160, e = tid % 160, quad = e % 20, cg = e / 20;
-            const int i0 = quad / 5, j0 = quad % 5;
-            float acc[4][4];
-            if (half < 2) quad_grad<32, 30, 6>(M.d3p, M.w3, half * 32, half * 32 + 32, i0, j0, cg * 4, acc);
-            if (half == 1) {
+            const int half = warp >> 3, cg = warp & 7, e = cg * 20 + lane;
+            const bool on = lane < 20;
+            const int i0 = on ? lane / 5 : 0, j0 = on ? lane % 5 : 0;
+            float acc[4][4], m[4][4];
+            if (on && half == 0) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        m[p][k] = a2[((size_t)b * 32 + cg * 4 + k) * 80 + (2 * i0 + (p >> 1)) * 10 + 2 * j0 + (p & 1)];
+            }
+            quad_grad<32, 30, 6>(M.d3p, M.w3, half * 32, half * 32 + 32, i0, j0, cg * 4, acc);
+            if (on && half == 1) {
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) M.tmp[(p * 4 + k) * 160 + e] = acc[p][k];
             }
             __syncthreads();
-            if (half == 0) {
+            if (on && half == 0) {
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const int yy = 2 * i0 + (p >> 1), xx = 2 * j0 + (p & 1);
+                    float v[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int c = cg * 4 + k;
-                        const bool on = M.a2[c * kP2 + (yy + 1) * 12 + split_col(xx + 1, 12)] > 0.0f;
-                        const float v = on ? acc[p][k] + M.tmp[(p * 4 + k) * 160 + e] : 0.0f;
-                        M.d2[(yy * 10 + xx) * 32 + c] = v;
-                        M.d2p[c * 99 + yy * 11 + xx] = v;
+                        v[k] = m[p][k] > 0.0f ? acc[p][k] + M.tmp[(p * 4 + k) * 160 + e] : 0.0f;
+                        M.d2p[(cg * 4 + k) * 99 + yy * 11 + xx] = v[k];
+                    }
+                    *reinterpret_cast<float4*>(d2 + ((size_t)b * 80 + yy * 10 + xx) * 32 + cg * 4) =
+                        make_float4(v[0], v[1], v[2], v[3]);
+                }
+            }
+            __syncthreads();
+        }
+        // d1: warps 0-11, 3 per channel group of 4
+        {
+            const int cg = warp / 3, quad = (warp % 3) * 32 + lane;
+            if (cg < 4 && quad < 80) {
+                const int i0 = quad / 10, j0 = quad % 10;
+                float acc[4][4];
+                quad_grad<16, 99, 11>(M.d2p, M.w2, 0, 32, i0, j0, cg * 4, acc);
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const int yy = 2 * i0 + (p >> 1), xx = 2 * j0 + (p & 1);
+                    if (yy >= 15) continue;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const size_t at = ((size_t)b * 16 + cg * 4 + k) * 300 + yy * 20 + xx;
+                        d1[at] = a1[at] > 0.0f ? acc[p][k] : 0.0f;
                     }
                 }
             }
         }
         __syncthreads();
-        if (third)
-            tap_grad<5, 12, 64>(M.d3, M.a2 + gc * kP2, 0, 20, gg, wg, bg);
-        else
-            tap_grad<10, 22, 32>(M.d2, M.a1 + gc * kP1, gs * 20, gs * 20 + 20, gg, wg, bg);
-        if (tid < 320) {
-            const int quad = tid % 80, cg = tid / 80, i0 = quad / 10, j0 = quad % 10;
-            float acc[4][4];
-            quad_grad<16, 99, 11>(M.d2p, M.w2, 0, 32, i0, j0, cg * 4, acc);
+    }
+}
+
+__global__ void __launch_bounds__(kBwThreads, 1)
+conv_weight_grad(const float* __restrict__ x, const float* __restrict__ a1, const float* __restrict__ a2,
+                 const float* __restrict__ d3, const float* __restrict__ d2, const float* __restrict__ d1, int B,
+                 float* __restrict__ part)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    WgSmem& M = *reinterpret_cast<WgSmem*>(raw);
+    const int tid = threadIdx.x;
+    for (int i = tid; i < 32 * 42 + 16 * kP1 + 32 * kP2; i += kBwThreads) M.x[i] = 0.0f;
+    // weight-gradient roles: threads 0-255 conv3 (8 output groups x 32 input
+    // channels), the others conv2 (4 position groups x 4 x 16)
+    const bool third = tid < 256;
+    const int u = tid & 255, gc = third ? u & 31 : u & 15, gg = third ? u >> 5 : (u >> 4) & 3, gs = u >> 6;
+    const int o1 = tid & 15, r1 = tid >> 4;               // conv1: channel, row (r1 < 15)
+    f32x2 wg[4][9], bg[4];
+    float w1g[9], b1g = 0.0f;
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const int yy = 2 * i0 + (p >> 1), xx = 2 * j0 + (p & 1);
-                if (yy >= 15) continue;
+    for (int k = 0; k < 4; ++k) {
+        bg[k] = 0ull;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int c = cg * 4 + k;
-                    const bool on = M.a1[c * kP1 + (yy + 1) * 22 + split_col(xx + 1, 22)] > 0.0f;
-                    M.d1[c * 301 + yy * 20 + xx] = on ? acc[p][k] : 0.0f;
-                }
+        for (int q = 0; q < 9; ++q) wg[k][q] = 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) w1g[q] = 0.0f;
+    __syncthreads();
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+#pragma unroll 5
+        for (int q = 0; q < 10; ++q) {
+            const int i = tid + q * kBwThreads;
+            if (i < 4800) {
+                const float va = a1[(size_t)b * 4800 + i], vd = d1[(size_t)b * 4800 + i];
+                const int c = i / 300, p = i % 300;
+                M.a1[c * kP1 + (p / 20 + 1) * 22 + split_col(p % 20 + 1, 22)] = va;
+                M.d1[c * 301 + p] = vd;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            const int i = tid + q * kBwThreads, c = i / 80, p = i % 80;
+            const float va = a2[(size_t)b * 2560 + i], vd = d2[(size_t)b * 2560 + i];
+            M.a2[c * kP2 + (p / 10 + 1) * 12 + split_col(p % 10 + 1, 12)] = va;
+            M.d2[(i >> 5) * kD2P + (i & 31)] = vd;
+            if (q < 3) {
+                if (i < kIn) M.x[(i / 40 + 1) * 42 + split_col(i % 40 + 1, 42)] = x[(size_t)b * kIn + i];
+                if (i < kFlat) M.d3[(i % 20) * kD3P + i / 20] = d3[(size_t)b * kFlat + i];
             }
         }
         __syncthreads();
+        if (third)
+            tap_grad<5, 12, kD3P>(M.d3, M.a2 + gc * kP2, 0, 20, gg, wg, bg);
+        else
+            tap_grad<10, 22, kD2P>(M.d2, M.a1 + gc * kP1, gs * 20, gs * 20 + 20, gg, wg, bg);
         if (r1 < 15) {
             const float* d = M.d1 + o1 * 301 + r1 * 20;
             const float* in = M.x + 2 * r1 * 42;
@@ -624,20 +968,22 @@ conv_backward(const float* __restrict__ x, const float* __restrict__ a1, const f
     // this block's sums: conv2's position groups and conv1's rows meet in
     // shared memory, in order
     float* out = part + (size_t)blockIdx.x * kPart;
-    float* red = M.w3;                                   // 4 x (kW2 + 32), then 15 x 160
-    if (third) {
+    float* red = M.red;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < 4; ++k) {
+        const int o = gg * 8 + 2 * k;
 #pragma unroll
-            for (int q = 0; q < 9; ++q) out[kPt3 + ((gg * 8 + k) * 32 + gc) * 9 + q] = wg[k][q];
-            if (gc == 0) out[kPt3 + kW3 + gg * 8 + k] = bg[k];
+        for (int q = 0; q < 9; ++q) {
+            const float2 v = unpack2(wg[k][q]);
+            float* to = third ? out + kPt3 + (q * 64 + o) * 32 + gc : red + gs * kW2 + (q * 32 + o) * 16 + gc;
+            to[0] = v.x;
+            to[third ? 32 : 16] = v.y;
         }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-#pragma unroll
-            for (int q = 0; q < 9; ++q) red[gs * kW2 + ((gg * 8 + k) * 16 + gc) * 9 + q] = wg[k][q];
-            if (gc == 0) M.tmp[gs * 32 + gg * 8 + k] = bg[k];
+        if (gc == 0) {
+            const float2 v = unpack2(bg[k]);
+            float* to = third ? out + kPt3 + kW3 + o : M.tmp + gs * 32 + o;
+            to[0] = v.x;
+            to[1] = v.y;
         }
     }
     if (r1 < 15) {
@@ -676,18 +1022,16 @@ adam_update(float* __restrict__ w, __nv_bfloat16* __restrict__ wbf, __nv_bfloat1
     float gi = 0.0f;
     if (blockIdx.x < kAdConv) {
         __shared__ float q4[4][64];
-        const int e = threadIdx.x & 63, q = threadIdx.x >> 6, c = blockIdx.x * 64 + e;
-        // parameter c in file order (conv1.w, conv1.b, conv2.w, ...) -> its place in a block's sums
-        const int at = c < 160 ? kPt1 + c : c < kC3.w ? kPt2 + c - kC2.w : kPt3 + c - kC3.w;
+        const int e = threadIdx.x & 63, q = threadIdx.x >> 6, at = blockIdx.x * 64 + e;
         float s = 0.0f;
-        if (c < kAdConvN) {
+        if (at < kAdConvN) {
 #pragma unroll 8
             for (int k = q; k < nparts; k += 4) s += part[(size_t)k * kPart + at];
         }
         q4[q][e] = s;
         __syncthreads();
-        if (q == 0 && c < kAdConvN) {
-            i = c;
+        if (q == 0 && at < kAdConvN) {
+            i = part_param(at);
             gi = ((q4[0][e] + q4[1][e]) + q4[2][e]) + q4[3][e];
             g[i] = gi;
         }
@@ -748,7 +1092,7 @@ struct glt_nn {
     // activations and gradients of up to max_batch samples, the backward
     // blocks' weight-gradient sums, loss terms
     float *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *h = nullptr, *y = nullptr, *dy = nullptr, *dh = nullptr,
-          *d3 = nullptr, *part = nullptr, *loss_b = nullptr;
+          *d3 = nullptr, *d2 = nullptr, *d1 = nullptr, *part = nullptr, *loss_b = nullptr;
     float* loss = nullptr;
 };
 
@@ -757,7 +1101,9 @@ using namespace glt::nn;
 
 namespace {
 
-constexpr size_t kFcSmem = (size_t)(kFcS * (kF + 2) + kFcSplit * kFcS * kHid) * sizeof(float);
+constexpr size_t kGwSmem = (size_t)2 * kGwK * (kHid + kGwI) * sizeof(float);
+// fc_forward_split up to this many samples, fc_forward_tile beyond
+constexpr int kFcSmall = 2048;
 
 int nn_alloc(glt_nn* n)
 {
@@ -783,6 +1129,8 @@ int nn_alloc(glt_nn* n)
     if (e == cudaSuccess) e = al(&n->dy, (size_t)B * kOut);
     if (e == cudaSuccess) e = al(&n->dh, (size_t)B * kHid);
     if (e == cudaSuccess) e = al(&n->d3, (size_t)B * kFlat);
+    if (e == cudaSuccess) e = al(&n->d2, (size_t)B * 32 * 8 * 10);
+    if (e == cudaSuccess) e = al(&n->d1, (size_t)B * 16 * 15 * 20);
     if (e == cudaSuccess) e = al(&n->part, (size_t)std::min(B, kBwBlocks) * kPart);
     if (e == cudaSuccess) e = al(&n->loss_b, (size_t)B);
     if (e == cudaSuccess) e = al(&n->loss, 1);
@@ -795,16 +1143,21 @@ int nn_alloc(glt_nn* n)
     if (e == cudaSuccess) e = smem(conv_forward<2, true>, sizeof(FwdSmem<2>));
     if (e == cudaSuccess) e = smem(conv_forward<4, false>, sizeof(FwdSmem<4>));
     if (e == cudaSuccess) e = smem(conv_forward<4, true>, sizeof(FwdSmem<4>));
-    if (e == cudaSuccess) e = smem(fc_forward<false>, kFcSmem);
-    if (e == cudaSuccess) e = smem(fc_forward<true>, kFcSmem);
-    if (e == cudaSuccess) e = smem(conv_backward, sizeof(BwdSmem));
+    if (e == cudaSuccess) e = smem(fc_forward_split<false>, sizeof(SplitSmem));
+    if (e == cudaSuccess) e = smem(fc_forward_split<true>, sizeof(SplitSmem));
+    if (e == cudaSuccess) e = smem(fc_forward_tile<false>, sizeof(TileSmem));
+    if (e == cudaSuccess) e = smem(fc_forward_tile<true>, sizeof(TileSmem));
+    if (e == cudaSuccess) e = smem(fc1_input_grad, kD3Smem);
+    if (e == cudaSuccess) e = smem(fc_weight_grad, kGwSmem);
+    if (e == cudaSuccess) e = smem(conv_input_grad, sizeof(IgSmem));
+    if (e == cudaSuccess) e = smem(conv_weight_grad, sizeof(WgSmem));
     return e == cudaSuccess ? GLT_OK : cuda_fail(e, "proposal network allocation");
 }
 
 void nn_free(glt_nn* n)
 {
     if (!n) return;
-    for (float* p : {n->w, n->g, n->m, n->v, n->a1, n->a2, n->a3, n->h, n->y, n->dy, n->dh, n->d3, n->part, n->loss_b,
+    for (float* p : {n->w, n->g, n->m, n->v, n->a1, n->a2, n->a3, n->h, n->y, n->dy, n->dh, n->d3, n->d2, n->d1, n->part, n->loss_b,
                      n->loss})
         cudaFree(p);
     cudaFree(n->wbf);
@@ -825,23 +1178,47 @@ void launch_conv_forward(const glt_nn* n, const float* x, int B, cudaStream_t s)
             x, n->wbf, n->wt, B, n->a1, n->a2, n->a3);
 }
 
+// fc1 and fc2 of B samples; TRAIN: up to dh
+template <bool TRAIN>
+cudaError_t launch_fc_forward(const glt_nn* n, const float* mo, int B, float* y, const float* t, cudaStream_t s)
+{
+    if (B > kFcSmall) {
+        fc_forward_tile<TRAIN><<<grid_for(B, kTlS), kTlThreads, sizeof(TileSmem), s>>>(n->a3, mo, n->wbf, n->wt, B, y, t, n->h,
+                                                                                      n->dy, n->dh, n->loss_b);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(grid_for(B, kFcS) * kSpC), 1, 1);
+    cfg.blockDim = dim3(kSpThreads, 1, 1);
+    cfg.dynamicSmemBytes = sizeof(SplitSmem);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kSpC;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fc_forward_split<TRAIN>, (const float*)n->a3, mo, (const __nv_bfloat16*)n->wbf,
+                              (const __nv_bfloat16*)n->wt, B, y, t, n->h, n->dy, n->dh, n->loss_b);
+}
+
 cudaError_t nn_forward(const glt_nn* n, const float* x, const float* mo, int B, float* y, cudaStream_t s)
 {
     launch_conv_forward<false>(n, x, B, s);
-    fc_forward<false><<<grid_for(B, kFcS), kFcThreads, kFcSmem, s>>>(n->a3, mo, n->wbf, n->wt, B, y, nullptr, nullptr,
-                                                                     nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    return launch_fc_forward<false>(n, mo, B, y, nullptr, s);
 }
 
 // forward and backward: the gradient sums up to adam_update, which completes them
 cudaError_t nn_backward(const glt_nn* n, const float* x, const float* mo, const float* t, int B, cudaStream_t s)
 {
     launch_conv_forward<true>(n, x, B, s);
-    fc_forward<true><<<grid_for(B, kFcS), kFcThreads, kFcSmem, s>>>(n->a3, mo, n->wbf, n->wt, B, n->y, t, n->h, n->dy,
-                                                                    n->dh, n->loss_b);
-    fc1_input_grad<<<dim3(grid_for(B, kFcS), kFlat / (2 * kD3Threads)), kD3Threads, 0, s>>>(n->dh, n->wbf, n->a3, B, n->d3);
-    fc_weight_grad<<<kGwBlocks, kGwThreads, 0, s>>>(n->dh, n->dy, n->a3, mo, n->h, B, n->g);
-    conv_backward<<<std::min(B, kBwBlocks), kBwThreads, sizeof(BwdSmem), s>>>(x, n->a1, n->a2, n->d3, n->wt, B, n->part);
+    const cudaError_t e = launch_fc_forward<true>(n, mo, B, n->y, t, s);
+    if (e != cudaSuccess) return e;
+    fc1_input_grad<<<dim3(grid_for(B, kFcS), kFlat / kD3Threads), kD3Threads, kD3Smem, s>>>(n->dh, n->wt, n->a3, B, n->d3);
+    fc_weight_grad<<<kGwBlocks, kGwThreads, kGwSmem, s>>>(n->dh, n->dy, n->a3, mo, n->h, B, n->g);
+    conv_input_grad<<<std::min(B, kBwBlocks), kBwThreads, sizeof(IgSmem), s>>>(n->d3, n->a1, n->a2, n->wt, B, n->d2, n->d1);
+    conv_weight_grad<<<std::min(B, kBwBlocks), kBwThreads, sizeof(WgSmem), s>>>(x, n->a1, n->a2, n->d3, n->d2, n->d1, B, n->part);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
 """The proposal network's kernels at the batch sizes where their tiling changes:
-one sample, ragged groups of the 8-sample fully connected blocks, the last size
-of the 2-sample convolution blocks and the first of the 4-sample ones, more
+one sample, ragged 8-sample clusters of the fully connected layers, the last size
+of the 2-sample convolution blocks and the first of the 4-sample ones, the last
+size of the clusters and the first of the 32-sample tiles, more
 samples than blocks of the backward pass.  Against the FP64 oracle network with
 the same BF16-rounded weights; tolerances as in test_gpu_nn.py (FP32 sums)."""
 import numpy as np
@@ -23,7 +24,7 @@ def onn():
     return nn
 
 
-@pytest.mark.parametrize("B", [2, 9, 303, 304, 305, 611])
+@pytest.mark.parametrize("B", [2, 9, 303, 304, 305, 2048, 2049])
 def test_forward_sizes(glt, onn, B):
     import torch
     w = make_params(onn, 3)
@@ -39,7 +40,7 @@ def test_forward_sizes(glt, onn, B):
     net.close()
 
 
-@pytest.mark.parametrize("B", [1, 3, 31, 33, 149, 310])
+@pytest.mark.parametrize("B", [1, 3, 63, 65, 149, 310])
 def test_gradient_sizes(glt, onn, B):
     w = make_params(onn, 5)
     x, m, t = make_inputs(B, 200 + B)
