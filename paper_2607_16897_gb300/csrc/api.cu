@@ -164,6 +164,8 @@ static void free_tracker(glt_tracker* t)
     cudaFree(t->I0);
     cudaFree(t->G0);
     cudaFree(t->Hc);
+    cudaFree(t->Hpart);
+    cudaFree(t->Hcount);
     cudaFree(t->desc_dev);
     cudaFree(t->desc_ptr_dev);
     cudaFree(t->user_dev);
@@ -368,9 +370,16 @@ int glt_create(const glt_config* cfg, glt_tracker** out)
     ALLOC(dalloc(&t->pt, (size_t)t->Npad));
     ALLOC(dalloc(&t->dz, (size_t)t->Npad));
     t->K = cfg->pattern == 0 ? 8 : cfg->pattern * cfg->pattern;
-    ALLOC(dalloc(&t->I0, (size_t)t->L * t->Npad * t->K));
-    if (cfg->jacobian == GLT_IC) ALLOC(dalloc(&t->G0, (size_t)t->L * t->Npad * t->K));
-    if (cfg->hessian == GLT_HESSIAN_CACHED) ALLOC(dalloc(&t->Hc, (size_t)t->L * 72));
+    const int tg = cfg->hessian == GLT_HESSIAN_CACHED ? hc_groups(cfg->pattern) : 1;
+    const size_t tab = table_size(t->L, t->Npad, cfg->pattern, tg);
+    ALLOC(dalloc(&t->I0, tab));
+    if (cfg->jacobian == GLT_IC) ALLOC(dalloc(&t->G0, tab));
+    if (cfg->hessian == GLT_HESSIAN_CACHED) {
+        ALLOC(dalloc(&t->Hc, (size_t)t->L * 72));
+        ALLOC(dalloc(&t->Hpart, (size_t)t->L * kHessSums * t->Npad));
+        ALLOC(dalloc(&t->Hcount, (size_t)t->L));
+        ALLOC(cudaMemset(t->Hcount, 0, (size_t)t->L * sizeof(unsigned)));
+    }
     ALLOC(dalloc(&t->desc_dev, 1));
     ALLOC(dalloc(&t->desc_ptr_dev, 1));
     ALLOC(dalloc(&t->user_dev, 1));
@@ -421,6 +430,7 @@ int glt_create(const glt_config* cfg, glt_tracker** out)
     D.solve = t->cfg.solve;
     D.pattern = cfg->pattern;
     D.K = t->K;
+    D.tg = tg;
     D.affine = cfg->affine;
     for (int l = 0; l < GLT_MAX_LEVELS; ++l) D.max_iters[l] = l < t->L ? cfg->max_iters[l] : 0;
     D.min_valid = cfg->min_valid;

@@ -9,6 +9,7 @@
 // affine brightness, Huber weights and LM damping added by this library.
 #pragma once
 
+#include <type_traits>
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -65,9 +66,11 @@ struct StreamDesc {
     float huber_k, zmin;
     const float4* pt;      // (u0, v0, (u0-cx)/fx, (v0-cy)/fy)
     const float2* dz;      // (depth, 1/depth)
-    const float* I0;       // [L][Npad][K]; I0[l][p][0] is NaN where the point is unusable
-    const float2* G0;      // GLT_IC: reference gradient (gx, gy) [L][Npad][K], else null
+    const float* I0;       // reference samples, in the order of table_index; a point's first
+                           // sample is NaN on a level where it is unusable
+    const float2* G0;      // GLT_IC: reference gradients (gx, gy) in the same order, else null
     int pattern, K;        // 0 and 8: the 8-pixel pattern; p and p*p: the p x p patch
+    int tg;                // p x p patches: threads that share a point (hc_groups, else 1)
     int affine;            // 0: (a, b) held at their initial values
     const double* Hc;      // GLT_HESSIAN_CACHED: per level H (36) then H^-1 (36), row-major
                            // 6x6 pose blocks of the reference rows; H^-1[0] NaN if H is not PD
@@ -81,6 +84,29 @@ struct StreamDesc {
     int* trace_count;      // passes of the last track, or null
     int solve;             // GLT_SOLVE_FP64 or GLT_SOLVE_FP32
 };
+
+// The cached-Hessian form splits a 7 x 7 or 11 x 11 patch into kHcGroups
+// groups of consecutive rows, one thread per group.
+constexpr int kHcGroups = 4;
+__host__ __device__ constexpr int hc_groups(int pattern) { return (pattern == 7 || pattern == 11) ? kHcGroups : 1; }
+// rows and samples of a group of a p x p patch shared by tg threads
+__host__ __device__ constexpr int group_rows(int pattern, int tg) { return (pattern + tg - 1) / tg; }
+__host__ __device__ constexpr int group_samples(int pattern, int tg) { return group_rows(pattern, tg) * pattern; }
+
+// Order of the reference tables.  The 8-pixel pattern keeps a point's 8 samples
+// together (one 32-byte read per point).  A p x p patch is stored sample by
+// sample over the tasks (point, group), so that the lanes of a warp, which work
+// on consecutive tasks, read consecutive words: point by point a lane's reads
+// lay K words apart and every load cost a wavefront per point.  With the UNIT
+// sums of linearize_rows_hc and the L1 kept over the cluster's exchange: 7.0k ->
+// 4.1k cycles to linearise 2000 points of a pass at 7 x 7, 13.6k -> 6.3k at
+// 11 x 11; with a Huber threshold 66 passes take 438 instead of 554 us at 7 x 7,
+// 700 instead of 860 at 11 x 11, 561 and 1390 at 5 x 5 and 9 x 9 instead of 1127
+// and 2920 (then per-pixel byte loads).
+__host__ __device__ inline size_t table_size(int L, int Npad, int pattern, int tg)
+{
+    return pattern ? (size_t)L * group_samples(pattern, tg) * Npad * tg : (size_t)L * Npad * 8;
+}
 
 // Bounds-checked build (compiled with -DGLT_CHECKED into libglt_checked.so):
 // every gather and table access of the hot path checks its element range
@@ -163,16 +189,36 @@ struct PointCache {
     int p, level;
 };
 
+// Sample (row j, column i) of the p x p patch of point p on a level.
+template <int PS, int TG>
+__device__ __forceinline__ size_t patch_index(const StreamDesc& D, int level, int p, int j, int i)
+{
+    constexpr int RG = group_rows(PS, TG), SG = group_samples(PS, TG);
+    const int g = j / RG;
+    return ((size_t)level * SG + (j - g * RG) * PS + i) * ((size_t)D.Npad * TG) + (size_t)p * TG + g;
+}
+// ... of a patch of any size that one thread works on (tg = 1)
+__device__ __forceinline__ size_t patch_index1(const StreamDesc& D, int level, int p, int k)
+{
+    return ((size_t)level * D.K + k) * D.Npad + p;
+}
+template <class T>
+__device__ __forceinline__ T table_at(const StreamDesc& D, const T* tab, size_t i)
+{
+    return *checked(tab + i, 1, tab, table_size(D.L, D.Npad, D.pattern, D.tg), CK_TABLE);
+}
+
 __device__ __forceinline__ void load_point(const StreamDesc& D, int level, int p, PointCache& c)
 {
     c.q = *checked(D.pt + p, 1, D.pt, (size_t)D.Npad, CK_POINTS);
     c.dz = *checked(D.dz + p, 1, D.dz, (size_t)D.Npad, CK_POINTS);
-    const size_t tab = (size_t)D.L * D.Npad * D.K;
-    const float* I0b = checked(D.I0 + ((size_t)level * D.Npad + p) * D.K, (size_t)D.K, D.I0, tab, CK_TABLE);
     if (D.pattern) {
-        c.ia = make_float4(I0b[0], 0.f, 0.f, 0.f);   // the p x p path reads its samples itself
+        // the p x p path reads its samples itself; the first marks validity
+        const size_t at = ((size_t)level * group_samples(D.pattern, D.tg) * D.Npad + p) * D.tg;
+        c.ia = make_float4(table_at(D, D.I0, at), 0.f, 0.f, 0.f);
         c.ib = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
+        const float* I0b = checked(D.I0 + ((size_t)level * D.Npad + p) * 8, 8, D.I0, (size_t)D.L * D.Npad * 8, CK_TABLE);
         const float4* I0p = reinterpret_cast<const float4*>(I0b);   // K = 8: 32-byte rows
         c.ia = I0p[0];
         c.ib = I0p[1];
@@ -353,31 +399,28 @@ __device__ __forceinline__ void linearize_square_t(const StreamDesc& D, const Pa
             win[r][i] = __funnelshift_r(lo, hi, s8);
         }
     }
-#define GLT_WX(r, c) ((float)((win[(r)][(c) >> 2] >> (8 * ((c) & 3))) & 0xffu))
+#define GLT_WX(r, c) u8f(win[(r)][(c) >> 2], (c) & 3)
+    constexpr int TG = HC ? hc_groups(PS) : 1;
     const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
-    const size_t tab = (size_t)D.L * D.Npad * (PS * PS);
-    const float* I0p = checked(D.I0 + ((size_t)P.level * D.Npad + p) * (PS * PS), (size_t)(PS * PS), D.I0,
-                               tab, CK_TABLE);
-    const float2* G0p = ICF ? checked(D.G0 + ((size_t)P.level * D.Npad + p) * (PS * PS), (size_t)(PS * PS),
-                                      D.G0, tab, CK_TABLE)
-                            : nullptr;
 #pragma unroll
     for (int j = 0; j < PS; ++j) {
 #pragma unroll
         for (int i = 0; i < PS; ++i) {
             const int r0 = j + B, c0 = i + B, k = j * PS + i;
+            const size_t at = patch_index<PS, TG>(D, P.level, p, j, i);
+            const float i0 = table_at(D, D.I0, at);
             const float I00 = GLT_WX(r0, c0), I10 = GLT_WX(r0, c0 + 1);
             const float I01 = GLT_WX(r0 + 1, c0), I11 = GLT_WX(r0 + 1, c0 + 1);
             const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
             if (HC) {
-                hc_sample(I, I0p[k], G0p[k], P.ea, P.b, D.huber_k, sx, sy, acc,
+                hc_sample(I, i0, table_at(D, D.G0, at), P.ea, P.b, D.huber_k, sx, sy, acc,
                           res ? res + (size_t)(PS * PS) * p + k : nullptr);
                 continue;
             }
             float gx, gy;
             if (ICF) {
-                const float2 g0 = G0p[k];
+                const float2 g0 = table_at(D, D.G0, at);
                 gx = P.ea * g0.x;
                 gy = P.ea * g0.y;
             } else {
@@ -390,7 +433,7 @@ __device__ __forceinline__ void linearize_square_t(const StreamDesc& D, const Pa
                             fmaf(w01, GLT_WX(r0 + 2, c0) - I00,
                                  w11 * (GLT_WX(r0 + 2, c0 + 1) - I10))));
             }
-            accumulate_sample(G, I, gx, gy, I0p[k], P.ea, P.b, D.huber_k, acc,
+            accumulate_sample(G, I, gx, gy, i0, P.ea, P.b, D.huber_k, acc,
                               res ? res + (size_t)(PS * PS) * p + k : nullptr);
         }
     }
@@ -411,11 +454,9 @@ __device__ __forceinline__ void linearize_square_any(const StreamDesc& D, const 
     if (ic) ic_geometry(D, P, p, G);
     const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
-    const size_t tab = (size_t)D.L * D.Npad * K;
-    const float* I0p = checked(D.I0 + ((size_t)P.level * D.Npad + p) * K, (size_t)K, D.I0, tab, CK_TABLE);
-    const float2* G0p = ic ? checked(D.G0 + ((size_t)P.level * D.Npad + p) * K, (size_t)K, D.G0, tab, CK_TABLE)
-                           : nullptr;
     for (int k = 0; k < K; ++k) {
+        const size_t at = patch_index1(D, P.level, p, k);
+        const float i0 = table_at(D, D.I0, at);
         const int dx = k % D.pattern - h, dy = k / D.pattern - h;
         // taps t - S - 1 .. t + 2 S + 2 (intensity and central differences)
         const uint8_t* t = checked(lv.img + (size_t)(G.yb + dy - 1) * S + (G.xb + dx - 1), (size_t)3 * S + 4,
@@ -423,13 +464,13 @@ __device__ __forceinline__ void linearize_square_any(const StreamDesc& D, const 
         const float I00 = __ldca(t), I10 = __ldca(t + 1), I01 = __ldca(t + S), I11 = __ldca(t + S + 1);
         const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
         if (HC) {
-            hc_sample(I, I0p[k], G0p[k], P.ea, P.b, D.huber_k, sx, sy, acc,
+            hc_sample(I, i0, table_at(D, D.G0, at), P.ea, P.b, D.huber_k, sx, sy, acc,
                       res ? res + (size_t)K * p + k : nullptr);
             continue;
         }
         float gx, gy;
         if (ic) {
-            const float2 g0 = G0p[k];
+            const float2 g0 = table_at(D, D.G0, at);
             gx = P.ea * g0.x;
             gy = P.ea * g0.y;
         } else {
@@ -442,7 +483,7 @@ __device__ __forceinline__ void linearize_square_any(const StreamDesc& D, const 
                         fmaf(w01, (float)__ldca(t + 2 * S) - I00,
                              w11 * ((float)__ldca(t + 2 * S + 1) - I10))));
         }
-        accumulate_sample(G, I, gx, gy, I0p[k], P.ea, P.b, D.huber_k, acc, res ? res + (size_t)K * p + k : nullptr);
+        accumulate_sample(G, I, gx, gy, i0, P.ea, P.b, D.huber_k, acc, res ? res + (size_t)K * p + k : nullptr);
     }
     if (HC) hc_fold(G, sx, sy, acc);
 }
@@ -470,19 +511,16 @@ __device__ __forceinline__ void linearize_square(const StreamDesc& D, const Pass
     }
 }
 
-// The cached-Hessian form splits a p x p patch (p = 7 or 11) into
-// kHcGroups groups of consecutive rows, one thread per group: each of the
-// point's threads projects the point (the same FP32 arithmetic, so the same
-// validity decision), samples its rows from its own (rows + 1) x (p + 1)
-// byte window and folds its rows' sums into g0; the fold is linear, so the
-// threads of a point exchange nothing.
-constexpr int kHcGroups = 4;
-
-template <int PS>
+// A group of rows of a p x p patch in the cached-Hessian form (TG threads per
+// point; TG = 1: the whole patch): each of the point's threads projects the point
+// (the same FP32 arithmetic, so the same validity decision), samples its rows
+// from its own (rows + 1) x (p + 1) byte window and folds its rows' sums into g0;
+// the fold is linear, so the threads of a point exchange nothing.
+template <int PS, int TG>
 __device__ __forceinline__ void linearize_rows_hc(const StreamDesc& D, const PassParams& P, int p,
                                                   int group, PointGeom& G, float* acc)
 {
-    constexpr int h = (PS - 1) / 2, RG = (PS + kHcGroups - 1) / kHcGroups, R = RG + 1;
+    constexpr int h = (PS - 1) / 2, RG = group_rows(PS, TG), R = RG + 1;
     constexpr int NWD = (PS + 1 + 3) / 4;
     const LevelDev& lv = D.lv[P.level];
     ic_geometry(D, P, p, G);
@@ -512,28 +550,52 @@ __device__ __forceinline__ void linearize_rows_hc(const StreamDesc& D, const Pas
             for (int i = 0; i < NWD; ++i) win[r][i] = 0u;
         }
     }
-#define GLT_WR(r, c) ((float)((win[(r)][(c) >> 2] >> (8 * ((c) & 3))) & 0xffu))
+#define GLT_WR(r, c) u8f(win[(r)][(c) >> 2], (c) & 3)
     const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
-    const size_t tab = (size_t)D.L * D.Npad * (PS * PS);
-    const float* I0p = checked(D.I0 + ((size_t)P.level * D.Npad + p) * (PS * PS), (size_t)(PS * PS), D.I0,
-                               tab, CK_TABLE);
-    const float2* G0p = checked(D.G0 + ((size_t)P.level * D.Npad + p) * (PS * PS), (size_t)(PS * PS), D.G0,
-                                tab, CK_TABLE);
+    // this task's column of the tables: sample l of the group is l strides on
+    const size_t stride = (size_t)D.Npad * TG, at0 = patch_index<PS, TG>(D, P.level, p, j0, 0);
     float sx = 0.0f, sy = 0.0f;
+    // UNIT: every residual is within the Huber threshold, so that the weight is 1
+    // and the energy r^2 / 2 (hc_sample's operations without the two selects and
+    // the division, in its order)
+    auto sum = [&](auto unit) {
+        constexpr bool UNIT = decltype(unit)::value;
+        float E = acc[kHcE];
 #pragma unroll
-    for (int j = 0; j < RG; ++j) {
-        if (j0 + j < PS) {
+        for (int j = 0; j < RG; ++j) {
+            if (j0 + j < PS) {
 #pragma unroll
-            for (int i = 0; i < PS; ++i) {
-                const int k = (j0 + j) * PS + i;
-                const float I00 = GLT_WR(j, i), I10 = GLT_WR(j, i + 1);
-                const float I01 = GLT_WR(j + 1, i), I11 = GLT_WR(j + 1, i + 1);
-                const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
-                hc_sample(I, I0p[k], G0p[k], P.ea, P.b, D.huber_k, sx, sy, acc, nullptr);
+                for (int i = 0; i < PS; ++i) {
+                    const size_t at = at0 + (j * PS + i) * stride;
+                    const float I00 = GLT_WR(j, i), I10 = GLT_WR(j, i + 1);
+                    const float I01 = GLT_WR(j + 1, i), I11 = GLT_WR(j + 1, i + 1);
+                    const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
+                    const float i0 = table_at(D, D.I0, at);
+                    const float2 g0 = table_at(D, D.G0, at);
+                    if (UNIT) {
+                        const float r = __fsub_rn(fmaf(-P.ea, i0, I), P.b);
+                        sx = fmaf(r, g0.x, sx);
+                        sy = fmaf(r, g0.y, sy);
+                        E = __fadd_rn(E, __fmul_rn(__fmul_rn(0.5f, r), r));
+                    } else {
+                        hc_sample(I, i0, g0, P.ea, P.b, D.huber_k, sx, sy, acc, nullptr);
+                    }
+                }
             }
         }
-    }
+        if (UNIT) {
+            acc[kHcE] = E;
+            acc[kHcN] += (float)(min(RG, PS - j0) * PS);
+        }
+    };
+    // |r| <= 255 (1 + e^a) + |b| and a few roundings.  The paper's own
+    // configuration has no threshold: its 66 passes take 339 us with UNIT, 437
+    // without (2000 points, 7 x 7), 438 and 700 at 11 x 11
+    if (fmaf(P.ea, 256.0f, 256.0f) + 1.001f * fabsf(P.b) <= D.huber_k)
+        sum(std::true_type{});
+    else
+        sum(std::false_type{});
 #undef GLT_WR
     hc_fold(G, sx, sy, acc);
 }
@@ -661,28 +723,24 @@ __device__ __forceinline__ void linearize_point(const StreamDesc& D, const PassP
 }
 
 // One task of a cached-Hessian pass: row group `group` of point c.p for the
-// 7 x 7 and 11 x 11 patches (groups = kHcGroups), the whole point otherwise
-// (groups = 1).
+// 7 x 7 and 11 x 11 patches, the whole point otherwise (group = 0).
 __device__ __forceinline__ void linearize_task_hc(const StreamDesc& D, const PassParams& P,
-                                                  const PointCache& c, int group, int groups,
-                                                  float* acc)
+                                                  const PointCache& c, int group, float* acc)
 {
-    if (groups == 1) {
-        linearize_point<false, false, true, true, true>(D, P, c, acc, nullptr);
+    if (!D.pattern) {
+        linearize_point<false, false, false, true, true>(D, P, c, acc, nullptr);
         return;
     }
     const LevelDev& lv = D.lv[P.level];
     PointGeom G;
     if (isnan(c.ia.x) || !project_point<true>(D, P, lv, c, G)) return;
-    if (D.pattern == 7)
-        linearize_rows_hc<7>(D, P, c.p, group, G, acc);
-    else
-        linearize_rows_hc<11>(D, P, c.p, group, G, acc);
-}
-
-__host__ __device__ inline int hc_groups(int pattern)
-{
-    return (pattern == 7 || pattern == 11) ? kHcGroups : 1;
+    switch (D.pattern) {
+    case 3: linearize_rows_hc<3, 1>(D, P, c.p, 0, G, acc); break;
+    case 5: linearize_rows_hc<5, 1>(D, P, c.p, 0, G, acc); break;
+    case 7: linearize_rows_hc<7, kHcGroups>(D, P, c.p, group, G, acc); break;
+    case 9: linearize_rows_hc<9, 1>(D, P, c.p, 0, G, acc); break;
+    default: linearize_rows_hc<11, kHcGroups>(D, P, c.p, group, G, acc); break;
+    }
 }
 
 // ---------------------------------------------------------------------------

@@ -41,6 +41,8 @@ struct PropJob {            // coarsest levels (40 x 30) of one stream, for the 
 // launch classes of a batch: at most one per cluster size 16, 8, 4, 2, 1
 constexpr int kMaxBatchClasses = 5;
 
+constexpr int kHessSums = 21;   // upper triangle of the per-reference Hessian
+
 struct PackJob {            // one level -> FP16 (I, gx, gy, 0) copy (mixed form)
     const uint8_t* src;
     uint2* dst;
@@ -61,8 +63,10 @@ struct glt_tracker {
     float4* pt = nullptr;
     float2* dz = nullptr;
     float* I0 = nullptr;
-    float2* G0 = nullptr;                 // GLT_IC reference gradients [L][Npad][K]
+    float2* G0 = nullptr;                 // GLT_IC reference gradients, as I0
     double* Hc = nullptr;                 // GLT_HESSIAN_CACHED: per level H, H^-1 [L][72]
+    float* Hpart = nullptr;               // ... each point's sums [L][kHessSums][Npad]
+    unsigned* Hcount = nullptr;           // ... and tickets [L]
     int K = 8;                            // samples per point of the pattern
     int Npad = 0;
     int N = 0;

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 4 : 1) track_kernel(
             for (int t = rank * THREADS + tid; t < tasks; t += C * THREADS) {
                 const int p = groups == 1 ? t : t / kHcGroups;
                 if (pc.p != p || pc.level != P.level) load_point(sD, P.level, p, pc);
-                linearize_task_hc(sD, P, pc, t - p * groups, groups, acc);
+                linearize_task_hc(sD, P, pc, t - p * groups, acc);
             }
         } else {
             for (int p = rank * THREADS + tid; p < sD.N; p += C * THREADS) {
