@@ -53,19 +53,25 @@ __device__ __forceinline__ void mbar_arrive_expect(unsigned long long* m, unsign
                  : "memory");
 }
 
-// true once the phase of parity `parity` has completed; false after `limit` cycles
+// true once the phase of parity `parity` has completed; false after `limit` cycles.
+// The acquire is cluster-wide, since the pushes come from other CTAs, but covers
+// shared memory only: a plain .acquire.cluster wait drops the SM's L1 each pass,
+// and with it the patch tables and window rows the next pass reads again.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* m, unsigned parity, long long limit)
 {
     const long long t0 = clock64();
     while (true) {
         unsigned done;
         asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done)
                      : "r"(smem_addr(m)), "r"(parity)
                      : "memory");
-        if (done) return true;
+        if (done) {
+            asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
+            return true;
+        }
         if (clock64() - t0 > limit) return false;
     }
 }
