@@ -885,26 +885,27 @@ __device__ __forceinline__ void block_reduce(float (&acc)[kAccPad], float (*red)
 //  * accept/reject compares E' n <= E n' instead of dividing, and only for
 //    steps that are not small enough to be taken anyway.
 // ---------------------------------------------------------------------------
-// 1 / d for a positive d in [2^-100, 2^100) without an FP64 instruction.  With
-// d = 2^E m, m = mh + ml in [1, 2) split at FP32's 24 bits (ml cut at 2^-46):
-// q = rcp.approx.ftz.f32(mh), the residual e = 1 - m q in two FP32 FMAs (error
-// below 2^-46, |e| <= 2^-22), and 1 / m = q / (1 - e) = q + q (e + e^2) +
-// O(e^3): the FP32 correction is added to q's significand as an integer in
-// units of 2^-52, and the exponent lowered by E.  Relative error below 2^-45;
-// the Newton step in FP64 that this replaces cost two dependent FP64
-// instructions (128 cycles) for 2^-44.
+// 1 / d for a positive d in [2^-100, 2^100) without an FP64 instruction: one
+// Newton step in integers.  With d = 2^E m, m = M / 2^52 in [1, 2), the seed q =
+// rcp.approx.ftz.f32 of m cut to FP32 is Q / 2^24 with a whole Q; the residual e
+// = 1 - m q, at most 2^-22, is exactly -(M Q) modulo 2^64 in units of 2^-76, and
+// q + q e is formed on the bits of the result (units of 2^-53) and lowered by E
+// in the exponent.  The value of r0 + r0 (1 - d r0) in FP64 to an ulp (relative
+// error e^2 < 2^-43.9 and that ulp), without its two dependent FP64 instructions
+// (128 cycles) and their way out of the FP64 pipe.
 __device__ __forceinline__ double rcp_mid(double d)
 {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const float mh = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u);
-    const float ml = fmaf(__uint_as_float(((lo >> 6) & 0x7fffffu) | 0x3f800000u), 0x1p-23f, -0x1p-23f);
     float q;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
-    const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
-    const int c = __float2int_rn((q * 0x1p52f) * fmaf(e, e, e));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(__uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u)));
+    const unsigned qb = __float_as_uint(q);
+    const unsigned Q = qb >= 0x3f800000u ? 0x1000000u : (qb & 0x7fffffu) | 0x800000u;
+    const unsigned long long M = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const long long e = -(long long)(M * Q);
+    const int es = (int)((e + (1ll << 23)) >> 24);
+    const long long c = ((long long)es * (int)Q + (1ll << 22)) >> 23;
     const unsigned off = ((896u + 1023u) << 20) - (hi & 0x7ff00000u);
-    const long long m = ((long long)__float_as_uint(q) << 29) + 2ll * c + ((long long)off << 32);
-    return __longlong_as_double(m);
+    return __longlong_as_double(((long long)qb << 29) + c + ((long long)off << 32));
 }
 
 // Reciprocal of any d: rcp_mid for 2^-100 <= |d| < 2^100 (exponent tested as
