@@ -509,10 +509,10 @@ int glt_build_pyramid(glt_tracker* t, int slot, const uint8_t* img, int pitch_by
     // every kernel after the first is a programmatic dependent of the one
     // before it (it starts early and waits on the device for its source level)
     if (is_device && t->L > 1) {
-        // level 1 straight from the caller's frame; its tiles write level 0
+        // level 1 straight from the caller's frame; its blocks write level 0
         for (int l = 1; l < t->L; ++l)
             GLT_CHECK(launch_pyr_down(t->jobs_dev + slot * GLT_MAX_LEVELS + (l - 1), nullptr,
-                                      pyr_tiles_x(t->W[l]) * pyr_tiles_y(t->H[l]), s, nullptr,
+                                      pyr_blocks(t->W[l], t->H[l]), s, nullptr,
                                       l == 1 ? img : nullptr, l == 1 ? pitch_bytes : 0, l > 1),
                       "pyramid kernel");
         if (slot == GLT_CUR && t->packed)
@@ -526,7 +526,7 @@ int glt_build_pyramid(glt_tracker* t, int slot, const uint8_t* img, int pitch_by
               "level-0 copy");
     for (int l = 1; l < t->L; ++l)
         GLT_CHECK(launch_pyr_down(t->jobs_dev + slot * GLT_MAX_LEVELS + (l - 1), nullptr,
-                                  pyr_tiles_x(t->W[l]) * pyr_tiles_y(t->H[l]), s, nullptr, nullptr, 0,
+                                  pyr_blocks(t->W[l], t->H[l]), s, nullptr, nullptr, 0,
                                   l > 1),
                   "pyramid kernel");
     if (slot == GLT_CUR && t->packed) {
@@ -983,15 +983,15 @@ int glt_batch_create(glt_tracker* const* trackers, int S, glt_batch** out)
             }
         }
     }
-    // per round, every output tile of every stream as (stream << 16) | tile:
-    // one CTA per entry in the batched pyramid kernel
+    // per round, every block of every stream as (stream << 16) | block: one CTA
+    // per entry in the batched pyramid kernel
     const int rounds = std::max(1, b->Lmax - 1);
     std::vector<unsigned> tmap;
     for (int r = 0; r < rounds; ++r) {
         b->tile_map_off[r] = tmap.size();
         for (int i = 0; i < S; ++i) {
             const PyrJob& J = jobs[(size_t)r * S + i];
-            const int n = pyr_tiles_x(J.dW) * pyr_tiles_y(J.dH);
+            const int n = pyr_blocks(J.dW, J.dH);
             for (int k = 0; k < n; ++k) tmap.push_back(((unsigned)i << 16) | (unsigned)k);
         }
         b->tile_total[r] = (int)(tmap.size() - b->tile_map_off[r]);

@@ -2,15 +2,14 @@
 // downsample; level 0 is the full-resolution frame).
 //
 // Level l from level l-1: out(x, y) = (sum_{i,j=-2..2} w_i w_j in(2x+i, 2y+j) + 128) >> 8
-// with w = [1 4 6 4 1], clamp-to-edge, computed exactly in integers.  Work is
-// cut into 64 x 16 output tiles: a CTA stages a tile's input window (2*64+8
-// columns from the 4-byte aligned column 2*x0-4, 2*16+3 rows) in shared memory
-// with 4-byte loads, runs the vertical pass (two columns per 32-bit lane pair)
-// and the horizontal pass, and stores 4 output bytes per thread.  The
-// grid has one CTA per tile over all jobs (one job per stream, so a whole
-// batch of streams builds a level in one launch).  Level 1 reads the caller's frame and
-// writes the level-0 copy from its staged windows, so a frame is read from HBM
-// once.
+// with w = [1 4 6 4 1], clamp-to-edge, computed exactly in integers.  A thread
+// makes 8 x 4 outputs in registers: it reads the 16 columns and 11 rows above
+// them with 16-byte loads, all issued before the first use, takes the three
+// columns beyond from its neighbours' registers, filters each row horizontally
+// (two outputs per 32-bit lane pair) and then five rows vertically.  The blocks
+// of a level are cut from the flat list of its threads, a whole batch of streams
+// in one launch.  Level 1 reads the caller's frame and writes the level-0 copy
+// from its registers, so a frame is read from HBM once.
 #include <algorithm>
 
 #include "glt_internal.h"
@@ -18,245 +17,216 @@
 namespace glt {
 
 namespace {
-constexpr int TW = 64;               // output tile width
-constexpr int TH = 16;               // output tile height
-constexpr int IW = 2 * TW + 8;       // staged input columns 2*ox0-4 .. 2*ox0+2*TW+3
-constexpr int IH = 2 * TH + 3;
-constexpr int PYR_THREADS = 256;
+constexpr int PX = 8, PY = 4;        // outputs of a thread
+constexpr int PR = 2 * PY + 3;       // input rows of a thread
+constexpr int PYR_THREADS = 128;
 }  // namespace
 
-__host__ __device__ int pyr_tiles_x(int dW) { return (dW + TW - 1) / TW; }
-__host__ __device__ int pyr_tiles_y(int dH) { return (dH + TH - 1) / TH; }
+// Blocks of a level of dW x dH outputs.
+__host__ __device__ int pyr_blocks(int dW, int dH)
+{
+    return (((dW + PX - 1) / PX) * ((dH + PY - 1) / PY) + PYR_THREADS - 1) / PYR_THREADS;
+}
 
-// One output tile of a launch: the level job (for level 1 with the caller's
-// frame as its source and the level-0 buffer as copy0), its corner, and
-// whether the source rows are 4-byte aligned (word loads; `interior`) or need
-// byte loads throughout.
+// One block of a launch: the level job (for level 1 with the caller's frame as
+// its source and the level-0 buffer as copy0) and its place in the job.
 struct Tile {
     PyrJob J;
     uint8_t* copy0;
-    int cp, ox0, oy0;
-    bool interior;
+    int cp, local;
 };
 
-// Tile f of the launch: tile_map[f] = (job << 16) | tile within the job
-// (row-major), or, for one job without a map, f itself.
+// Block f of the launch: tile_map[f] = (job << 16) | block within the job, or,
+// for one job without a map, f itself.
 __device__ __forceinline__ Tile tile_at(const PyrJob* __restrict__ jobs, const unsigned* __restrict__ tile_map,
                                         const uint8_t* const* frames, const uint8_t* src, int sp, int f)
 {
-    int z = 0, local = f;
+    int z = 0;
+    Tile t;
+    t.local = f;
     if (tile_map) {
         const unsigned m = tile_map[f];
         z = (int)(m >> 16);
-        local = (int)(m & 0xffffu);
+        t.local = (int)(m & 0xffffu);
     }
-    Tile t;
     t.J = jobs[z];
-    const int tx = pyr_tiles_x(t.J.dW);
-    const int ty = local / tx;
-    t.ox0 = (local - ty * tx) * TW;
-    t.oy0 = ty * TH;
     t.copy0 = nullptr;
     t.cp = 0;
     if (frames || src) {
-        // level 1 from the caller's frame; the tiles also write the level-0 copy
+        // level 1 from the caller's frame; the blocks also write the level-0 copy
         t.copy0 = const_cast<uint8_t*>(t.J.src);
         t.cp = t.J.sp;
         t.J.src = frames ? frames[z] : src;
         t.J.sp = frames ? t.J.sW : sp;
     }
-    t.interior = ((t.J.sp & 3) == 0) && ((reinterpret_cast<uintptr_t>(t.J.src) & 3) == 0);
     return t;
 }
 
-constexpr int kWordsPerRow = IW / 4, kWords = IH * kWordsPerRow;
-constexpr int kPer = (kWords + PYR_THREADS - 1) / PYR_THREADS;
-
-// Source loads: a level written by the previous kernel of a programmatic
-// chain is read from L2 (ld.global.cg); the caller's frame, which no kernel
-// of the chain writes (level 1 is launched as an ordinary kernel), through
-// the read-only path.
-__device__ __forceinline__ uint32_t src_word(const Tile& t, const uint8_t* p)
+// Source loads are L2 loads: a level written by the previous kernel of a
+// programmatic chain, or a frame of which nothing is read twice but the rows
+// that two threads share.
+template <class T>
+__device__ __forceinline__ T src_load(const PyrJob& J, const uint8_t* p)
 {
-    p = checked(p, 4, t.J.src, (size_t)t.J.sp * t.J.sH, CK_PYR_SRC);
-    const unsigned int* w = reinterpret_cast<const unsigned int*>(p);
-    return t.copy0 ? __ldg(w) : __ldcg(w);
+    return __ldcg(reinterpret_cast<const T*>(checked(p, sizeof(T), J.src, (size_t)J.sp * J.sH, CK_PYR_SRC)));
 }
-__device__ __forceinline__ uint8_t src_byte(const Tile& t, const uint8_t* p)
+__device__ __forceinline__ uint32_t src_byte(const PyrJob& J, const uint8_t* row, int x)
 {
-    p = checked(p, 1, t.J.src, (size_t)t.J.sp * t.J.sH, CK_PYR_SRC);
-    return t.copy0 ? __ldg(p) : __ldcg(p);
+    return src_load<uint8_t>(J, row + min(max(x, 0), J.sW - 1));
 }
 
-// The staged window's 4-byte words for a tile with aligned source rows,
-// issued into registers (all of a thread's loads before any use: one memory
-// round trip).  A word whose 4 source columns lie inside the row is one load;
-// a word at the left or right border is assembled from its clamped columns.
-__device__ __forceinline__ void issue_window(const Tile& t, uint32_t (&v)[kPer])
-{
-    const int ix0 = 2 * t.ox0 - 4, iy0 = 2 * t.oy0 - 2;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int i = threadIdx.x + k * PYR_THREADS;
-        if (i < kWords) {
-            const int r = i / kWordsPerRow, c = i % kWordsPerRow;
-            const uint8_t* row = t.J.src + (size_t)min(max(iy0 + r, 0), t.J.sH - 1) * t.J.sp;
-            const int x = ix0 + 4 * c;
-            if (x >= 0 && x + 3 < t.J.sW) {
-                v[k] = src_word(t, row + x);
-            } else {
-                uint32_t w = 0;
-#pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    w |= (uint32_t)src_byte(t, row + min(max(x + b, 0), t.J.sW - 1)) << (8 * b);
-                v[k] = w;
-            }
-        }
-    }
-}
-
-// Lands the window in shared memory: the issued words of an aligned tile,
-// or (unaligned source rows) byte loads with clamped columns, in groups of 8
-// per thread.
-__device__ __forceinline__ void land_window(const Tile& t, const uint32_t (&v)[kPer], uint8_t (*in)[IW])
-{
-    if (t.interior) {
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) {
-            const int i = threadIdx.x + k * PYR_THREADS;
-            if (i < kWords) *reinterpret_cast<uint32_t*>(&in[i / kWordsPerRow][4 * (i % kWordsPerRow)]) = v[k];
-        }
-        return;
-    }
-    const int ix0 = 2 * t.ox0 - 4, iy0 = 2 * t.oy0 - 2;
-    constexpr int NB = IH * IW, PER = (NB + PYR_THREADS - 1) / PYR_THREADS, G = 8;
-#pragma unroll
-    for (int k0 = 0; k0 < PER; k0 += G) {
-        uint8_t b[G];
-#pragma unroll
-        for (int k = 0; k < G; ++k) {
-            const int i = threadIdx.x + (k0 + k) * PYR_THREADS;
-            if (k0 + k < PER && i < NB) {
-                const int r = i / IW, c = i % IW;
-                const int gy = min(max(iy0 + r, 0), t.J.sH - 1);
-                const int gx = min(max(ix0 + c, 0), t.J.sW - 1);
-                b[k] = src_byte(t, t.J.src + (size_t)gy * t.J.sp + gx);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < G; ++k) {
-            const int i = threadIdx.x + (k0 + k) * PYR_THREADS;
-            if (k0 + k < PER && i < NB) in[i / IW][i % IW] = b[k];
-        }
-    }
-}
-
-// The tile's outputs from its staged window.  If copy0 is set (level 1 built
-// straight from the source frame), the tile also writes its share of the
-// level-0 copy (pitch cp): source rows [2 oy0, 2 oy0 + 2 TH) and columns
-// [2 ox0, 2 ox0 + 2 TW), extended to the frame's last row / column on the last
-// tile row / column, so the tiles partition level 0.
-__device__ __forceinline__ void tile_outputs(const Tile& t, uint8_t (*in)[IW], uint32_t* vs)
-{
-    const PyrJob& J = t.J;
-    const int ox0 = t.ox0, oy0 = t.oy0;
-    if (t.copy0) {
-        const int y0 = 2 * oy0, y1 = oy0 + TH >= J.dH ? J.sH : 2 * oy0 + 2 * TH;
-        const int x0 = 2 * ox0, x1 = ox0 + TW >= J.dW ? J.sW : 2 * ox0 + 2 * TW;
-        const int nw = (x1 - x0) >> 2;          // whole 4-byte words (x0 is a multiple of 128): <= 32
-        const int tail = (x1 - x0) & 3;
-        // staged row r + 2 is source row y0 + r, staged column 4 source column x0;
-        // 32 word slots per row, then the 0-3 tail bytes of every row
-        for (int i = threadIdx.x; i < (y1 - y0) * 32; i += PYR_THREADS) {
-            const int r = i >> 5, k = i & 31;
-            if (k < nw)
-                *reinterpret_cast<uint32_t*>(checked(t.copy0 + (size_t)(y0 + r) * t.cp + x0 + 4 * k, 4, t.copy0,
-                                                     (size_t)t.cp * J.sH, CK_PYR_DST)) =
-                    *reinterpret_cast<const uint32_t*>(&in[r + 2][4 + 4 * k]);
-        }
-        if (tail) {
-            for (int i = threadIdx.x; i < (y1 - y0) * 4; i += PYR_THREADS) {
-                const int r = i >> 2, k = i & 3;
-                if (k < tail)
-                    *checked(t.copy0 + (size_t)(y0 + r) * t.cp + x0 + 4 * nw + k, 1, t.copy0, (size_t)t.cp * J.sH,
-                             CK_PYR_DST) = in[r + 2][4 + 4 * nw + k];
-            }
-        }
-    }
-    // vertical 5-tap pass, one 4-byte word (4 staged columns) per item: both
-    // 16-bit lanes of a u32 carry one column's sum (at most 16 * 255), so one
-    // 32-bit multiply-add serves two columns; the sums go to two planes by
-    // column parity, ve[y][w] = (V[4w], V[4w+2]) and vo[y][w] = (V[4w+1], V[4w+3])
-    uint32_t* ve = vs;
-    uint32_t* vo = vs + TH * (IW / 4);
-    for (int i = threadIdx.x; i < TH * (IW / 4); i += PYR_THREADS) {
-        const int y = i / (IW / 4), w = i - y * (IW / 4);
-        const uint32_t* col = reinterpret_cast<const uint32_t*>(&in[2 * y][0]) + w;
-        uint32_t lo = 0, hi = 0;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            const uint32_t a = col[k * (IW / 4)];
-            const uint32_t wk = k == 2 ? 6u : (k == 1 || k == 3) ? 4u : 1u;
-            lo += wk * (a & 0x00ff00ffu);
-            hi += wk * ((a >> 8) & 0x00ff00ffu);
-        }
-        ve[i] = lo;
-        vo[i] = hi;
-    }
-    __syncthreads();
-    // horizontal pass, 4 output pixels per item, two per 32-bit lane pair:
-    // output x (tile-local) takes staged columns 2x+2 .. 2x+6, i.e.
-    // Ve[x+1] + 4 Vo[x+1] + 6 Ve[x+2] + 4 Vo[x+2] + Ve[x+3], where Ve[e] = V[2e]
-    // and Vo[e] = V[2e+1]; a lane sum is at most 16 * 16 * 255 + 128 < 2^16
-    for (int i = threadIdx.x; i < TH * (TW / 4); i += PYR_THREADS) {
-        const int y = i / (TW / 4), x4 = (i % (TW / 4)) * 4;
-        const int gy = oy0 + y;
-        if (gy >= J.dH) continue;
-        const uint32_t* e = ve + y * (IW / 4) + (x4 >> 1);
-        const uint32_t* o = vo + y * (IW / 4) + (x4 >> 1);
-        const uint32_t e0 = e[0], e1 = e[1], e2 = e[2], e3 = e[3];
-        const uint32_t o0 = o[0], o1 = o[1], o2 = o[2];
-        // pair (x4, x4+1): A = Ve(x+1, x+2), B = Ve(x+2, x+3), C = Ve(x+3, x+4),
-        // D = Vo(x+1, x+2), E = Vo(x+2, x+3) with x = x4; pair (x4+2, x4+3) one word on
-        const uint32_t s01 = __byte_perm(e0, e1, 0x5432) + 6u * e1 + __byte_perm(e1, e2, 0x5432) +
-                             4u * (__byte_perm(o0, o1, 0x5432) + o1) + 0x00800080u;
-        const uint32_t s23 = __byte_perm(e1, e2, 0x5432) + 6u * e2 + __byte_perm(e2, e3, 0x5432) +
-                             4u * (__byte_perm(o1, o2, 0x5432) + o2) + 0x00800080u;
-        const uint32_t packed = __byte_perm(s01 >> 8, s23 >> 8, 0x6420);
-        const int gx = ox0 + x4;
-        uint8_t* dst = J.dst + (size_t)gy * J.dp + gx;
-        if (gx < J.dW) dst = checked(dst, (size_t)min(4, J.dW - gx), J.dst, (size_t)J.dp * J.dH, CK_PYR_DST);
-        if (gx + 4 <= J.dW && ((reinterpret_cast<uintptr_t>(dst) & 3) == 0)) {
-            *reinterpret_cast<uint32_t*>(dst) = packed;
-        } else {
-            for (int k = 0; k < 4 && gx + k < J.dW; ++k) dst[k] = (uint8_t)(packed >> (8 * k));
-        }
-    }
-}
-
-// One level of S streams, one CTA per output tile over all jobs (no idle
-// CTAs for the smaller streams of a batch).  For level 1 the source can be
-// the caller's frame instead of the level-0 buffer: `frames` (a device table
+// One level of S streams, PX x PY outputs a thread.  For level 1 the source can
+// be the caller's frame instead of the level-0 buffer: `frames` (a device table
 // of S contiguous frames, pitch = width) or `src` / `sp` (one stream); the
-// tiles then also write the level-0 copy into the job's source buffer.
-__global__ void __launch_bounds__(PYR_THREADS, 8) pyr_down_kernel(const PyrJob* __restrict__ jobs,
+// threads then also write the level-0 copy into the job's source buffer.
+//
+// Bound in a batch by the loads in flight (256 frames of 640 x 480, 4 levels:
+// 62 us, 43% of the copy bandwidth), for one frame by the launch and one memory
+// round trip.  8 x 4 outputs: 16-byte loads, three rows in eleven read twice
+// (from L2), 44 words a thread in flight, ~16 instructions an output.  Staging
+// 64 x 16 tiles in shared memory with 4-byte loads was bound by issue (~150
+// instructions an output): 136 us for the batch, 47 instead of 23 us for 64
+// frames of mixed sizes.
+__global__ void __launch_bounds__(PYR_THREADS, 5) pyr_down_kernel(const PyrJob* __restrict__ jobs,
                                                                   const unsigned* __restrict__ tile_map,
                                                                   const uint8_t* const* frames,
                                                                   const uint8_t* src, int sp)
 {
-    __shared__ __align__(16) uint8_t in[IH][IW];
-    __shared__ __align__(16) uint32_t vs[2 * TH * (IW / 4)];   // the two parity planes
     // the next level's kernel (or the track kernel) may start its setup now;
-    // the tile's description (tables written before the chain started) is
+    // the block's description (tables written before the chain started) is
     // read at once, this level's source only once the previous kernel is done
     griddep_launch_dependents();
     const Tile t = tile_at(jobs, tile_map, frames, src, sp, (int)blockIdx.x);
+    const PyrJob& J = t.J;
+    const int nx = (J.dW + PX - 1) / PX, ny = (J.dH + PY - 1) / PY;
+    const int idx = t.local * PYR_THREADS + (int)threadIdx.x, lane = (int)threadIdx.x & 31;
+    // (threads beyond the last repeat it without stores, for the shuffles)
+    const bool active = idx < nx * ny;
+    const int i = min(idx, nx * ny - 1), by = i / nx, bx = i - by * nx;
+    const int ix = 2 * PX * bx, iy = 2 * PY * by - 2;
+    const int nv = J.sW - ix;            // columns of the row from ix on
+    const bool wide = ((reinterpret_cast<uintptr_t>(J.src) | (uintptr_t)J.sp) & 15u) == 0;
     griddep_wait();
-    uint32_t v[kPer];
-    if (t.interior) issue_window(t, v);
-    land_window(t, v, in);
-    __syncthreads();
-    tile_outputs(t, in, vs);
+    // rows iy .. iy + 10 (clamped), columns ix .. ix + 15; and, where no
+    // neighbour in the warp has them, columns ix - 2, ix - 1 or ix + 16
+    const bool left = lane == 0 && bx > 0, right = lane == 31 || bx == nx - 1;
+    uint32_t m[PR][4], ed[PR];
+    // Bytes beyond a row are any (replaced below) but never read from outside
+    // the source: a level's rows have their pitch, a frame ends with its last row.
+    auto row_at = [&](int r) { return J.src + (size_t)min(max(iy + r, 0), J.sH - 1) * J.sp; };
+    const uint8_t* end = J.src + (t.copy0 ? (size_t)(J.sH - 1) * J.sp + J.sW : (size_t)J.sH * J.sp);
+    if (wide && row_at(PR - 1) + ix + 16 <= end) {
+#pragma unroll
+        for (int r = 0; r < PR; ++r) {
+            const uint4 v = src_load<uint4>(J, row_at(r) + ix);
+            m[r][0] = v.x;
+            m[r][1] = v.y;
+            m[r][2] = v.z;
+            m[r][3] = v.w;
+        }
+    } else {
+        // rows of any alignment (a frame): the aligned words around the columns;
+        // lo and hi are the first and the last word that lie in the frame, head and
+        // tail its bytes before and after them
+        const unsigned a0 = (unsigned)(reinterpret_cast<uintptr_t>(J.src) & 3u);
+        const long long n = end - J.src, lo = -a0 & 3u, hi = n - (long long)((n + a0) & 3u) - 4;
+        uint32_t head = 0, tail = 0;
+#pragma unroll
+        for (int b = 1; b < 4; ++b)
+            if (lo - 4 + b >= 0) head |= (uint32_t)src_load<uint8_t>(J, J.src + lo - 4 + b) << (8 * b);
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            if (hi + 4 + b < n) tail |= (uint32_t)src_load<uint8_t>(J, J.src + hi + 4 + b) << (8 * b);
+#pragma unroll
+        for (int r = 0; r < PR; ++r) {
+            const long long at = row_at(r) - J.src + ix;
+            const unsigned a = (unsigned)(at + a0) & 3u;
+            uint32_t w[5];
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const long long o = at - a + 4 * q;
+                w[q] = src_load<uint32_t>(J, J.src + min(max(o, lo), hi));
+                w[q] = o < lo ? head : o > hi ? tail : w[q];     // (words beyond the tail hold no column of the row)
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) m[r][q] = __funnelshift_r(w[q], w[q + 1], 8 * a);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < PR; ++r) {
+        const uint8_t* row = row_at(r);
+        ed[r] = 0;
+        if (left) ed[r] = src_byte(J, row, ix - 2) << 16 | src_byte(J, row, ix - 1) << 24;
+        if (right) ed[r] |= src_byte(J, row, ix + 16);
+    }
+    if (nv < 16) {
+        // the row ends within the 16 columns: its last byte beyond
+        const int k = (nv - 1) & 3;
+#pragma unroll
+        for (int r = 0; r < PR; ++r) {
+            const uint32_t lw = nv > 12 ? m[r][3] : nv > 8 ? m[r][2] : nv > 4 ? m[r][1] : m[r][0];
+            const uint32_t rep = __byte_perm(lw, 0, 0x1111u * k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int n = nv - 4 * q;
+                if (n < 4) m[r][q] = __byte_perm(m[r][q], rep, n <= 0 ? 0x4444 : n == 1 ? 0x4440 : n == 2 ? 0x4410 : 0x4210);
+            }
+        }
+    }
+    if (t.copy0 && active) {
+        // source rows 8 by .. 8 by + 7 and, of the last thread row, what is left
+#pragma unroll
+        for (int r = 2; r < PR; ++r) {
+            const int y = iy + r;
+            if (y < J.sH && (r < PR - 1 || by == ny - 1)) {
+                uint8_t* d = checked(t.copy0 + (size_t)y * t.cp + ix, 16, t.copy0, (size_t)t.cp * J.sH, CK_PYR_DST);
+                *reinterpret_cast<uint4*>(d) = make_uint4(m[r][0], m[r][1], m[r][2], m[r][3]);
+                if (bx == nx - 1 && nv > 16) d[16] = (uint8_t)ed[r];
+            }
+        }
+    }
+    // horizontal sums of two outputs in the halves of a word (at most 16 * 255):
+    // E = even columns, O = odd; output x of the pair is Ve[x-1] + 4 Vo[x-1] +
+    // 6 Ve[x] + 4 Vo[x] + Ve[x+1]
+    uint32_t h[5][4];
+#pragma unroll
+    for (int r = 0; r < PR; ++r) {
+        uint32_t L = __shfl_up_sync(0xffffffffu, m[r][3], 1), R = __shfl_down_sync(0xffffffffu, m[r][0], 1);
+        if (bx == 0)
+            L = __byte_perm(m[r][0], 0, 0x0000);
+        else if (lane == 0)
+            L = ed[r];
+        if (right) R = ed[r];
+        uint32_t E[4], O[4], e[5], o[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            E[q] = m[r][q] & 0x00ff00ffu;
+            O[q] = __byte_perm(m[r][q], 0, 0x4341);
+        }
+        e[0] = __byte_perm(L, E[0], 0x5452);
+        o[0] = __byte_perm(L, O[0], 0x5453);
+#pragma unroll
+        for (int q = 1; q < 4; ++q) {
+            e[q] = __byte_perm(E[q - 1], E[q], 0x5432);
+            o[q] = __byte_perm(O[q - 1], O[q], 0x5432);
+        }
+        e[4] = __byte_perm(E[3], R & 0xffu, 0x5432);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) h[r % 5][q] = e[q] + e[q + 1] + 6u * E[q] + 4u * (o[q] + O[q]);
+        // rows r-4 .. r are output row (r - 4) / 2's (a sum is at most 16 * 16 * 255 + 128 < 2^16)
+        if (r >= 4 && r % 2 == 0) {
+            const int j = (r - 4) / 2, gy = PY * by + j;
+            uint32_t v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[q] = h[(r + 1) % 5][q] + h[r % 5][q] + 0x00800080u + 6u * h[(r + 3) % 5][q] +
+                       4u * (h[(r + 2) % 5][q] + h[(r + 4) % 5][q]);
+            // (columns from dW on lie in the pitch's padding)
+            if (active && gy < J.dH)
+                *reinterpret_cast<uint2*>(checked(J.dst + (size_t)gy * J.dp + PX * bx, 8, J.dst, (size_t)J.dp * J.dH, CK_PYR_DST)) =
+                    make_uint2(__byte_perm(v[0], v[1], 0x7531), __byte_perm(v[2], v[3], 0x7531));
+        }
+    }
 }
 
 namespace {
