@@ -640,11 +640,13 @@ __device__ __forceinline__ void linearize_point(const StreamDesc& D, const PassP
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
     if (!MIXED) {
         // 8x8 byte window, rows yb-3..yb+4, columns xb-3..xb+4: two aligned
-        // 8-byte loads per row, then a funnel shift to the window start.
+        // 8-byte loads per row, those that hold a byte of the row in use (12 of 16
+        // on average: every lane's load is a tag lookup of its own), then a funnel
+        // shift to the window start.
         float hsx = 0.0f, hsy = 0.0f;   // cached-Hessian form: the point's (sx, sy)
         const int xs = G.xb - 3;
         const int a8 = xs & ~7;
-        const int sh = (xs - a8) * 8;
+        const int off = xs - a8, sh = off * 8;
         const bool far = sh >= 32;
         const uint8_t* base = lv.img + (size_t)(G.yb - 3) * lv.pitch + a8;
         uint32_t rw[8][2];
@@ -653,7 +655,8 @@ __device__ __forceinline__ void linearize_point(const StreamDesc& D, const PassP
             const uint2* rp = checked(reinterpret_cast<const uint2*>(base + (size_t)r * lv.pitch), 2,
                                       reinterpret_cast<const uint2*>(lv.img), (size_t)lv.pitch * lv.H / 8,
                                       CK_IMAGE);
-            const uint2 w0 = __ldca(rp), w1 = __ldca(rp + 1);
+            const int lo = r < 4 ? 3 - r : r - 4, hi = 7 - lo;      // the row's columns of the pattern and its gradients
+            const uint2 w0 = off + lo < 8 ? __ldca(rp) : make_uint2(0u, 0u), w1 = off + hi >= 8 ? __ldca(rp + 1) : make_uint2(0u, 0u);
             const uint32_t v0 = far ? w0.y : w0.x, v1 = far ? w1.x : w0.y, v2 = far ? w1.y : w1.x;
             rw[r][0] = __funnelshift_r(v0, v1, sh);      // (by sh modulo 32)
             rw[r][1] = __funnelshift_r(v1, v2, sh);
