@@ -859,6 +859,64 @@ __device__ __forceinline__ void block_reduce(float (&acc)[kAccPad], float (*red)
     __syncthreads();
 }
 
+// f as a double, in integers: the conversion would hold the FP64 pipe for 64
+// cycles, as long as the addition that follows it.
+__device__ __forceinline__ double exact_double(float f)
+{
+    const unsigned u = __float_as_uint(f), sign = u & 0x80000000u;
+    unsigned m = u & 0x7fffffffu, off = 0x38000000u;           // exponent bias 1023 - 127
+    if (m >= 0x7f800000u) off = 0x70000000u;                   // infinities, NaN
+    if (m < 0x00800000u) {                                     // zero, subnormals: normalised
+        const int lz = m ? __clz((int)m) - 8 : 0;
+        off = m ? 0x38100000u - ((unsigned)lz << 20) : 0u;
+        m = (m << lz) & 0x7fffffu;
+    }
+    return __hiloint2double((int)(sign | ((m >> 3) + off)), (int)(m << 29));
+}
+
+// Sums of the blocks' partials [blocks][kAccPad] in FP64, by the last block (of
+// 128 threads) of a linearisation: 10 interleaved chains of 12 threads with four
+// sums each, eight loads in flight a thread.  Bound by the FP64 additions, 64
+// cycles each on the four pipes of the SM: 10.7k cycles for 157 blocks, 19.8k with
+// one chain per sum and a load at a time.
+template <int NSUM>
+__device__ __forceinline__ void sum_partials(const float* partials, unsigned blocks, double* out)
+{
+    constexpr int QUADS = kAccPad / 4, CHAINS = 128 / QUADS, AHEAD = 8;
+    __shared__ double red[CHAINS][kAccPad];
+    const int t = threadIdx.x, q = t % QUADS, chain = t / QUADS;
+    if (chain < CHAINS) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        for (unsigned b0 = chain; b0 < blocks; b0 += AHEAD * CHAINS) {
+            float4 v[AHEAD];
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k) {
+                const unsigned b = b0 + k * CHAINS;
+                v[k] = b < blocks ? __ldcg(reinterpret_cast<const float4*>(partials + (size_t)b * kAccPad) + q)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k) {
+                if (b0 + k * CHAINS < blocks) {
+                    s[0] += exact_double(v[k].x);
+                    s[1] += exact_double(v[k].y);
+                    s[2] += exact_double(v[k].z);
+                    s[3] += exact_double(v[k].w);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[chain][4 * q + i] = s[i];
+    }
+    __syncthreads();
+    if (t < NSUM) {
+        double s = red[0][t];
+#pragma unroll
+        for (int c = 1; c < CHAINS; ++c) s += red[c][t];
+        out[t] = s;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Solver tail, run by one warp of every CTA
 //

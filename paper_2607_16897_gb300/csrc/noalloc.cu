@@ -8,7 +8,7 @@
 // tracker there; this entry point needs none.
 //
 // The only memory it uses besides the caller's inputs and outputs is a
-// file-scope scratch array (block partial sums and the last-block ticket),
+// file-scope scratch array (block partial sums, group sums and tickets),
 // which every GPU that loads the library holds until the process exits.
 #include <cmath>
 #include <cstring>
@@ -22,10 +22,15 @@ namespace {
 constexpr int kNaThreads = 128;
 constexpr int kNaMaxBlocks = 512;
 constexpr int kNaMaxPoints = kNaThreads * kNaMaxBlocks;   // 65536 map points
-constexpr int kNaTicket = kNaMaxBlocks * kAccPad;         // index of the ticket word
-constexpr int kNaWords = kNaTicket + 64;
+constexpr int kNaGroup = 16;                              // blocks summed together
+constexpr int kNaGroups = kNaMaxBlocks / kNaGroup;
+constexpr int kNaTicket = kNaMaxBlocks * kAccPad;         // index of the ticket words: all groups', each group's
+constexpr int kNaSums = kNaTicket + 64;                   // index of the groups' sums (doubles)
+constexpr int kNaWords = kNaSums + 2 * kNaGroups * kAccPad;
+static_assert(kNaGroups < 64 && kNaSums % 2 == 0, "the tickets fit their words, the doubles are aligned");
 
-// block partial sums (floats) followed by the ticket counter (as unsigned)
+// block partial sums (floats), tickets (as unsigned; zero between calls: the last
+// block to take one sets it back), group sums (as doubles)
 static __device__ __align__(256) float g_noalloc_scratch[kNaWords];
 
 struct NaArgs {
@@ -38,14 +43,70 @@ struct NaArgs {
     float huber_k, zmin;
 };
 
-// Reference sample (same bilinear weights for all 8 pattern pixels).
-__device__ __forceinline__ float na_tap(const uint8_t* img, int pitch, int x, int y, float w00,
-                                        float w10, float w01, float w11)
-{
-    const uint8_t* t = img + (size_t)y * pitch + x;
-    return fmaf(w00, (float)t[0], fmaf(w10, (float)t[1], fmaf(w01, (float)t[pitch], w11 * (float)t[pitch + 1])));
-}
+// ROWS rows of 8 bytes from (x, y) of a W x H level whose address and pitch may
+// have any alignment: the aligned 8-byte words around them that hold a byte in
+// use, shifted.  `inside`: those words lie in the level (not so at its first and
+// last bytes; then the bytes themselves are read).  Row r is used from column
+// use(r) to 7 - use(r): the pattern, its bilinear taps and (8 rows) gradients.
+template <int ROWS>
+struct NaWindow {
+    const uint8_t* p;
+    int pitch;
+    bool inside;
+    uint2 w[ROWS][2];
 
+    static __device__ constexpr int use(int r)
+    {
+        return ROWS == 8 ? (r < 4 ? 3 - r : r - 4) : r < 3 ? 3 - r : r > 3 ? r - 2 : 1;
+    }
+    __device__ __forceinline__ NaWindow(const uint8_t* img, int pitch_, int W, int H, int x, int y)
+        : p(img + (size_t)y * pitch_ + x), pitch(pitch_),
+          inside(p - (reinterpret_cast<uintptr_t>(p) & 7u) >= img &&
+                 p + (size_t)(ROWS - 1) * pitch_ + 16 <= img + (size_t)(H - 1) * pitch_ + W)
+    {
+    }
+    __device__ __forceinline__ void load()
+    {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const uint8_t* q = p + (size_t)r * pitch;
+            const int a = (int)(reinterpret_cast<uintptr_t>(q) & 7u);
+            const uint2* b = reinterpret_cast<const uint2*>(q - a);
+            w[r][0] = a + use(r) < 8 ? __ldg(b) : make_uint2(0u, 0u);
+            w[r][1] = a + 7 - use(r) >= 8 ? __ldg(b + 1) : make_uint2(0u, 0u);
+        }
+    }
+    __device__ __forceinline__ void shift(uint32_t (&win)[ROWS][2]) const
+    {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const unsigned a = (unsigned)(reinterpret_cast<uintptr_t>(p + (size_t)r * pitch) & 7u);
+            const bool far = a >= 4;
+            const uint32_t v0 = far ? w[r][0].y : w[r][0].x, v1 = far ? w[r][1].x : w[r][0].y, v2 = far ? w[r][1].y : w[r][1].x;
+            win[r][0] = __funnelshift_r(v0, v1, 8 * a);      // (modulo 32)
+            win[r][1] = __funnelshift_r(v1, v2, 8 * a);
+        }
+    }
+    __device__ __forceinline__ void bytes(uint32_t (&win)[ROWS][2]) const
+    {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                uint32_t v = 0;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) v |= (uint32_t)__ldg(p + (size_t)r * pitch + 4 * i + b) << (8 * b);
+                win[r][i] = v;
+            }
+        }
+    }
+};
+
+// One point a thread.  Bound by a chain: the point, its two windows (4.5k cycles:
+// every lane's word is an L1 miss of its own; 9k one window after the other in
+// 4-byte words), the samples (2.3k), the block's reduction, and the sum over the
+// blocks below.  20000 points: 25 us with byte loads, a serial sum over the blocks
+// and a memset before the kernel, now 12.4 us (10.6 us of it the call on the host).
 __global__ void __launch_bounds__(kNaThreads)
     linearize_noalloc_kernel(NaArgs A, PassParams P, float* __restrict__ scratch,
                              double* __restrict__ out)
@@ -67,21 +128,17 @@ __global__ void __launch_bounds__(kNaThreads)
         d = A.uvd[3 * p + 2];
         ok = isfinite(u0) && isfinite(v0) && isfinite(d) && d > 0.0f && fabsf(u0) < 1e7f && fabsf(v0) < 1e7f;
     }
-    // reference patch I0 on this level
-    float i0[8];
+    // where the reference patch I0 lies on this level
+    int xr = 0, yr = 0;
+    float ral = 0.f, rbe = 0.f;
     if (ok) {
         const float U = u0 * s, V = v0 * s;
         const float fu = floorf(U), fv = floorf(V);
-        const int xr = (int)fu, yr = (int)fv;
+        xr = (int)fu;
+        yr = (int)fv;
         ok = xr >= 3 && xr <= A.W - 5 && yr >= 3 && yr <= A.H - 5;
-        if (ok) {
-            const float al = U - fu, be = V - fv;
-            const float w00 = (1.0f - al) * (1.0f - be), w10 = al * (1.0f - be);
-            const float w01 = (1.0f - al) * be, w11 = al * be;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                i0[k] = na_tap(A.ref, A.ref_pitch, xr + pat_dx(k), yr + pat_dy(k), w00, w10, w01, w11);
-        }
+        ral = U - fu;
+        rbe = V - fv;
     }
     // projection relative to the reference pixel (as in the tracker)
     PointGeom G;
@@ -124,40 +181,96 @@ __global__ void __launch_bounds__(kNaThreads)
         }
     }
     if (ok) {
+        // both windows in flight together
+        uint32_t rw[6][2], win[8][2];
+        {
+            NaWindow<6> R(A.ref, A.ref_pitch, A.W, A.H, xr - 3, yr - 2);
+            NaWindow<8> C(A.cur, A.cur_pitch, A.W, A.H, G.xb - 3, G.yb - 3);
+            if (R.inside && C.inside) {
+                R.load();
+                C.load();
+                R.shift(rw);
+                C.shift(win);
+            } else {
+                R.bytes(rw);
+                C.bytes(win);
+            }
+        }
+#define GLT_NA(w, r, c) u8f(w[(r)][(c) >> 2], (c) & 3)
+        float i0[8];
+        {
+            const float w00 = (1.0f - ral) * (1.0f - rbe), w10 = ral * (1.0f - rbe);
+            const float w01 = (1.0f - ral) * rbe, w11 = ral * rbe;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int r = pat_dy(k) + 2, c = pat_dx(k) + 3;
+                i0[k] = fmaf(w00, GLT_NA(rw, r, c),
+                             fmaf(w10, GLT_NA(rw, r, c + 1), fmaf(w01, GLT_NA(rw, r + 1, c), w11 * GLT_NA(rw, r + 1, c + 1))));
+            }
+        }
         const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
         const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const uint8_t* t = A.cur + (size_t)(G.yb + pat_dy(k)) * A.cur_pitch + (G.xb + pat_dx(k));
-            const int pc = A.cur_pitch;
-            const float I00 = t[0], I10 = t[1], I01 = t[pc], I11 = t[pc + 1];
+            const int r = pat_dy(k) + 3, c = pat_dx(k) + 3;
+            const float I00 = GLT_NA(win, r, c), I10 = GLT_NA(win, r, c + 1), I01 = GLT_NA(win, r + 1, c), I11 = GLT_NA(win, r + 1, c + 1);
             const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
-            const float gx = 0.5f * fmaf(w00, I10 - (float)t[-1],
-                                   fmaf(w10, (float)t[2] - I00,
-                                   fmaf(w01, I11 - (float)t[pc - 1], w11 * ((float)t[pc + 2] - I01))));
-            const float gy = 0.5f * fmaf(w00, I01 - (float)t[-pc],
-                                   fmaf(w10, I11 - (float)t[1 - pc],
-                                   fmaf(w01, (float)t[2 * pc] - I00, w11 * ((float)t[2 * pc + 1] - I10))));
+            const float gx = 0.5f * fmaf(w00, I10 - GLT_NA(win, r, c - 1),
+                                   fmaf(w10, GLT_NA(win, r, c + 2) - I00,
+                                   fmaf(w01, I11 - GLT_NA(win, r + 1, c - 1), w11 * (GLT_NA(win, r + 1, c + 2) - I01))));
+            const float gy = 0.5f * fmaf(w00, I01 - GLT_NA(win, r - 1, c),
+                                   fmaf(w10, I11 - GLT_NA(win, r - 1, c + 1),
+                                   fmaf(w01, GLT_NA(win, r + 2, c) - I00, w11 * (GLT_NA(win, r + 2, c + 1) - I10))));
             accumulate_sample(G, I, gx, gy, i0[k], P.ea, P.b, A.huber_k, acc, nullptr);
         }
+#undef GLT_NA
     }
     block_reduce<kNaThreads, false>(acc, red, part, nullptr);
     if (threadIdx.x < kNumAcc) scratch[(size_t)blockIdx.x * kAccPad + threadIdx.x] = part[threadIdx.x];
-    __threadfence();
-    __syncthreads();
+    // The sum over the blocks in FP64: a group's last block adds the group's,
+    // the last group's adds the groups'.  An addition holds an FP64 pipe for 64
+    // cycles, so one block summing all 157 of 20000 points took 10.7k cycles
+    // (19.8k with one chain per sum), half of the kernel.
+    __shared__ double odd[kAccPad];
     unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kNaTicket);
-    if (threadIdx.x == 0) is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (is_last) {
+    double* sums = reinterpret_cast<double*>(scratch + kNaSums);
+    const unsigned g = blockIdx.x / kNaGroup, groups = (gridDim.x + kNaGroup - 1) / kNaGroup;
+    const unsigned members = min((unsigned)kNaGroup, gridDim.x - g * kNaGroup);
+    const int chain = threadIdx.x / kAccPad, j = threadIdx.x % kAccPad;
+    auto last_of = [&](unsigned* t, unsigned n) {
         __threadfence();
-        if (threadIdx.x < kNumAcc) {
-            double acc_d = 0.0;
-            for (unsigned b = 0; b < gridDim.x; ++b)
-                acc_d += (double)__ldcg(scratch + (size_t)b * kAccPad + threadIdx.x);
-            out[threadIdx.x] = acc_d;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            is_last = atomicAdd(t, 1u) == n - 1;
+            if (is_last) *t = 0u;
         }
-        if (threadIdx.x == 0) *ticket = 0u;
+        __syncthreads();
+        __threadfence();
+        return is_last != 0;
+    };
+    if (!last_of(ticket + 1 + g, members)) return;
+    double sum = 0.0;
+    if (chain < 2 && j < kNumAcc) {
+        float v[kNaGroup / 2];
+#pragma unroll
+        for (int k = 0; k < kNaGroup / 2; ++k)
+            v[k] = 2 * k + chain < members ? __ldcg(scratch + (size_t)(g * kNaGroup + 2 * k + chain) * kAccPad + j) : 0.0f;
+#pragma unroll
+        for (int k = 0; k < kNaGroup / 2; ++k)
+            if (2 * k + chain < members) sum += exact_double(v[k]);
+        if (chain == 1) odd[j] = sum;
     }
+    __syncthreads();
+    if (chain == 0 && j < kNumAcc) sums[(size_t)g * kAccPad + j] = sum + odd[j];
+    if (!last_of(ticket, groups)) return;
+    sum = 0.0;
+    if (chain < 2 && j < kNumAcc) {
+#pragma unroll 8
+        for (unsigned b = chain; b < groups; b += 2) sum += __ldcg(sums + (size_t)b * kAccPad + j);
+        if (chain == 1) odd[j] = sum;
+    }
+    __syncthreads();
+    if (chain == 0 && j < kNumAcc) out[j] = sum + odd[j];
 }
 
 // Device address of the scratch array, looked up once per device and kept
@@ -224,12 +337,8 @@ extern "C" int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, cons
     int rc = na_scratch(&scratch);
     if (rc != GLT_OK) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // the ticket must start at zero (a previous call that was cut short
-    // could have left it non-zero)
-    cudaError_t e = cudaMemsetAsync(scratch + kNaTicket, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return cuda_fail(e, "glt_linearize_noalloc ticket reset");
     if (n == 0) {
-        e = cudaMemsetAsync(out_dev, 0, kNumAcc * sizeof(double), s);
+        const cudaError_t e = cudaMemsetAsync(out_dev, 0, kNumAcc * sizeof(double), s);
         return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_linearize_noalloc");
     }
     NaArgs A;
@@ -251,6 +360,6 @@ extern "C" int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, cons
     make_pass_params(T, a, b, level, P);
     const int blocks = (n + kNaThreads - 1) / kNaThreads;
     linearize_noalloc_kernel<<<blocks, kNaThreads, 0, s>>>(A, P, scratch, out_dev);
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_linearize_noalloc kernel");
 }

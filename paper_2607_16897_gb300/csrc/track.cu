@@ -415,12 +415,7 @@ __global__ void __launch_bounds__(THREADS) linearize_kernel(const StreamDesc* __
     __syncthreads();
     if (is_last) {
         __threadfence();
-        if (threadIdx.x < NSUM) {
-            double s = 0.0;
-            for (unsigned b = 0; b < gridDim.x; ++b)
-                s += (double)__ldcg(partials + (size_t)b * kAccPad + threadIdx.x);
-            out[threadIdx.x] = s;
-        }
+        sum_partials<NSUM>(partials, gridDim.x, out);
         if (threadIdx.x == 0) *counter = 0u;  // ready for the next launch
     }
 }
