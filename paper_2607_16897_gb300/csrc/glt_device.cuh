@@ -202,10 +202,11 @@ __device__ __forceinline__ size_t patch_index1(const StreamDesc& D, int level, i
 {
     return ((size_t)level * D.K + k) * D.Npad + p;
 }
+// tab + i, from where n elements are read
 template <class T>
-__device__ __forceinline__ T table_at(const StreamDesc& D, const T* tab, size_t i)
+__device__ __forceinline__ const T* table_from(const StreamDesc& D, const T* tab, size_t i, size_t n)
 {
-    return *checked(tab + i, 1, tab, table_size(D.L, D.Npad, D.pattern, D.tg), CK_TABLE);
+    return checked(tab + i, n, tab, table_size(D.L, D.Npad, D.pattern, D.tg), CK_TABLE);
 }
 
 __device__ __forceinline__ void load_point(const StreamDesc& D, int level, int p, PointCache& c)
@@ -215,7 +216,7 @@ __device__ __forceinline__ void load_point(const StreamDesc& D, int level, int p
     if (D.pattern) {
         // the p x p path reads its samples itself; the first marks validity
         const size_t at = ((size_t)level * group_samples(D.pattern, D.tg) * D.Npad + p) * D.tg;
-        c.ia = make_float4(table_at(D, D.I0, at), 0.f, 0.f, 0.f);
+        c.ia = make_float4(*table_from(D, D.I0, at, 1), 0.f, 0.f, 0.f);
         c.ib = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
         const float* I0b = checked(D.I0 + ((size_t)level * D.Npad + p) * 8, 8, D.I0, (size_t)D.L * D.Npad * 8, CK_TABLE);
@@ -401,6 +402,10 @@ __device__ __forceinline__ void linearize_square_t(const StreamDesc& D, const Pa
     }
 #define GLT_WX(r, c) u8f(win[(r)][(c) >> 2], (c) & 3)
     constexpr int TG = HC ? hc_groups(PS) : 1;
+    // the point's samples of the tables, all groups'
+    const size_t from = patch_index<PS, TG>(D, P.level, p, 0, 0), count = (size_t)(group_samples(PS, TG) - 1) * D.Npad * TG + TG;
+    const float* I0p = table_from(D, D.I0, from, count);
+    const float2* G0p = ICF ? table_from(D, D.G0, from, count) : nullptr;
     const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
 #pragma unroll
@@ -408,19 +413,19 @@ __device__ __forceinline__ void linearize_square_t(const StreamDesc& D, const Pa
 #pragma unroll
         for (int i = 0; i < PS; ++i) {
             const int r0 = j + B, c0 = i + B, k = j * PS + i;
-            const size_t at = patch_index<PS, TG>(D, P.level, p, j, i);
-            const float i0 = table_at(D, D.I0, at);
+            const size_t at = patch_index<PS, TG>(D, P.level, p, j, i) - from;
+            const float i0 = I0p[at];
             const float I00 = GLT_WX(r0, c0), I10 = GLT_WX(r0, c0 + 1);
             const float I01 = GLT_WX(r0 + 1, c0), I11 = GLT_WX(r0 + 1, c0 + 1);
             const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
             if (HC) {
-                hc_sample(I, i0, table_at(D, D.G0, at), P.ea, P.b, D.huber_k, sx, sy, acc,
+                hc_sample(I, i0, G0p[at], P.ea, P.b, D.huber_k, sx, sy, acc,
                           res ? res + (size_t)(PS * PS) * p + k : nullptr);
                 continue;
             }
             float gx, gy;
             if (ICF) {
-                const float2 g0 = table_at(D, D.G0, at);
+                const float2 g0 = G0p[at];
                 gx = P.ea * g0.x;
                 gy = P.ea * g0.y;
             } else {
@@ -454,9 +459,12 @@ __device__ __forceinline__ void linearize_square_any(const StreamDesc& D, const 
     if (ic) ic_geometry(D, P, p, G);
     const float w00 = (1.0f - G.al) * (1.0f - G.be), w10 = G.al * (1.0f - G.be);
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
+    const size_t from = patch_index1(D, P.level, p, 0), count = (size_t)(K - 1) * D.Npad + 1;
+    const float* I0p = table_from(D, D.I0, from, count);
+    const float2* G0p = HC || ic ? table_from(D, D.G0, from, count) : nullptr;
     for (int k = 0; k < K; ++k) {
-        const size_t at = patch_index1(D, P.level, p, k);
-        const float i0 = table_at(D, D.I0, at);
+        const size_t at = (size_t)k * D.Npad;
+        const float i0 = I0p[at];
         const int dx = k % D.pattern - h, dy = k / D.pattern - h;
         // taps t - S - 1 .. t + 2 S + 2 (intensity and central differences)
         const uint8_t* t = checked(lv.img + (size_t)(G.yb + dy - 1) * S + (G.xb + dx - 1), (size_t)3 * S + 4,
@@ -464,13 +472,13 @@ __device__ __forceinline__ void linearize_square_any(const StreamDesc& D, const 
         const float I00 = __ldca(t), I10 = __ldca(t + 1), I01 = __ldca(t + S), I11 = __ldca(t + S + 1);
         const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
         if (HC) {
-            hc_sample(I, i0, table_at(D, D.G0, at), P.ea, P.b, D.huber_k, sx, sy, acc,
+            hc_sample(I, i0, G0p[at], P.ea, P.b, D.huber_k, sx, sy, acc,
                       res ? res + (size_t)K * p + k : nullptr);
             continue;
         }
         float gx, gy;
         if (ic) {
-            const float2 g0 = table_at(D, D.G0, at);
+            const float2 g0 = G0p[at];
             gx = P.ea * g0.x;
             gy = P.ea * g0.y;
         } else {
@@ -555,6 +563,9 @@ __device__ __forceinline__ void linearize_rows_hc(const StreamDesc& D, const Pas
     const float w01 = (1.0f - G.al) * G.be, w11 = G.al * G.be;
     // this task's column of the tables: sample l of the group is l strides on
     const size_t stride = (size_t)D.Npad * TG, at0 = patch_index<PS, TG>(D, P.level, p, j0, 0);
+    const size_t count = (size_t)(min(RG, PS - j0) * PS - 1) * stride + 1;
+    const float* I0p = table_from(D, D.I0, at0, count);
+    const float2* G0p = table_from(D, D.G0, at0, count);
     float sx = 0.0f, sy = 0.0f;
     // UNIT: every residual is within the Huber threshold, so that the weight is 1
     // and the energy r^2 / 2 (hc_sample's operations without the two selects and
@@ -567,12 +578,12 @@ __device__ __forceinline__ void linearize_rows_hc(const StreamDesc& D, const Pas
             if (j0 + j < PS) {
 #pragma unroll
                 for (int i = 0; i < PS; ++i) {
-                    const size_t at = at0 + (j * PS + i) * stride;
+                    const size_t at = (j * PS + i) * stride;
                     const float I00 = GLT_WR(j, i), I10 = GLT_WR(j, i + 1);
                     const float I01 = GLT_WR(j + 1, i), I11 = GLT_WR(j + 1, i + 1);
                     const float I = fmaf(w00, I00, fmaf(w10, I10, fmaf(w01, I01, w11 * I11)));
-                    const float i0 = table_at(D, D.I0, at);
-                    const float2 g0 = table_at(D, D.G0, at);
+                    const float i0 = I0p[at];
+                    const float2 g0 = G0p[at];
                     if (UNIT) {
                         const float r = __fsub_rn(fmaf(-P.ea, i0, I), P.b);
                         sx = fmaf(r, g0.x, sx);

@@ -43,27 +43,29 @@ __device__ __forceinline__ RefPoint ref_point(const LevelDev& lv, float u0, floa
     return r;
 }
 
+// tab + i, where n elements are written; null without a table
 template <class T>
-__device__ __forceinline__ void table_put(const StreamDesc& D, T* tab, size_t i, T v)
+__device__ __forceinline__ T* table_to(const StreamDesc& D, T* tab, size_t i, size_t n)
 {
-    *checked(tab + i, 1, tab, table_size(D.L, D.Npad, D.pattern, D.tg), CK_SET_POINTS) = v;
+    return tab ? checked(tab + i, n, tab, table_size(D.L, D.Npad, D.pattern, D.tg), CK_SET_POINTS) : nullptr;
 }
 
 // The 8-pixel pattern of one point on one level.
 __device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint& r, const uint8_t* img, int P, int l, int p,
                                              float* I0, float2* G0)
 {
-    const size_t at = ((size_t)l * D.Npad + p) * 8;
+    I0 = table_to(D, I0, ((size_t)l * D.Npad + p) * 8, 8);
+    G0 = table_to(D, G0, ((size_t)l * D.Npad + p) * 8, 8);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         if (!r.ok) {
-            table_put(D, I0, at + k, k == 0 ? __int_as_float(0x7fc00000) : 0.0f);
-            if (G0) table_put(D, G0, at + k, make_float2(0.0f, 0.0f));
+            I0[k] = k == 0 ? __int_as_float(0x7fc00000) : 0.0f;
+            if (G0) G0[k] = make_float2(0.0f, 0.0f);
             continue;
         }
         const uint8_t* t = img + (size_t)(r.yb + pat_dy(k)) * P + (r.xb + pat_dx(k));
         const float I00 = t[0], I10 = t[1], I01 = t[P], I11 = t[P + 1];
-        table_put(D, I0, at + k, fmaf(r.w00, I00, fmaf(r.w10, I10, fmaf(r.w01, I01, r.w11 * I11))));
+        I0[k] = fmaf(r.w00, I00, fmaf(r.w10, I10, fmaf(r.w01, I01, r.w11 * I11)));
         if (G0) {
             // central differences at the four taps, bilinear weights, then the 1/2
             const float gx = 0.5f * fmaf(r.w00, I10 - (float)t[-1],
@@ -72,7 +74,7 @@ __device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint
             const float gy = 0.5f * fmaf(r.w00, I01 - (float)t[-P],
                                     fmaf(r.w10, I11 - (float)t[1 - P],
                                     fmaf(r.w01, (float)t[2 * P] - I00, r.w11 * ((float)t[2 * P + 1] - I10))));
-            table_put(D, G0, at + k, make_float2(gx, gy));
+            G0[k] = make_float2(gx, gy);
         }
     }
 }
@@ -88,12 +90,14 @@ __device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r
     constexpr int h = (PS - 1) / 2, RG = group_rows(PS, TG), R = RG + 3, NB = PS + 3, NW = (NB + 3) / 4;
     const int j0 = g * RG, rows = min(RG, PS - j0);
     const size_t stride = (size_t)D.Npad * TG, at0 = ((size_t)l * group_samples(PS, TG)) * stride + (size_t)p * TG + g;
+    I0 = table_to(D, I0, at0, (size_t)(rows * PS - 1) * stride + 1);
+    G0 = table_to(D, G0, at0, (size_t)(rows * PS - 1) * stride + 1);
     if (!r.ok) {
 #pragma unroll
         for (int q = 0; q < RG * PS; ++q) {
             if (q >= rows * PS) break;
-            table_put(D, I0, at0 + q * stride, q == 0 && g == 0 ? __int_as_float(0x7fc00000) : 0.0f);
-            if (G0) table_put(D, G0, at0 + q * stride, make_float2(0.0f, 0.0f));
+            I0[q * stride] = q == 0 && g == 0 ? __int_as_float(0x7fc00000) : 0.0f;
+            if (G0) G0[q * stride] = make_float2(0.0f, 0.0f);
         }
         return;
     }
@@ -121,9 +125,9 @@ __device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r
 #pragma unroll
         for (int i = 0; i < PS; ++i) {
             const int y = j + 1, x = i + 1;
-            const size_t at = at0 + (j * PS + i) * stride;
+            const size_t at = (j * PS + i) * stride;
             const float I00 = px(y, x), I10 = px(y, x + 1), I01 = px(y + 1, x), I11 = px(y + 1, x + 1);
-            table_put(D, I0, at, fmaf(r.w00, I00, fmaf(r.w10, I10, fmaf(r.w01, I01, r.w11 * I11))));
+            I0[at] = fmaf(r.w00, I00, fmaf(r.w10, I10, fmaf(r.w01, I01, r.w11 * I11)));
             if (G0) {
                 const float gx = 0.5f * fmaf(r.w00, I10 - px(y, x - 1),
                                         fmaf(r.w10, px(y, x + 2) - I00,
@@ -131,7 +135,7 @@ __device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r
                 const float gy = 0.5f * fmaf(r.w00, I01 - px(y - 1, x),
                                         fmaf(r.w10, I11 - px(y - 1, x + 1),
                                         fmaf(r.w01, px(y + 2, x) - I00, r.w11 * (px(y + 2, x + 1) - I10))));
-                table_put(D, G0, at, make_float2(gx, gy));
+                G0[at] = make_float2(gx, gy);
             }
         }
     }
