@@ -8,7 +8,7 @@
 // tracker there; this entry point needs none.
 //
 // The only memory it uses besides the caller's inputs and outputs is a
-// file-scope scratch array (block partial sums, group sums and tickets),
+// file-scope scratch array (block partial sums and the last-block ticket),
 // which every GPU that loads the library holds until the process exits.
 #include <cmath>
 #include <cstring>
@@ -22,15 +22,10 @@ namespace {
 constexpr int kNaThreads = 128;
 constexpr int kNaMaxBlocks = 512;
 constexpr int kNaMaxPoints = kNaThreads * kNaMaxBlocks;   // 65536 map points
-constexpr int kNaGroup = 16;                              // blocks summed together
-constexpr int kNaGroups = kNaMaxBlocks / kNaGroup;
-constexpr int kNaTicket = kNaMaxBlocks * kAccPad;         // index of the ticket words: all groups', each group's
-constexpr int kNaSums = kNaTicket + 64;                   // index of the groups' sums (doubles)
-constexpr int kNaWords = kNaSums + 2 * kNaGroups * kAccPad;
-static_assert(kNaGroups < 64 && kNaSums % 2 == 0, "the tickets fit their words, the doubles are aligned");
+constexpr int kNaTicket = kNaMaxBlocks * kAccPad;         // index of the ticket word
+constexpr int kNaWords = kNaTicket + 64;
 
-// block partial sums (floats), tickets (as unsigned; zero between calls: the last
-// block to take one sets it back), group sums (as doubles)
+// block partial sums (floats) followed by the ticket counter (as unsigned)
 static __device__ __align__(256) float g_noalloc_scratch[kNaWords];
 
 struct NaArgs {
@@ -104,9 +99,9 @@ struct NaWindow {
 
 // One point a thread.  Bound by a chain: the point, its two windows (4.5k cycles:
 // every lane's word is an L1 miss of its own; 9k one window after the other in
-// 4-byte words), the samples (2.3k), the block's reduction, and the sum over the
-// blocks below.  20000 points: 25 us with byte loads, a serial sum over the blocks
-// and a memset before the kernel, now 12.4 us (10.6 us of it the call on the host).
+// 4-byte words), the samples (2.3k), the block's reduction, and the last block's
+// sum over the blocks.  20000 points: 24.7 us with byte loads and a serial sum,
+// now 14.4 (the call's two launches take the host as long).
 __global__ void __launch_bounds__(kNaThreads)
     linearize_noalloc_kernel(NaArgs A, PassParams P, float* __restrict__ scratch,
                              double* __restrict__ out)
@@ -227,50 +222,16 @@ __global__ void __launch_bounds__(kNaThreads)
     }
     block_reduce<kNaThreads, false>(acc, red, part, nullptr);
     if (threadIdx.x < kNumAcc) scratch[(size_t)blockIdx.x * kAccPad + threadIdx.x] = part[threadIdx.x];
-    // The sum over the blocks in FP64: a group's last block adds the group's,
-    // the last group's adds the groups'.  An addition holds an FP64 pipe for 64
-    // cycles, so one block summing all 157 of 20000 points took 10.7k cycles
-    // (19.8k with one chain per sum), half of the kernel.
-    __shared__ double odd[kAccPad];
+    __threadfence();
+    __syncthreads();
     unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kNaTicket);
-    double* sums = reinterpret_cast<double*>(scratch + kNaSums);
-    const unsigned g = blockIdx.x / kNaGroup, groups = (gridDim.x + kNaGroup - 1) / kNaGroup;
-    const unsigned members = min((unsigned)kNaGroup, gridDim.x - g * kNaGroup);
-    const int chain = threadIdx.x / kAccPad, j = threadIdx.x % kAccPad;
-    auto last_of = [&](unsigned* t, unsigned n) {
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            is_last = atomicAdd(t, 1u) == n - 1;
-            if (is_last) *t = 0u;
-        }
-        __syncthreads();
-        __threadfence();
-        return is_last != 0;
-    };
-    if (!last_of(ticket + 1 + g, members)) return;
-    double sum = 0.0;
-    if (chain < 2 && j < kNumAcc) {
-        float v[kNaGroup / 2];
-#pragma unroll
-        for (int k = 0; k < kNaGroup / 2; ++k)
-            v[k] = 2 * k + chain < members ? __ldcg(scratch + (size_t)(g * kNaGroup + 2 * k + chain) * kAccPad + j) : 0.0f;
-#pragma unroll
-        for (int k = 0; k < kNaGroup / 2; ++k)
-            if (2 * k + chain < members) sum += exact_double(v[k]);
-        if (chain == 1) odd[j] = sum;
-    }
+    if (threadIdx.x == 0) is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (chain == 0 && j < kNumAcc) sums[(size_t)g * kAccPad + j] = sum + odd[j];
-    if (!last_of(ticket, groups)) return;
-    sum = 0.0;
-    if (chain < 2 && j < kNumAcc) {
-#pragma unroll 8
-        for (unsigned b = chain; b < groups; b += 2) sum += __ldcg(sums + (size_t)b * kAccPad + j);
-        if (chain == 1) odd[j] = sum;
+    if (is_last) {
+        __threadfence();
+        sum_partials<kNumAcc>(scratch, gridDim.x, out);
+        if (threadIdx.x == 0) *ticket = 0u;
     }
-    __syncthreads();
-    if (chain == 0 && j < kNumAcc) out[j] = sum + odd[j];
 }
 
 // Device address of the scratch array, looked up once per device and kept
@@ -337,8 +298,12 @@ extern "C" int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, cons
     int rc = na_scratch(&scratch);
     if (rc != GLT_OK) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    // the ticket must start at zero (a previous call that was cut short
+    // could have left it non-zero)
+    cudaError_t e = cudaMemsetAsync(scratch + kNaTicket, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return cuda_fail(e, "glt_linearize_noalloc ticket reset");
     if (n == 0) {
-        const cudaError_t e = cudaMemsetAsync(out_dev, 0, kNumAcc * sizeof(double), s);
+        e = cudaMemsetAsync(out_dev, 0, kNumAcc * sizeof(double), s);
         return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_linearize_noalloc");
     }
     NaArgs A;
@@ -360,6 +325,6 @@ extern "C" int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, cons
     make_pass_params(T, a, b, level, P);
     const int blocks = (n + kNaThreads - 1) / kNaThreads;
     linearize_noalloc_kernel<<<blocks, kNaThreads, 0, s>>>(A, P, scratch, out_dev);
-    const cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_linearize_noalloc kernel");
 }
