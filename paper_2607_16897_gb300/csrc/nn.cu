@@ -1256,7 +1256,7 @@ namespace nn {
 // layer's weights in the [K][O] layout (a tile's 4 weights are one 8-byte
 // load), copied into shared memory with asynchronous 16-byte copies issued at
 // the start and awaited just before conv2.  The sum order per output (bias,
-// then channel, row, column) is that of conv_fwd.
+// then channel, row, column) is that of conv_forward.
 constexpr int kPropThreads = 512;
 constexpr int kXp = 32 * 42, kA1p = 16 * 17 * 22, kA2p = 32 * 10 * 12;
 constexpr int kPropSmemFloats = kXp + kA1p + kA2p + (kF + 2) + kHid + kOut;
@@ -1443,7 +1443,7 @@ __device__ void motion_feature(const double* __restrict__ M, float* __restrict__
 // stream of its cluster, from the streams' feature vectors copied out of the
 // peers' shared memory, and writes each result into its stream's block, so
 // the 329 KB of fc1 weights are read from L2 once per cluster instead of once
-// per stream.  Each output keeps conv_fwd's lane split and reduction order.
+// per stream.  Each output keeps its lane split and reduction order.
 constexpr int kPropCluster = 4;
 static_assert(kHid % (kPropCluster * (kPropThreads / 32)) == 0, "whole rows per warp");
 static_assert(kPropCluster * (kF + 2) <= kA1p, "the peers' feature vectors fit where conv1's output was");
