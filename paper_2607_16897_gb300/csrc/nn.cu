@@ -1203,17 +1203,25 @@ cudaError_t launch_fc_forward(const glt_nn* n, const float* mo, int B, float* y,
                               (const __nv_bfloat16*)n->wt, B, y, t, n->h, n->dy, n->dh, n->loss_b);
 }
 
+// The status of a call's launches so far: `e`, that of the last one, or the
+// error an earlier `<<<>>>` left (none is left for a later call either way).
+cudaError_t launches_status(cudaError_t e)
+{
+    const cudaError_t earlier = cudaGetLastError();
+    return e != cudaSuccess ? e : earlier;
+}
+
 cudaError_t nn_forward(const glt_nn* n, const float* x, const float* mo, int B, float* y, cudaStream_t s)
 {
     launch_conv_forward<false>(n, x, B, s);
-    return launch_fc_forward<false>(n, mo, B, y, nullptr, s);
+    return launches_status(launch_fc_forward<false>(n, mo, B, y, nullptr, s));
 }
 
 // forward and backward: the gradient sums up to adam_update, which completes them
 cudaError_t nn_backward(const glt_nn* n, const float* x, const float* mo, const float* t, int B, cudaStream_t s)
 {
     launch_conv_forward<true>(n, x, B, s);
-    const cudaError_t e = launch_fc_forward<true>(n, mo, B, n->y, t, s);
+    const cudaError_t e = launches_status(launch_fc_forward<true>(n, mo, B, n->y, t, s));
     if (e != cudaSuccess) return e;
     fc1_input_grad<<<dim3(grid_for(B, kFcS), kFlat / kD3Threads), kD3Threads, kD3Smem, s>>>(n->dh, n->wt, n->a3, B, n->d3);
     fc_weight_grad<<<kGwBlocks, kGwThreads, kGwSmem, s>>>(n->dh, n->dy, n->a3, mo, n->h, B, n->g);
