@@ -1230,6 +1230,8 @@ cudaError_t nn_backward(const glt_nn* n, const float* x, const float* mo, const 
     return cudaGetLastError();
 }
 
+bool unaligned(const float* p) { return (reinterpret_cast<uintptr_t>(p) & (alignof(float) - 1)) != 0; }
+
 int check_batch(const glt_nn* n, int B)
 {
     if (!n) return invalid_arg_msg("network is NULL");
@@ -1753,12 +1755,14 @@ int glt_nn_forward(glt_nn* n, const float* x_dev, const float* m_dev, float* y_d
     if (rc != GLT_OK) return rc;
     if (!x_dev || !m_dev || !y_dev) return invalid_arg_msg("NULL argument");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // an output that overlaps an input is written when all inputs have been read
+    // an output that overlaps an input is written when all inputs have been
+    // read; one that no kernel can store to (its address is no multiple of 4) by
+    // a copy
     auto overlap = [&](const float* p, size_t len) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(y_dev);
         return a < b + (size_t)B * kOut * sizeof(float) && b < a + len * sizeof(float);
     };
-    const bool staged = overlap(x_dev, (size_t)B * kIn) || overlap(m_dev, (size_t)B * kMotion);
+    const bool staged = unaligned(y_dev) || overlap(x_dev, (size_t)B * kIn) || overlap(m_dev, (size_t)B * kMotion);
     cudaError_t e = nn_forward(n, x_dev, m_dev, B, staged ? n->y : y_dev, s);
     if (e == cudaSuccess && staged)
         e = cudaMemcpyAsync(y_dev, n->y, (size_t)B * kOut * sizeof(float), cudaMemcpyDeviceToDevice, s);
@@ -1795,13 +1799,15 @@ int glt_nn_train_step(glt_nn* n, const float* x_dev, const float* m_dev, const f
     cudaError_t e = nn_backward(n, x_dev, m_dev, t_dev, B, s);
     if (e != cudaSuccess) return cuda_fail(e, "glt_nn_train_step");
     n->step += 1;
+    float* const loss = loss_dev && !unaligned(loss_dev) ? loss_dev : n->loss;
     const double b1 = 0.9, b2 = 0.999;
     const float c1 = (float)(1.0 / (1.0 - std::pow(b1, n->step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(b2, n->step)));
     adam_update<true><<<kAdBlocks, 256, 0, s>>>(n->w, n->wbf, n->wt, n->g, n->part, std::min(B, kBwBlocks), n->m, n->v, lr,
-                                                (float)b1, (float)b2, 1e-8f, c1, c2, n->loss_b, B,
-                                                loss_dev ? loss_dev : n->loss);
-    if (e == cudaSuccess) e = cudaGetLastError();
+                                                (float)b1, (float)b2, 1e-8f, c1, c2, n->loss_b, B, loss);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && loss_dev && loss != loss_dev)
+        e = cudaMemcpyAsync(loss_dev, loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_nn_train_step");
 }
 

@@ -2,7 +2,8 @@
 stand-in for the CUDA runtime (preloaded in a child process) keeps "device"
 memory on the host, runs no kernel and refuses the launch it is told to.
 Every call must report the refused launch, whichever it is, and leave no error
-behind for the next call."""
+behind for the next call; an output at an address that no kernel can store a
+float to is written by a copy."""
 import os
 import subprocess
 import sys
@@ -17,6 +18,10 @@ FAKE = r"""
 typedef int err;                     /* cudaError_t: 0 success, 719 launch failure */
 typedef struct { unsigned x, y, z; } dim3_;
 static int refuse = -1, seen = 0, last = 0;
+static const void *odd = 0;          /* an address only copies may write */
+static int copied = 0;
+void fake_watch(const void *p) { odd = p; copied = 0; }
+int fake_copied(void) { return copied; }
 void fake_refuse(int k) { refuse = k; seen = 0; }
 int fake_launches(void) { return seen; }
 /* the error of the launch, which the runtime keeps until it is asked for */
@@ -26,7 +31,7 @@ err cudaFree(void *p) { free(p); return 0; }
 err cudaMemset(void *p, int v, size_t n) { memset(p, v, n); return 0; }
 err cudaMemcpy(void *d, const void *s, size_t n, int k) { (void)k; memcpy(d, s, n); return 0; }
 err cudaMemcpyAsync(void *d, const void *s, size_t n, int k, void *st)
-{ (void)k; (void)st; memcpy(d, s, n); return 0; }
+{ (void)k; (void)st; if (d == odd) copied = 1; memcpy(d, s, n); return 0; }
 err cudaGetDevice(int *d) { *d = 0; return 0; }
 err cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
 err cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
@@ -52,7 +57,8 @@ sys.path.insert(0, ".")
 import paper_2607_16897_gb300 as glt
 
 fake = ctypes.CDLL(sys.argv[1])
-B = int(sys.argv[2])
+fake.fake_watch.argtypes = [ctypes.c_void_p]
+B, mode = int(sys.argv[2]), sys.argv[3]
 net = glt.NN(B, np.zeros(glt.GLT_NN_PARAMS, np.float32))
 x, m, t, y = (np.zeros((B, k), np.float32) for k in (1200, 6, 8, 8))
 p = [a.ctypes.data for a in (x, m, t, y)]
@@ -60,7 +66,7 @@ loss = np.zeros(2, np.float32)
 calls = {"forward": lambda: net.forward(p[0], p[1], p[3], B, stream=0),
          "gradient": lambda: net.gradient(p[0], p[1], p[2], B, stream=0),
          "train_step": lambda: net.train_step(p[0], p[1], p[2], B, 1e-3, loss.ctypes.data, stream=0)}
-for name, call in calls.items():
+for name, call in calls.items() if mode == "launches" else ():
     fake.fake_refuse(-1)
     call()
     n = fake.fake_launches()
@@ -78,12 +84,20 @@ for name, call in calls.items():
         except glt.GltError as e:
             print("error left behind by", name, "launch", k, "of", n)
             fake.cudaGetLastError()
+raw = np.zeros(B * 8 * 4 + 8, np.uint8)
+for off in (0, 1, 2, 3) if mode == "addresses" else ():
+    a = (raw.ctypes.data + 3) // 4 * 4 + off
+    for name, call in (("forward", lambda: net.forward(p[0], p[1], a, B, stream=0)),
+                       ("train_step", lambda: net.train_step(p[0], p[1], p[2], B, 1e-3, a, stream=0))):
+        fake.fake_watch(a)
+        call()
+        if off and not fake.fake_copied():
+            print("a kernel stores the output of", name, "at offset", off)
 print("done")
 """
 
 
-@pytest.mark.parametrize("B", [5, 2100])
-def test_refused_launches_are_reported(tmp_path, B):
+def run_child(tmp_path, B, mode):
     import importlib.util
     spec = importlib.util.spec_from_file_location("_glt_build", os.path.join(ROOT, "paper_2607_16897_gb300", "build.py"))
     mod = importlib.util.module_from_spec(spec)
@@ -94,5 +108,16 @@ def test_refused_launches_are_reported(tmp_path, B):
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-o", lib, str(src)], check=True)
     env = dict(os.environ, LD_PRELOAD=lib)
     env.pop("GLT_LIBRARY", None)
-    r = subprocess.run([sys.executable, "-c", CHILD, lib, str(B)], cwd=ROOT, env=env, capture_output=True, text=True, timeout=300)
+    r = subprocess.run([sys.executable, "-c", CHILD, lib, str(B), mode], cwd=ROOT, env=env, capture_output=True, text=True,
+                       timeout=300)
     assert r.returncode == 0 and r.stdout.split("\n")[:-1] == ["done"], r.stdout + r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("B", [5, 2100])
+def test_refused_launches_are_reported(tmp_path, B):
+    run_child(tmp_path, B, "launches")
+
+
+@pytest.mark.parametrize("B", [5, 2100])
+def test_outputs_at_any_address(tmp_path, B):
+    run_child(tmp_path, B, "addresses")
