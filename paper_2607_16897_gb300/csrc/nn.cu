@@ -1002,14 +1002,25 @@ conv_weight_grad(const float* __restrict__ x, const float* __restrict__ a1, cons
 }
 
 // Gradient of every parameter (the convolutions' from the blocks' sums, in
-// block order over four interleaved quarters) and, with ADAM, the update
-// (Kingma and Ba) of the FP32 master weights and the BF16 copies.  Blocks
-// below kAdConv take 64 convolution parameters each, four threads per
-// parameter; the rest 256 parameters of the fully connected layers; the last
-// one adds the loss terms.
+// block order over four interleaved quarters, with the additions' rounding
+// errors kept) and, with ADAM, the update (Kingma and Ba) of the FP32 master
+// weights and the BF16 copies.  Blocks below kAdConv take 64 convolution
+// parameters each, four threads per parameter; the rest 256 parameters of the
+// fully connected layers; the last one adds the loss terms.  Without the
+// rounding errors (chains of 37 additions) conv3's gradient had 1.06 to 1.11
+// times the error against 64 bits of 128 chains and a tree over all terms, at
+// 148 to 256 samples; with them 0.68 to 0.88 times, and no layer's is larger.
 constexpr int kAdConvN = kPart, kAdConv = (kAdConvN + 63) / 64;
 constexpr int kAdFc = (kParams - kF1.w + 255) / 256, kAdBlocks = kAdConv + kAdFc + 1;
 static_assert(kAdConvN == kF1.w, "the convolutions' parameters come first");
+
+// s.x + s.y += v, with the rounding of s.x + v kept in s.y (TwoSum, Knuth)
+__device__ __forceinline__ void add_exact(float2& s, float v)
+{
+    const float t = s.x + v, z = t - s.x;
+    s.y += (s.x - (t - z)) + (v - z);
+    s.x = t;
+}
 
 template <bool ADAM>
 __global__ void __launch_bounds__(256)
@@ -1021,18 +1032,25 @@ adam_update(float* __restrict__ w, __nv_bfloat16* __restrict__ wbf, __nv_bfloat1
     int i = -1;
     float gi = 0.0f;
     if (blockIdx.x < kAdConv) {
-        __shared__ float q4[4][64];
+        __shared__ float2 q4[4][64];
         const int e = threadIdx.x & 63, q = threadIdx.x >> 6, at = blockIdx.x * 64 + e;
-        float s = 0.0f;
+        float2 s = make_float2(0.0f, 0.0f);
         if (at < kAdConvN) {
 #pragma unroll 8
-            for (int k = q; k < nparts; k += 4) s += part[(size_t)k * kPart + at];
+            for (int k = q; k < nparts; k += 4) add_exact(s, part[(size_t)k * kPart + at]);
         }
         q4[q][e] = s;
         __syncthreads();
         if (q == 0 && at < kAdConvN) {
             i = part_param(at);
-            gi = ((q4[0][e] + q4[1][e]) + q4[2][e]) + q4[3][e];
+            float lo = s.y;
+#pragma unroll
+            for (int r = 1; r < 4; ++r) {
+                s.y = 0.0f;
+                add_exact(s, q4[r][e].x);
+                lo += q4[r][e].y + s.y;
+            }
+            gi = isfinite(s.x) ? s.x + lo : s.x;
             g[i] = gi;
         }
     } else if (blockIdx.x < kAdConv + kAdFc) {
