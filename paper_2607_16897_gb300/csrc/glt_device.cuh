@@ -885,15 +885,19 @@ __device__ __forceinline__ double exact_double(float f)
     return __hiloint2double((int)(sign | ((m >> 3) + off)), (int)(m << 29));
 }
 
-// Sums of the blocks' partials [blocks][kAccPad] in FP64, by the last block (of
-// 128 threads) of a linearisation: 10 interleaved chains of 12 threads with four
-// sums each, eight loads in flight a thread.  Bound by the FP64 additions, 64
-// cycles each on the four pipes of the SM: 10.7k cycles for 157 blocks, 19.8k with
-// one chain per sum and a load at a time.
-template <int NSUM>
+// Sums of the blocks' partials [blocks][kAccPad] in FP64, by the last block of a
+// linearisation: 10 interleaved chains of sum_cols(NSUM) / 4 threads with four
+// sums each, eight loads in flight a thread.  A block stores sum_cols(NSUM)
+// columns, zeros beyond its NSUM sums.  Bound by the FP64 additions, 64 cycles
+// each on the four pipes of the SM: 10.7k cycles for 46 sums of 157 blocks, 19.8k
+// with one chain per sum and a load at a time.
+__host__ __device__ constexpr int sum_cols(int nsum) { return (nsum + 3) / 4 * 4; }
+
+template <int NSUM, int THREADS>
 __device__ __forceinline__ void sum_partials(const float* partials, unsigned blocks, double* out)
 {
-    constexpr int QUADS = kAccPad / 4, CHAINS = 128 / QUADS, AHEAD = 8;
+    constexpr int QUADS = sum_cols(NSUM) / 4, CHAINS = 10, AHEAD = 8;
+    static_assert(QUADS * CHAINS <= THREADS && NSUM <= THREADS && sum_cols(NSUM) <= kAccPad, "a thread per quad of a chain and per sum");
     __shared__ double red[CHAINS][kAccPad];
     const int t = threadIdx.x, q = t % QUADS, chain = t / QUADS;
     if (chain < CHAINS) {
@@ -908,12 +912,11 @@ __device__ __forceinline__ void sum_partials(const float* partials, unsigned blo
             }
 #pragma unroll
             for (int k = 0; k < AHEAD; ++k) {
-                if (b0 + k * CHAINS < blocks) {
-                    s[0] += exact_double(v[k].x);
-                    s[1] += exact_double(v[k].y);
-                    s[2] += exact_double(v[k].z);
-                    s[3] += exact_double(v[k].w);
-                }
+                if (b0 + k * CHAINS >= blocks) break;
+                s[0] += exact_double(v[k].x);
+                s[1] += exact_double(v[k].y);
+                s[2] += exact_double(v[k].z);
+                s[3] += exact_double(v[k].w);
             }
         }
 #pragma unroll
@@ -922,8 +925,7 @@ __device__ __forceinline__ void sum_partials(const float* partials, unsigned blo
     __syncthreads();
     if (t < NSUM) {
         double s = red[0][t];
-#pragma unroll
-        for (int c = 1; c < CHAINS; ++c) s += red[c][t];
+        for (unsigned c = 1; c < CHAINS && c < blocks; ++c) s += red[c][t];
         out[t] = s;
     }
 }

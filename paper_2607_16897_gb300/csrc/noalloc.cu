@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(kNaThreads)
 #undef GLT_NA
     }
     block_reduce<kNaThreads, false>(acc, red, part, nullptr);
-    if (threadIdx.x < kNumAcc) scratch[(size_t)blockIdx.x * kAccPad + threadIdx.x] = part[threadIdx.x];
+    if (threadIdx.x < sum_cols(kNumAcc))
+        scratch[(size_t)blockIdx.x * kAccPad + threadIdx.x] = threadIdx.x < kNumAcc ? part[threadIdx.x] : 0.0f;
     __threadfence();
     __syncthreads();
     unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kNaTicket);
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(kNaThreads)
     __syncthreads();
     if (is_last) {
         __threadfence();
-        sum_partials<kNumAcc>(scratch, gridDim.x, out);
+        sum_partials<kNumAcc, kNaThreads>(scratch, gridDim.x, out);
         if (threadIdx.x == 0) *ticket = 0u;
     }
 }

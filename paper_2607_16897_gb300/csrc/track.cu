@@ -372,8 +372,8 @@ __global__ void __launch_bounds__(THREADS, 1) pass_floor_kernel(int passes, int 
 }
 
 // One linearisation pass over all points of one tracker, many blocks, with a
-// single-pass finish: each block writes its 46 sums, the last block to arrive
-// (ticket counter) adds the block sums in block order in FP64.
+// single-pass finish: each block writes its 46 (cached Hessian: 8) sums, the last
+// block to arrive (ticket counter) adds the block sums in FP64 (sum_partials).
 template <int THREADS, int VAR>
 __global__ void __launch_bounds__(THREADS) linearize_kernel(const StreamDesc* __restrict__ desc,
                                                             PassParams P,
@@ -407,15 +407,16 @@ __global__ void __launch_bounds__(THREADS) linearize_kernel(const StreamDesc* __
         block_reduce8<THREADS>(acc, red, part);
     else
         block_reduce<THREADS, MIXED>(acc, red, part, part_c);
-    if (threadIdx.x < NSUM)
-        partials[(size_t)blockIdx.x * kAccPad + threadIdx.x] = part[threadIdx.x] + (MIXED ? part_c[threadIdx.x] : 0.0f);
+    if (threadIdx.x < sum_cols(NSUM))
+        partials[(size_t)blockIdx.x * kAccPad + threadIdx.x] =
+            threadIdx.x < NSUM ? part[threadIdx.x] + (MIXED ? part_c[threadIdx.x] : 0.0f) : 0.0f;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
     __syncthreads();
     if (is_last) {
         __threadfence();
-        sum_partials<NSUM>(partials, gridDim.x, out);
+        sum_partials<NSUM, THREADS>(partials, gridDim.x, out);
         if (threadIdx.x == 0) *counter = 0u;  // ready for the next launch
     }
 }
