@@ -376,9 +376,11 @@ int glt_debug_checked_flags(unsigned* flags);
 /* Positive control of the bounds-checked build: a one-thread kernel reads
  * one element inside a 64-float device buffer and one 5 elements past its
  * end through the range check, which sends the second to the buffer's first
- * element and sets flag 4; *flags = the flags that kernel set.  Synchronous.
+ * element and sets flag 4; *flags = the flags that kernel set.  Then the
+ * map-point kernels run on descriptions that claim less than their buffers
+ * hold, and each must set the flags of what it accesses.  Synchronous.
  * Errors: INVALID_ARG (flags NULL), UNSUPPORTED (the normal build: nothing is
- * launched, *flags = 0), CUDA. */
+ * launched, *flags = 0; or a map-point kernel whose flags stayed clear), CUDA. */
 int glt_debug_checked_probe(unsigned* flags);
 
 /* The (cluster, threads) shape the tracker's solve launches with (chosen at

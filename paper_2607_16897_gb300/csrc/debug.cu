@@ -113,7 +113,12 @@ extern "C" int glt_debug_checked_probe(unsigned* flags)
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) *flags = check_flags_debug();
     cudaFree(buf);
-    return e == cudaSuccess ? GLT_OK : cuda_fail(e, "glt_debug_checked_probe");
+    bool caught = false;
+    if (e == cudaSuccess) e = probe_points(&caught);
+    if (e != cudaSuccess) return cuda_fail(e, "glt_debug_checked_probe");
+    if (caught) return GLT_OK;
+    set_error("glt_debug_checked_probe: a map-point kernel accesses memory unchecked");
+    return GLT_ERR_UNSUPPORTED;
 #else
     set_error("glt_debug_checked_probe: not a bounds-checked build (libglt_checked.so)");
     return GLT_ERR_UNSUPPORTED;

@@ -167,6 +167,8 @@ cudaError_t launch_ic_hessian(const glt_tracker* t, cudaStream_t s);
 unsigned check_flags_track();
 unsigned check_flags_pyramid();
 unsigned check_flags_points();
+// points.cu: positive control of the map-point kernels
+cudaError_t probe_points(bool* caught);
 #endif
 
 // track.cu

@@ -15,6 +15,12 @@ namespace glt {
 // positive or a sample leaves 1 <= q < W-2, 1 <= q < H-2.
 struct RefLevels {
     const uint8_t* img[kMaxLevels];
+#ifdef GLT_CHECKED
+    size_t size[kMaxLevels];     // bytes of a level
+    __device__ __forceinline__ size_t bytes(int l) const { return size[l]; }
+#else
+    __device__ __forceinline__ size_t bytes(int) const { return 0; }
+#endif
 };
 
 struct RefPoint {
@@ -43,6 +49,13 @@ __device__ __forceinline__ RefPoint ref_point(const LevelDev& lv, float u0, floa
     return r;
 }
 
+// p, from where n words of the level (img, size bytes) are read
+template <class T>
+__device__ __forceinline__ const T* level_read(const uint8_t* img, size_t size, const uint8_t* p, size_t n)
+{
+    return checked(reinterpret_cast<const T*>(p), n, reinterpret_cast<const T*>(img), size / sizeof(T), CK_IMAGE);
+}
+
 // tab + i, where n elements are written; null without a table
 template <class T>
 __device__ __forceinline__ T* table_to(const StreamDesc& D, T* tab, size_t i, size_t n)
@@ -51,9 +64,12 @@ __device__ __forceinline__ T* table_to(const StreamDesc& D, T* tab, size_t i, si
 }
 
 // The 8-pixel pattern of one point on one level.
-__device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint& r, const uint8_t* img, int P, int l, int p,
+__device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint& r, const uint8_t* img, size_t size, int P, int l, int p,
                                              float* I0, float2* G0)
 {
+    // the samples' and gradients' taps: 8 x 8 bytes from (xb - 3, yb - 3)
+    const uint8_t* win = nullptr;
+    if (r.ok) win = level_read<uint8_t>(img, size, img + (size_t)(r.yb - 3) * P + (r.xb - 3), (size_t)7 * P + 8);
     I0 = table_to(D, I0, ((size_t)l * D.Npad + p) * 8, 8);
     G0 = table_to(D, G0, ((size_t)l * D.Npad + p) * 8, 8);
 #pragma unroll
@@ -63,7 +79,7 @@ __device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint
             if (G0) G0[k] = make_float2(0.0f, 0.0f);
             continue;
         }
-        const uint8_t* t = img + (size_t)(r.yb + pat_dy(k)) * P + (r.xb + pat_dx(k));
+        const uint8_t* t = win + (3 + pat_dy(k)) * P + (3 + pat_dx(k));
         const float I00 = t[0], I10 = t[1], I01 = t[P], I11 = t[P + 1];
         I0[k] = fmaf(r.w00, I00, fmaf(r.w10, I10, fmaf(r.w01, I01, r.w11 * I11)));
         if (G0) {
@@ -84,7 +100,7 @@ __device__ __forceinline__ void set_pattern8(const StreamDesc& D, const RefPoint
 // and to the right, is read once with aligned 8-byte loads (those that hold a
 // byte of it) and every sample and gradient is interpolated from registers.
 template <int PS, int TG>
-__device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r, const uint8_t* img, int P, int l, int p,
+__device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r, const uint8_t* img, size_t size, int P, int l, int p,
                                           int g, float* I0, float2* G0)
 {
     constexpr int h = (PS - 1) / 2, RG = group_rows(PS, TG), R = RG + 3, NB = PS + 3, NW = (NB + 3) / 4;
@@ -107,7 +123,7 @@ __device__ __forceinline__ void set_patch(const StreamDesc& D, const RefPoint& r
 #pragma unroll
     for (int q = 0; q < R; ++q) {
         if (q < rows + 3) {
-            const uint2* rp = reinterpret_cast<const uint2*>(img + (size_t)(ys + q) * P + a8);
+            const uint2* rp = level_read<uint2>(img, size, img + (size_t)(ys + q) * P + a8, wide ? 3 : sh + NB > 8 ? 2 : 1);
             const uint2 u0 = rp[0], u1 = (sh + NB > 8) ? rp[1] : make_uint2(0u, 0u), u2 = wide ? rp[2] : make_uint2(0u, 0u);
             const uint32_t v[7] = {u0.x, u0.y, u1.x, u1.y, u2.x, u2.y, 0u};
 #pragma unroll
@@ -162,15 +178,16 @@ set_points_kernel(StreamDesc* __restrict__ desc, int n, RefLevels ref, const flo
     const LevelDev& lv = D.lv[l];
     const RefPoint r = ref_point(lv, u0, v0, d, l, D.pattern ? (D.pattern - 1) / 2 : 2);
     const uint8_t* img = ref.img[l];
+    const size_t size = ref.bytes(l);
     switch (D.pattern * 8 + tg) {
-    case 1: set_pattern8(D, r, img, lv.pitch, l, p, I0, G0); break;
-    case 3 * 8 + 1: set_patch<3, 1>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 5 * 8 + 1: set_patch<5, 1>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 7 * 8 + 1: set_patch<7, 1>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 9 * 8 + 1: set_patch<9, 1>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 11 * 8 + 1: set_patch<11, 1>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 7 * 8 + kHcGroups: set_patch<7, kHcGroups>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
-    case 11 * 8 + kHcGroups: set_patch<11, kHcGroups>(D, r, img, lv.pitch, l, p, g, I0, G0); break;
+    case 1: set_pattern8(D, r, img, size, lv.pitch, l, p, I0, G0); break;
+    case 3 * 8 + 1: set_patch<3, 1>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 5 * 8 + 1: set_patch<5, 1>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 7 * 8 + 1: set_patch<7, 1>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 9 * 8 + 1: set_patch<9, 1>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 11 * 8 + 1: set_patch<11, 1>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 7 * 8 + kHcGroups: set_patch<7, kHcGroups>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
+    case 11 * 8 + kHcGroups: set_patch<11, kHcGroups>(D, r, img, size, lv.pitch, l, p, g, I0, G0); break;
     }
 }
 
@@ -206,11 +223,12 @@ hess_points_kernel(const StreamDesc* __restrict__ desc, float* __restrict__ part
     float h[kHessSums];
 #pragma unroll
     for (int i = 0; i < kHessSums; ++i) h[i] = 0.0f;
-    float* out = part + (size_t)l * kHessSums * D.Npad + p;
+    float* out = checked(part + (size_t)l * kHessSums * D.Npad + p, (size_t)(kHessSums - 1) * D.Npad + 1, part,
+                         (size_t)D.L * kHessSums * D.Npad, CK_TABLE);
     // a point that is not usable on this level of the reference adds zeros
-    const bool usable = !isnan(D.I0[base]);
-    const float4 q = D.pt[p];
-    const float2 dz = D.dz[p];
+    const bool usable = !isnan(*table_from(D, D.I0, base, 1));
+    const float4 q = *checked(D.pt + p, 1, D.pt, (size_t)D.Npad, CK_POINTS);
+    const float2 dz = *checked(D.dz + p, 1, D.dz, (size_t)D.Npad, CK_POINTS);
     const float fxl = D.fx * s * dz.y, fyl = D.fy * s * dz.y;
     const float a0[3] = {fxl, 0.0f, -fxl * q.z};
     const float a1[3] = {0.0f, fyl, -fyl * q.w};
@@ -219,7 +237,7 @@ hess_points_kernel(const StreamDesc* __restrict__ desc, float* __restrict__ part
     const int groups = !usable ? 0 : ps ? tg : 1;
     for (int g = 0; g < groups; ++g) {
         const int m = ps ? min(RG, ps - g * RG) * ps : 8;
-        const float2* G = D.G0 + base + g;
+        const float2* G = table_from(D, D.G0, base + g, (size_t)(m - 1) * stride + 1);
 #pragma unroll 4
         for (int k = 0; k < m; ++k) {
             const float2 g0 = G[k * stride];
@@ -253,7 +271,7 @@ hess_finish_kernel(const StreamDesc* __restrict__ desc, const float* __restrict_
     __shared__ int last;
     const StreamDesc& D = *desc;
     const int e = blockIdx.x, l = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-    const float* in = part + ((size_t)l * kHessSums + e) * D.Npad;
+    const float* in = checked(part + ((size_t)l * kHessSums + e) * D.Npad, (size_t)D.N, part, (size_t)D.L * kHessSums * D.Npad, CK_TABLE);
     double acc = 0.0;
 #pragma unroll 4
     for (int p = tid; p < D.N; p += kHessChains) acc += (double)in[p];
@@ -340,7 +358,12 @@ cudaError_t launch_set_points(const glt_tracker* t, const float* uvd_dev, int n,
     const long long tasks = (long long)n * t->desc_host.tg;
     const long long blocks = tasks > 0 ? (tasks + threads - 1) / threads : 1;
     RefLevels ref{};
-    for (int l = 0; l < t->L; ++l) ref.img[l] = t->pyr[GLT_REF].base + t->pyr[GLT_REF].off[l];
+    for (int l = 0; l < t->L; ++l) {
+        ref.img[l] = t->pyr[GLT_REF].base + t->pyr[GLT_REF].off[l];
+#ifdef GLT_CHECKED
+        ref.size[l] = (size_t)t->pitch[l] * t->H[l];
+#endif
+    }
     set_points_kernel<<<dim3((unsigned)blocks, (unsigned)t->L), threads, 0, s>>>(
         t->desc_dev, n, ref, uvd_dev, (float)t->cfg.cx, (float)t->cfg.cy, t->pt, t->dz, t->I0, t->G0);
     return cudaGetLastError();
@@ -354,7 +377,76 @@ unsigned check_flags_points()
     cudaMemcpyToSymbol(g_check_flags, &z, sizeof(z));
     return v;
 }
+
+// Positive control of the map-point kernels: descriptions that claim less than
+// the buffers hold (a level of 8 rows instead of 48, arrays of 32 points instead
+// of 64), so that the checks send accesses back that would have been in range.
+// *caught: every kernel set the flags of what it accesses.
+cudaError_t probe_points(bool* caught)
+{
+    constexpr int W = 64, H = 48, P = 80, N = 64, CLAIM = 32;
+    constexpr size_t TAB = (size_t)128 * N * kHcGroups;      // any pattern's table
+    struct Buffers {
+        StreamDesc desc;
+        alignas(16) uint8_t img[P * H];
+        float uvd[3 * N];
+        alignas(16) float4 pt[N];
+        float2 dz[N];
+        alignas(16) float I0[TAB];
+        alignas(16) float2 G0[TAB];
+        float part[kHessSums * N];
+        double Hc[72];
+        unsigned count;
+    };
+    Buffers* B = nullptr;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&B), sizeof(Buffers));
+    if (e != cudaSuccess) return e;
+    auto flags = [&](unsigned want) {
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return false;
+        return (check_flags_points() & want) == want;
+    };
+    *caught = true;
+    for (const int pattern : {0, 5, 7}) {
+        StreamDesc D{};
+        D.L = 1;
+        D.N = N;
+        D.Npad = CLAIM;
+        D.fx = D.fy = 50.0f;
+        D.pattern = pattern;
+        D.K = pattern ? pattern * pattern : 8;
+        D.tg = hc_groups(pattern);
+        D.lv[0].W = W;
+        D.lv[0].H = H;
+        D.lv[0].pitch = P;
+        D.pt = B->pt;
+        D.dz = B->dz;
+        D.I0 = B->I0;
+        D.G0 = B->G0;
+        float uvd[3 * N];
+        for (int i = 0; i < N; ++i) {
+            uvd[3 * i] = 16.0f + i % 32;
+            uvd[3 * i + 1] = 20.0f + i % 8;
+            uvd[3 * i + 2] = 2.0f;
+        }
+        if (e == cudaSuccess) e = cudaMemset(B, 0, sizeof(Buffers));
+        if (e == cudaSuccess) e = cudaMemcpy(&B->desc, &D, sizeof(D), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(B->uvd, uvd, sizeof(uvd), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) break;
+        RefLevels ref{};
+        ref.img[0] = B->img;
+        ref.size[0] = (size_t)P * 8;
+        set_points_kernel<<<(N * D.tg + 127) / 128, 128>>>(&B->desc, N, ref, B->uvd, 32.0f, 24.0f, B->pt, B->dz, B->I0, B->G0);
+        *caught = flags((1u << CK_IMAGE) | (1u << CK_SET_POINTS)) && *caught;
+        hess_points_kernel<<<1, kHessThreads>>>(&B->desc, B->part);
+        *caught = flags((1u << CK_TABLE) | (1u << CK_POINTS)) && *caught;
+        hess_finish_kernel<<<kHessSums, kHessChains>>>(&B->desc, B->part, &B->count, B->Hc);
+        *caught = flags(1u << CK_TABLE) && *caught;
+    }
+    cudaFree(B);
+    return e;
+}
 #endif
 
 }  // namespace glt
-
