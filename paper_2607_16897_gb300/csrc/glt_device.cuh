@@ -935,10 +935,10 @@ __device__ __forceinline__ void sum_partials(const float* partials, unsigned blo
 // it: measured on the part, an FP64 instruction occupies its sub-partition's
 // pipe for 64 cycles whether 1 or 32 lanes take part; the next FP64
 // instruction has its result after the same 64, any other after ~110, an
-// FP64 compare costs ~105; a shuffle costs ~24 and an FP32 FMA 4.  So the tail is written for the fewest FP64
-// instructions on the dependent chain: independent quantities share one
-// instruction on different lanes, comparisons go through the bit pattern, and
-// what a decision does not need is not computed.  The state, the normal
+// FP64 compare costs ~105; a shuffle costs ~24 and an FP32 FMA 4.  So the tail
+// is written for the fewest FP64 instructions on the dependent chain:
+// independent quantities share one instruction on different lanes, comparisons
+// go through the bit pattern, and what a decision does not need is not computed.  The state, the normal
 // equations, the accept/reject decision and the composition are FP64 in both
 // solve modes; GLT_SOLVE_FP64 (the default) also factorises and exponentiates
 // in FP64, GLT_SOLVE_FP32 does those two in FP32 (their inputs carry FP32
@@ -948,7 +948,8 @@ __device__ __forceinline__ void sum_partials(const float* partials, unsigned blo
 //    GLT_SOLVE_FP32 first in FP32, and a pivot below 1e-4 of its damped
 //    diagonal sends the system to the FP64 elimination, which alone decides
 //    "not positive definite";
-//  * FP64 pivot reciprocals are an FP32 seed and an FP32 correction of it;
+//  * FP64 pivot reciprocals are an FP32 seed and one Newton step in 64-bit
+//    integers (rcp_mid);
 //  * the SE(3) exponential uses the power series of its coefficients in
 //    theta^2 below theta = 0.1 (sincos only beyond), each lane one element
 //    of exp(delta) (GLT_SOLVE_FP32: of exp(delta) - I in FP32, composed with
@@ -1099,10 +1100,6 @@ __device__ __forceinline__ void make_pass_params_warp(const double* T, double a,
     }
 }
 
-// LM state machine, replicated in every CTA of a stream's cluster (each CTA
-// runs it on bit-identical inputs, so all take the same decisions).
-enum { PH_START = 0, PH_CAND = 1 };
-
 // Constants behind the two states and behind the step, so that a lane fetches
 // every operand by index (no selects, no divergence).
 constexpr int kSt0 = 14, kSt1 = 15, kStM1 = 16, kStDown = 17, kStUp = 18, kStSize = 20;
@@ -1117,6 +1114,8 @@ constexpr int kFlStop = 16;    // ... below the level's stop threshold
 constexpr int kFlMoved = 32;   // the pose changed since the initial state
 constexpr int kFlLevel = 8;    // the level, from this bit on
 
+// LM state machine, replicated in every CTA of a stream's cluster (each CTA
+// runs it on bit-identical inputs, so all take the same decisions).
 struct Solver {
     // two states [T (12), a, b, then the constants 0, 1, -1 and the damping
     // factors]: the accepted one and the candidate under evaluation
@@ -1260,8 +1259,9 @@ __device__ inline void tail_map_init(Solver& S, int lane)
     for (int i = lane; i < 2 * kAccPad; i += 32) (&S.tot[0][0])[i] = 0.0;
 }
 
-// -x where `on`, through the sign bit (a conditional negation of an FP64 operand
-// otherwise becomes two FP64 instructions and a select)
+// -x where `on`, through the sign bit, so that neither an FP64 instruction nor a
+// select joins the chain (with the selects of the exponential gone too and a
+// shorter pivot test: 7.2k -> 6.9k cycles a tail)
 __device__ __forceinline__ double flip_sign(double x, bool on)
 {
     return __hiloint2double(__double2hiint(x) ^ (on ? (int)0x80000000 : 0), __double2loint(x));

@@ -314,12 +314,6 @@ hess_finish_kernel(const StreamDesc* __restrict__ desc, const float* __restrict_
         if (lane < 6 && lane > j) Ls[lane][j] = L[j];
         if (lane == j) ds[j] = dj;
         __syncwarp();
-        // the next column's row of L, complete up to column j
-        if (j < 5 && lane == j + 1) {
-#pragma unroll
-            for (int k = 0; k <= j; ++k) Ls[j + 1][k] = L[k];
-        }
-        __syncwarp();
     }
     // column `lane` of H^-1: L y = e, z = D^-1 y, L^T x = z
     double x[6];
