@@ -537,7 +537,10 @@ int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, const uint8_t* 
  * [64,32,3,3], conv3.b [64], fc1.w [128,1286], fc1.b [128], fc2.w [8,128],
  * fc2.b [8], each row-major.  The kernels use BF16 copies of the weights
  * (rounded to nearest even from the FP32 master copy), FP32 activations and
- * FP32 accumulation in a fixed order (results are deterministic).
+ * FP32 accumulation.  The order of the sums is fixed for a batch size, so that
+ * repeated calls give the same bits; it differs between ranges of batch sizes,
+ * between this network on its own and the batch's proposal stage, and, for
+ * gradients, with the device's number of multiprocessors.
  * Inputs x are [B][1200] (row-major 30 x 40 images), motions m [B][6],
  * outputs and targets [B][8], all FP32 DEVICE arrays.
  * A network object is not thread-safe; work on it is ordered on the stream

@@ -112,7 +112,8 @@ __device__ __forceinline__ f32x2 bfx2(unsigned v)
 // lanes of a warp share their weights), conv3 in two halves of its input
 // channels, conv1 8 channels of one pixel.  S = 4 fills the
 // shared memory and has the larger tiles; S = 2 has twice the blocks, and is
-// taken while those still fit one round (kFwdSmall).  Training also
+// taken while those still fit one round (kFwdSmall; 256 samples 31 us, 39 with S =
+// 4; 305 samples 50, 43 with S = 4).  Training also
 // stores the activations (a1, a2) that the backward pass reads.  5000 samples:
 // 2.03 ms by one thread per output on global memory, 0.27 ms here; 256: 139 ->
 // 24 us (caches flushed).
@@ -712,7 +713,7 @@ fc_weight_grad(const float* __restrict__ dh, const float* __restrict__ dy, const
 //    banks.  The blocks' sums go to `part`; adam_update adds them in order.
 // Both bound by FP32 issue and the shared-memory pipe.
 // ---------------------------------------------------------------------------
-constexpr int kBwThreads = 512, kBwBlocks = 148;
+constexpr int kBwThreads = 512;
 constexpr int kP1 = 375, kP2 = 121;                       // plane strides of a1 (17 x 22) and a2 (10 x 12)
 constexpr int kD3P = 68, kD2P = 36;                       // position strides of d3 and d2 (banks staggered)
 constexpr int kPart = kW3 + 64 + kW2 + 32 + 144 + 16;     // one block's sums: conv3, conv2, conv1 (w, b each)
@@ -1120,7 +1121,9 @@ using namespace glt::nn;
 namespace {
 
 constexpr size_t kGwSmem = (size_t)2 * kGwK * (kHid + kGwI) * sizeof(float);
-// fc_forward_split up to this many samples, fc_forward_tile beyond
+// fc_forward_split up to this many samples, fc_forward_tile beyond.  Split against
+// tile: 512 samples forward 48 / 74 us, 1536 115 / 119, 2048 148 / 142, 4096 264 /
+// 214; a training step of 1536 495 / 514 us, 2048 651 / 658, 2560 807 / 803.
 constexpr int kFcSmall = 2048;
 
 int nn_alloc(glt_nn* n)
@@ -1149,7 +1152,7 @@ int nn_alloc(glt_nn* n)
     if (e == cudaSuccess) e = al(&n->d3, (size_t)B * kFlat);
     if (e == cudaSuccess) e = al(&n->d2, (size_t)B * 32 * 8 * 10);
     if (e == cudaSuccess) e = al(&n->d1, (size_t)B * 16 * 15 * 20);
-    if (e == cudaSuccess) e = al(&n->part, (size_t)std::min(B, kBwBlocks) * kPart);
+    if (e == cudaSuccess) e = al(&n->part, (size_t)std::min(B, n->sms) * kPart);
     if (e == cudaSuccess) e = al(&n->loss_b, (size_t)B);
     if (e == cudaSuccess) e = al(&n->loss, 1);
     if (e == cudaSuccess) e = cudaMemset(n->m, 0, kParams * sizeof(float));
@@ -1184,6 +1187,12 @@ void nn_free(glt_nn* n)
 }
 
 int grid_for(int n, int t) { return (n + t - 1) / t; }
+
+// Blocks of the convolutions' backward kernels, and so of the sums in `part`: one
+// per multiprocessor, each of whole samples.  148 on this part's 152 left four
+// idle and cost a round where B just passes a multiple: 149 samples 113 instead of
+// 93 us a training step, 304 148 instead of 128, 256 the same.
+int bw_blocks(const glt_nn* n, int B) { return std::min(B, n->sms); }
 
 // conv1-conv3 of B samples; TRAIN: the activations are kept
 template <bool TRAIN>
@@ -1243,8 +1252,8 @@ cudaError_t nn_backward(const glt_nn* n, const float* x, const float* mo, const 
     if (e != cudaSuccess) return e;
     fc1_input_grad<<<dim3(grid_for(B, kFcS), kFlat / kD3Threads), kD3Threads, kD3Smem, s>>>(n->dh, n->wt, n->a3, B, n->d3);
     fc_weight_grad<<<kGwBlocks, kGwThreads, kGwSmem, s>>>(n->dh, n->dy, n->a3, mo, n->h, B, n->g);
-    conv_input_grad<<<std::min(B, kBwBlocks), kBwThreads, sizeof(IgSmem), s>>>(n->d3, n->a1, n->a2, n->wt, B, n->d2, n->d1);
-    conv_weight_grad<<<std::min(B, kBwBlocks), kBwThreads, sizeof(WgSmem), s>>>(x, n->a1, n->a2, n->d3, n->d2, n->d1, B, n->part);
+    conv_input_grad<<<bw_blocks(n, B), kBwThreads, sizeof(IgSmem), s>>>(n->d3, n->a1, n->a2, n->wt, B, n->d2, n->d1);
+    conv_weight_grad<<<bw_blocks(n, B), kBwThreads, sizeof(WgSmem), s>>>(x, n->a1, n->a2, n->d3, n->d2, n->d1, B, n->part);
     return cudaGetLastError();
 }
 
@@ -1283,8 +1292,9 @@ namespace nn {
 // input channel x tap) with register tiles of PT pixels x 4 channels, on the
 // layer's weights in the [K][O] layout (a tile's 4 weights are one 8-byte
 // load), copied into shared memory with asynchronous 16-byte copies issued at
-// the start and awaited just before conv2.  The sum order per output (bias,
-// then channel, row, column) is that of conv_forward.
+// the start and awaited just before conv2.  The sum order per output is bias,
+// then channel, row, column; conv_forward adds conv3 in two halves of its input
+// channels and fc1 in other parts, so the two round differently.
 constexpr int kPropThreads = 512;
 constexpr int kXp = 32 * 42, kA1p = 16 * 17 * 22, kA2p = 32 * 10 * 12;
 constexpr int kPropSmemFloats = kXp + kA1p + kA2p + (kF + 2) + kHid + kOut;
@@ -1796,7 +1806,7 @@ int glt_nn_gradient(glt_nn* n, const float* x_dev, const float* m_dev, const flo
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e = nn_backward(n, x_dev, m_dev, t_dev, B, s);
     if (e == cudaSuccess) {
-        adam_update<false><<<kAdBlocks, 256, 0, s>>>(n->w, n->wbf, n->wt, n->g, n->part, std::min(B, kBwBlocks), n->m, n->v,
+        adam_update<false><<<kAdBlocks, 256, 0, s>>>(n->w, n->wbf, n->wt, n->g, n->part, bw_blocks(n, B), n->m, n->v,
                                                      0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, n->loss_b, B, n->loss);
         e = cudaGetLastError();
     }
@@ -1821,7 +1831,7 @@ int glt_nn_train_step(glt_nn* n, const float* x_dev, const float* m_dev, const f
     const double b1 = 0.9, b2 = 0.999;
     const float c1 = (float)(1.0 / (1.0 - std::pow(b1, n->step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(b2, n->step)));
-    adam_update<true><<<kAdBlocks, 256, 0, s>>>(n->w, n->wbf, n->wt, n->g, n->part, std::min(B, kBwBlocks), n->m, n->v, lr,
+    adam_update<true><<<kAdBlocks, 256, 0, s>>>(n->w, n->wbf, n->wt, n->g, n->part, bw_blocks(n, B), n->m, n->v, lr,
                                                 (float)b1, (float)b2, 1e-8f, c1, c2, n->loss_b, B, loss);
     e = cudaGetLastError();
     if (e == cudaSuccess && loss_dev && loss != loss_dev)

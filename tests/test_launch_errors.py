@@ -3,7 +3,8 @@ stand-in for the CUDA runtime (preloaded in a child process) keeps "device"
 memory on the host, runs no kernel and refuses the launch it is told to.
 Every call must report the refused launch, whichever it is, and leave no error
 behind for the next call; an output at an address that no kernel can store a
-float to is written by a copy."""
+float to is written by a copy; the grids follow the device's number of
+multiprocessors."""
 import os
 import subprocess
 import sys
@@ -25,7 +26,15 @@ int fake_copied(void) { return copied; }
 void fake_refuse(int k) { refuse = k; seen = 0; }
 int fake_launches(void) { return seen; }
 /* the error of the launch, which the runtime keeps until it is asked for */
-static err launch(void) { if (seen++ == refuse) { last = 719; return 719; } return 0; }
+static int sms = 152, grids[64];
+void fake_sms(int n) { sms = n; }
+int fake_grid(int k) { return grids[k]; }
+static err launch(unsigned grid)
+{
+    if (seen < 64) grids[seen] = (int)grid;
+    if (seen++ == refuse) { last = 719; return 719; }
+    return 0;
+}
 err cudaMalloc(void **p, size_t n) { *p = calloc(n, 1); return 0; }
 err cudaFree(void *p) { free(p); return 0; }
 err cudaMemset(void *p, int v, size_t n) { memset(p, v, n); return 0; }
@@ -33,7 +42,7 @@ err cudaMemcpy(void *d, const void *s, size_t n, int k) { (void)k; memcpy(d, s, 
 err cudaMemcpyAsync(void *d, const void *s, size_t n, int k, void *st)
 { (void)k; (void)st; if (d == odd) copied = 1; memcpy(d, s, n); return 0; }
 err cudaGetDevice(int *d) { *d = 0; return 0; }
-err cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
+err cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = sms; return 0; }
 err cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
 err cudaDeviceSynchronize(void) { return 0; }
 err cudaStreamSynchronize(void *s) { (void)s; return 0; }
@@ -41,10 +50,10 @@ err cudaGetLastError(void) { err e = last; last = 0; return e; }
 const char *cudaGetErrorString(err e) { return e ? "launch failure" : "no error"; }
 err __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return 0; }
 err __cudaLaunchKernel(void *k, dim3_ g, dim3_ b, void **a, size_t m, void *s)
-{ (void)k; (void)g; (void)b; (void)a; (void)m; (void)s; return launch(); }
+{ (void)k; (void)b; (void)a; (void)m; (void)s; return launch(g.x); }
 err cudaLaunchKernel(const void *f, dim3_ g, dim3_ b, void **a, size_t m, void *s)
-{ (void)f; (void)g; (void)b; (void)a; (void)m; (void)s; return launch(); }
-err cudaLaunchKernelExC(const void *c, const void *f, void **a) { (void)c; (void)f; (void)a; return launch(); }
+{ (void)f; (void)b; (void)a; (void)m; (void)s; return launch(g.x); }
+err cudaLaunchKernelExC(const void *c, const void *f, void **a) { (void)f; (void)a; return launch(*(const unsigned *)c); }   /* gridDim comes first */
 """
 
 CHILD = r"""
@@ -59,6 +68,8 @@ import paper_2607_16897_gb300 as glt
 fake = ctypes.CDLL(sys.argv[1])
 fake.fake_watch.argtypes = [ctypes.c_void_p]
 B, mode = int(sys.argv[2]), sys.argv[3]
+if mode == "grids":
+    fake.fake_sms(37)
 net = glt.NN(B, np.zeros(glt.GLT_NN_PARAMS, np.float32))
 x, m, t, y = (np.zeros((B, k), np.float32) for k in (1200, 6, 8, 8))
 p = [a.ctypes.data for a in (x, m, t, y)]
@@ -93,6 +104,12 @@ for off in (0, 1, 2, 3) if mode == "addresses" else ():
         call()
         if off and not fake.fake_copied():
             print("a kernel stores the output of", name, "at offset", off)
+if mode == "grids":
+    fake.fake_refuse(-1)
+    calls["train_step"]()
+    g = [fake.fake_grid(k) for k in range(fake.fake_launches())]
+    if g.count(min(B, 37)) != 3:          # forward, input gradient, weight gradient of the convolutions
+        print("grids of a training step of", B, "samples on 37 multiprocessors:", g)
 print("done")
 """
 
@@ -121,3 +138,8 @@ def test_refused_launches_are_reported(tmp_path, B):
 @pytest.mark.parametrize("B", [5, 2100])
 def test_outputs_at_any_address(tmp_path, B):
     run_child(tmp_path, B, "addresses")
+
+
+@pytest.mark.parametrize("B", [150, 2100])
+def test_convolutions_take_a_block_per_multiprocessor(tmp_path, B):
+    run_child(tmp_path, B, "grids")
