@@ -45,7 +45,7 @@ def flops_per_sample(wl):
 # (dram__bytes_read.sum + dram__bytes_write.sum, caches flushed before the
 # launch as in the timed steps) on the workload named by the key; a value is
 # removed whenever the kernel changes after it was taken.
-TRACK_TRAFFIC = {}
+TRACK_TRAFFIC = {"c2": 808448, "c2p": 7692032}
 # the trained proposal network's parameters (data file; read here as plain
 # numbers so that the oracle legs need nothing but oracle/ and synth/)
 WEIGHTS_PATH = os.path.join(ROOT, "paper_2607_16897_gb300", "proposal_weights.npy")
