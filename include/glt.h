@@ -196,6 +196,11 @@ void glt_default_config(glt_config* cfg, int width, int height, double fx, doubl
 
 /* Creates a tracker on the current CUDA device and allocates all its device
  * memory (both pyramids, map-point arrays for max_points, solver state).
+ * The reference tables take 4 bytes (8 more with GLT_IC) per point, level and
+ * sample, 8 samples of the pattern or p * p; with GLT_HESSIAN_CACHED the 7 x 7
+ * and 11 x 11 patches are padded to 56 and 132 samples (four row groups of one
+ * size), and 84 bytes per point and level hold the sums that a new reference's
+ * Hessian is made of.
  * Errors: INVALID_ARG for a bad config, CUDA on allocation failure. */
 int glt_create(const glt_config* cfg, glt_tracker** out);
 
@@ -552,8 +557,11 @@ int glt_linearize_noalloc(const uint8_t* ref_dev, int ref_pitch, const uint8_t* 
 #define GLT_NN_OUTPUT 8
 
 /* Allocates a network for batches of up to max_batch (1..65536) samples:
- * FP32 master weights, BF16 copy, Adam moments, activations.  Weights are
- * uninitialised until glt_nn_set_params.  Errors: INVALID_ARG, CUDA. */
+ * FP32 master weights, BF16 copies, Adam moments, the activations and gradients
+ * of max_batch samples (about 70 KB a sample) and, for the gradients' sums, 93 KB
+ * per multiprocessor or sample, whichever are fewer (14 MB on 152); all of it
+ * also for a network that only infers.  Weights are uninitialised until
+ * glt_nn_set_params.  Errors: INVALID_ARG, CUDA. */
 int glt_nn_create(int max_batch, glt_nn** out);
 void glt_nn_destroy(glt_nn* nn);
 
@@ -600,14 +608,14 @@ int glt_nn_load(glt_nn* nn, const char* path);
 /* Attaches `nn` (or detaches it, nn = NULL) as the proposal stage of the
  * batch: from then on glt_batch_track and glt_batch_capture first build each
  * stream's residual image from its REF and CUR coarsest levels, compute each
- * stream's motion input log(M) / 0.02 in FP64 from motion_dev[S][12] (a DEVICE
- * array of doubles read at run time: the last inter-frame motion M of every
- * stream, row-major 3x4, as glt_state.motion holds it; the identity for a
- * stream without two tracked frames), run the network on all S streams and
- * start every stream's LM from the proposed state instead of init_dev.  Every tracker of the batch needs a 40 x 30 coarsest
- * level (640 x 480 with 5 levels, 320 x 240 with 4).  The batch references
- * the network, which must outlive it and must not be trained while the batch
- * uses it.  Invalidates a captured graph.  The autotuner ignores the stage.
+ * stream's motion input log(M) / 0.02 (FP32, from FP64 differences of M's entries)
+ * from motion_dev[S][12] (a DEVICE array of doubles read at run time: the last
+ * inter-frame motion M of every stream, row-major 3x4, as glt_state.motion holds
+ * it; the identity for a stream without two tracked frames), run the network on
+ * all S streams and start every stream's LM from the proposed state instead of
+ * init_dev.  Every tracker of the batch needs a 40 x 30 coarsest level (640 x
+ * 480 with 5 levels, 320 x 240 with 4).  The batch references the network, which
+ * must outlive it and must not be trained while the batch uses it.  Invalidates a captured graph.  The autotuner ignores the stage.
  * Errors: INVALID_ARG (size, max_batch < S), CUDA. */
 int glt_batch_set_proposal(glt_batch* batch, glt_nn* nn, const double* motion_dev);
 

@@ -698,7 +698,8 @@ fc_weight_grad(const float* __restrict__ dh, const float* __restrict__ dy, const
 
 // ---------------------------------------------------------------------------
 // Backward pass of the convolutions, in two kernels (together they would hold
-// 80 gradient sums a thread beside the input gradients' registers and spill):
+// 80 gradient sums a thread beside the input gradients' registers and spilled as
+// many; conv_weight_grad alone spills 84 bytes):
 //  * conv_input_grad: d2 from d3 and d1 from d2, a sample per block at a time.
 //    A thread owns a 2 x 2 quad of input pixels x 4 channels, whose nine
 //    (pixel, tap) pairs use each weight once (36 FMAs per 9 + 4 shared loads);

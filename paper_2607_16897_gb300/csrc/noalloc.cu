@@ -101,7 +101,9 @@ struct NaWindow {
 // every lane's word is an L1 miss of its own; 9k one window after the other in
 // 4-byte words), the samples (2.3k), the block's reduction, and the last block's
 // sum over the blocks.  20000 points: 24.7 us with byte loads and a serial sum,
-// now 14.4 (the call's two launches take the host as long).
+// now 14.4 (the call's two launches take the host as long), on buffers that were
+// read before; ten calls from idle on buffers that none has met 28.1 us each then,
+// 18.8 now (27.4 and 18.2 on known ones).
 __global__ void __launch_bounds__(kNaThreads)
     linearize_noalloc_kernel(NaArgs A, PassParams P, float* __restrict__ scratch,
                              double* __restrict__ out)

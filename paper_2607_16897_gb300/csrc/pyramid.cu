@@ -83,10 +83,10 @@ __device__ __forceinline__ uint32_t src_byte(const PyrJob& J, const uint8_t* row
 // Bound in a batch by the loads in flight (256 frames of 640 x 480, 4 levels:
 // 62 us, 43% of the copy bandwidth), for one frame by the launch and one memory
 // round trip.  8 x 4 outputs: 16-byte loads, three rows in eleven read twice
-// (from L2), 44 words a thread in flight, ~16 instructions an output.  Staging
-// 64 x 16 tiles in shared memory with 4-byte loads was bound by issue (~150
-// instructions an output): 136 us for the batch, 47 instead of 23 us for 64
-// frames of mixed sizes.
+// (from L2), 44 words a thread in flight, ~16 instructions an output; five blocks
+// an SM cost 48 bytes of spills.  Staging 64 x 16 tiles in shared memory with
+// 4-byte loads was bound by issue (~150 instructions an output): 136 us for the
+// batch, 47 instead of 23 us for 64 frames of mixed sizes.
 __global__ void __launch_bounds__(PYR_THREADS, 5) pyr_down_kernel(const PyrJob* __restrict__ jobs,
                                                                   const unsigned* __restrict__ tile_map,
                                                                   const uint8_t* const* frames,
