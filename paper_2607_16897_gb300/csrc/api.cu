@@ -243,7 +243,13 @@ static void resolve_shape(glt_tracker* t)
     int cluster = t->cfg.cluster;
     if (cluster == 0) {
         // about one point per thread, in units of the 8-pixel pattern's work
-        // (the cached-Hessian form: one task per thread)
+        // (the cached-Hessian form: one task per thread).  us a frame, cluster x
+        // threads, taken shape first: 500 points (320 x 240) 2 x 256 70.0, 4 x 128
+        // 68.1, 8 x 256 70.1, 1 x 256 86.4; 2000 (640 x 480) 8 x 256 78.3, 16 x 256
+        // 79.9, 16 x 128 84.3, 8 x 512 102.9, 4 x 256 99.9; 8000 (1280 x 720) 16 x 256
+        // 141.9, 16 x 512 147.8, 8 x 256 200.6; cached Hessian, 7 x 7, 500 points 4 x
+        // 512 162, 8 x 512 166, 2 x 512 228.  With less than half a point a thread the
+        // exchange takes back what the samples gain
         const long long work = variant == 4 ? (long long)t->N * hc_groups(t->cfg.pattern)
                                             : (long long)t->N * std::max(1, t->K / 8);
         cluster = (int)std::min<long long>(16, std::max<long long>(1, (work + threads - 1) / threads));
